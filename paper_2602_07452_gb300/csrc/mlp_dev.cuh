@@ -58,14 +58,20 @@ __device__ __forceinline__ int layer_mma(uint32_t tbase, const uint8_t* sA, cons
 
 // Epilogue of a hidden layer: z = acc + b; a = bf16(relu(z)) into sH.  Row
 // r = thread % 128 (its TMEM lane); the two halves of the block take
-// columns [0, 64) and [64, 128).  Optionally to global H (bf16 [B][128]).
-__device__ __forceinline__ void hidden_epilogue(uint32_t tbase, const float* b, uint8_t* sH, uint16_t* Hg,
-                                                long long row, long long B)
+// columns [0, 64) and [64, 128).  TRAIN: also this row's activations to
+// global memory (Hrow, bf16 [128]) and the bits of the positive ones of
+// this thread's 64 columns to mask[2].
+template <bool TRAIN = false>
+__device__ __forceinline__ void hidden_epilogue(uint32_t tbase, const float* b, uint8_t* sH, uint16_t* Hrow = nullptr,
+                                                uint32_t* mask = nullptr)
 {
     const int r = threadIdx.x & 127, warp = (threadIdx.x >> 5) & 3, half = threadIdx.x >> 7;
-    for (int c0 = 64 * half; c0 < 64 * half + 64; c0 += 32) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c0 = 64 * half + 32 * h;
         float v[32];
         tc::tmem_ld32(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+        uint32_t pos = 0;
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             uint32_t pk[4];
@@ -74,11 +80,16 @@ __device__ __forceinline__ void hidden_epilogue(uint32_t tbase, const float* b, 
                 const int c = c0 + g * 8 + 2 * q;
                 const float z0 = v[g * 8 + 2 * q] + b[c], z1 = v[g * 8 + 2 * q + 1] + b[c + 1];
                 pk[q] = tc::pack_bf2(z0 > 0.f ? z0 : 0.f, z1 > 0.f ? z1 : 0.f);
+                if (TRAIN) {
+                    pos |= ((pk[q] & 0xffffu) ? 1u : 0u) << (g * 8 + 2 * q);
+                    pos |= ((pk[q] >> 16) ? 1u : 0u) << (g * 8 + 2 * q + 1);
+                }
             }
             const uint4 u = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             *(uint4*)(sH + tc::kmajor_off(r, c0 + g * 8, 128)) = u;
-            if (Hg && row < B) *(uint4*)(Hg + (size_t)row * 128 + c0 + g * 8) = u;
+            if (TRAIN) *(uint4*)(Hrow + c0 + g * 8) = u;
         }
+        if (TRAIN) mask[h] = pos;
     }
 }
 
@@ -106,19 +117,21 @@ __device__ __forceinline__ uint32_t mlp_cta_setup(const MlpDev& w, uint8_t* smem
 }
 
 // The four layers of one 128-row tile whose bf16 inputs are in FW_X; the
-// output layer's accumulators stay in TMEM columns 0-15.  Hg (nullable):
-// bf16 hidden activations for training, 3 x B x 128.  Returns 0 if a
-// bounded tensor-core wait ran out.
+// output layer's accumulators stay in TMEM columns 0-15.  TRAIN: the hidden
+// activations also go to Hrow (this thread's row of layer 1; layer l's is
+// l * hstride further) and the positive ones' bits to mask[6].  Returns 0 if
+// a bounded tensor-core wait ran out.
+template <bool TRAIN = false>
 __device__ __forceinline__ int mlp_tile_layers(uint32_t tbase, uint8_t* smem, uint64_t* mbar, uint32_t& phase,
-                                               uint16_t* Hg, long long row, long long B)
+                                               uint16_t* Hrow = nullptr, size_t hstride = 0, uint32_t* mask = nullptr)
 {
     const float* sb = (const float*)(smem + FW_B);
     if (!layer_mma(tbase, smem + FW_X, smem + FW_W1, 128, 16, mbar, phase)) return 0;
-    hidden_epilogue(tbase, sb, smem + FW_H, Hg, row, B);
+    hidden_epilogue<TRAIN>(tbase, sb, smem + FW_H, Hrow, mask);
     if (!layer_mma(tbase, smem + FW_H, smem + FW_W2, 128, 128, mbar, phase)) return 0;
-    hidden_epilogue(tbase, sb + 128, smem + FW_H, Hg ? Hg + (size_t)B * 128 : nullptr, row, B);
+    hidden_epilogue<TRAIN>(tbase, sb + 128, smem + FW_H, Hrow + hstride, mask + 2);
     if (!layer_mma(tbase, smem + FW_H, smem + FW_W3, 128, 128, mbar, phase)) return 0;
-    hidden_epilogue(tbase, sb + 256, smem + FW_H, Hg ? Hg + (size_t)2 * B * 128 : nullptr, row, B);
+    hidden_epilogue<TRAIN>(tbase, sb + 256, smem + FW_H, Hrow + 2 * hstride, mask + 4);
     return layer_mma(tbase, smem + FW_H, smem + FW_W4, 16, 128, mbar, phase);
 }
 
