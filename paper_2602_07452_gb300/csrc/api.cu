@@ -290,6 +290,7 @@ extern "C" void fpic_destroy(fpic_ctx* c)
     cudaDeviceSynchronize();
     if (c->d_nodes) cudaFree(c->d_nodes);
     if (c->d_metric) cudaFree(c->d_metric);
+    if (c->d_poly) cudaFree(c->d_poly);
     if (c->d_cnt) cudaFree(c->d_cnt);
     if (c->h_cnt) cudaFreeHost(c->h_cnt);
     if (c->d_scratch) cudaFree(c->d_scratch);

@@ -1,0 +1,215 @@
+// The deposit's subvolumes on fine grids from a per-cell polynomial of
+// sqrt(gamma), in place of evaluating the trapezoid lattice point by point.
+//
+// On a sub-grid cell of centre (xm, yc) and size (dx, dy), with xi, eta in
+// [-1/2, 1/2] its local coordinates,
+//   sqrt(gamma) = K (sin th / sin yc) (1 + sum_{1 <= m+n <= 5} f_mn xi^m eta^n),
+// sqrt(gamma) / sin th = sqrt((r^2 + A)(r^2 + 2 M r + A)), A = a^2 cos^2 th.
+// The 4-point trapezoid rule over an interval of centre u and half-width w
+// is the mean over u + w {-1, -1/3, 1/3, 1} with weights {1, 2, 2, 1} / 6: its
+// moments of xi^m are polynomials M_m(u, w) (mu_2 = 11/27, mu_4 = 83/243,
+// mu_6 = 731/2187), so a subvolume is its area times
+//   sum_n R_n E_n,  R_n = sum_m f_mn M_m (r part),  E_n the moments of
+//   (sin th / sin yc) eta^n (th part; sin th by its own series about yc, so
+//   the cells at the poles are no worse than the others).
+// The same rule's values as the lattices' to the truncation at degree 5 and
+// rounding: the terms up to degree 2 and everything they multiply run in
+// paired FP32, the others (below 2^-22 of the sum where the table is used)
+// in FP32.
+#pragma once
+#include "ff.cuh"
+
+namespace fpic {
+
+constexpr int POLY_STRIDE = 28;      // floats of a cell (25 used): seven 16-byte loads
+// The polynomial is used where poly_bound, the largest error of a node share
+// over every cell of the grid, stays below POLY_TOL = 2^-45.5: the lattice
+// form's own square root is good to 2^-44.5.  Grids uniform in ln r and th from
+// 0.9 r_+ to 50 M meet it from about 200 cells a side (there the shares
+// differ from an extended-precision quadrature by at most 7e-16 in 200 random
+// cells, 2e-17 at 512); coarser ones keep the lattices.
+constexpr double POLY_TOL = 2e-14;
+constexpr double POLY_MAX_DTH = 0.03, POLY_MAX_TAU = 4.0;     // limits of the sin th series
+
+// f_mn (m + n <= 6, f[m][n]) of the cell of centre (x, y) and size (dx, dy).
+__host__ __device__ inline void poly_series(double M, double a, double x, double y, double dx, double dy,
+                                            double f[7][7])
+{
+    constexpr int D = 6;
+    // P1 = r^2 + a^2 cos^2 th = sum_n p[n] eta^n + p1 xi + p2 xi^2
+    double p[D + 1];
+    const double c = cos(y), s2y = 2.0 * sin(y) * c, c2y = 2.0 * c * c - 1.0;
+    double h = 0.5 * a * a;
+#pragma unroll
+    for (int n = 1; n <= D; ++n) {
+        h *= 2.0 * dy / n;
+        const double t = (n & 1) ? s2y : c2y;
+        p[n] = ((n & 3) == 1 || (n & 3) == 2) ? -h * t : h * t;
+    }
+    p[0] = x * x + a * a * c * c;
+    const double p1 = 2.0 * x * dx, p2 = dx * dx;
+    // g = P1 (P1 + 2 M r) / g_00, then f = sqrt(g)
+    const double q0 = 2.0 * M * x, q1 = 2.0 * M * dx;
+    const double ig = 1.0 / (p[0] * (p[0] + q0));
+#pragma unroll
+    for (int d = 0; d <= D; ++d)
+#pragma unroll
+        for (int m = 0; m <= d; ++m) {
+            const int n = d - m;
+            double g = 0.0;
+            if (m == 0) {
+                g = q0 * p[n];
+#pragma unroll
+                for (int j = 0; j <= n; ++j) g += p[j] * p[n - j];
+            } else if (m == 1) {
+                g = (2.0 * p1 + q1) * p[n] + (n == 0 ? q0 * p1 : 0.0);
+            } else if (m == 2) {
+                g = 2.0 * p2 * p[n] + (n == 0 ? p1 * p1 + q0 * p2 + q1 * p1 : 0.0);
+            } else if (n == 0 && m == 3) {
+                g = 2.0 * p1 * p2 + q1 * p2;
+            } else if (n == 0 && m == 4) {
+                g = p2 * p2;
+            }
+            if (d == 0) {
+                f[0][0] = 1.0;
+                continue;
+            }
+            double t = g * ig;
+#pragma unroll
+            for (int i = 0; i <= m; ++i)
+#pragma unroll
+                for (int j = 0; j <= n; ++j)
+                    if (i + j > 0 && i + j < d) t -= f[i][j] * f[m - i][n - j];
+            f[m][n] = 0.5 * t;
+        }
+}
+
+// Bound on the error of a node share (a fraction of the cell): the terms of
+// degree 6 that are left out and the FP32 rounding of those of degree 3 to 5,
+// an interval's share of a cell's moment of xi^m being at most 2^-m / (2 m + 1).
+__host__ __device__ inline double poly_bound(const double f[7][7])
+{
+    double e = 0.0;
+#pragma unroll
+    for (int d = 3; d <= 6; ++d)
+#pragma unroll
+        for (int m = 0; m <= d; ++m) {
+            const int n = d - m;
+            e += fabs(f[m][n]) * (d == 6 ? 1.0 : 5.9604644775390625e-8) / ((1 << d) * (2.0 * m + 1.0) * (2.0 * n + 1.0));
+        }
+    return e;
+}
+
+struct PolyTab {
+    double lo[4], hi[4];    // first and last rn, rh, tn, th
+    const float4* c[3];     // cells of the (i, j), (i+1/2, j), (i, j+1/2) sub-grids, row stride Nth
+    const float2* ir[2];    // 1 / dr of the integer and half r cells
+    const float4* t[2];     // two per integer and half th cell: 1 / dth and tau = dth cot yc (pairs);
+                            // dth^2 / 2 and dth^2 / 6 (pairs)
+};
+
+#ifdef __CUDACC__
+// One interval's moments: [0] below the particle, [1] above it.
+struct Mom {
+    ff len, m1, m2, m3;
+    float m4, m5, m6;
+};
+
+// Both intervals of a cell split at the fraction al (ab = 1 - al): lower
+// u = -ab/2, w = al/2; upper u = al/2, w = ab/2.
+__device__ __forceinline__ void moments(ff al, ff ab, Mom M[2])
+{
+    const ff mu2 = {__uint_as_float(0x3ed097b4u), __uint_as_float(0x3197b426u)};     // 11/27
+    const ff a2 = ff_sqr(al), b2 = ff_sqr(ab);
+    const ff ma = ff_mul(mu2, a2), mb = ff_mul(mu2, b2);
+    constexpr float k6 = 22.f / 9.f, k10 = 110.f / 27.f, m4 = 83.f / 243.f, k5 = 415.f / 243.f, k15 = 165.f / 27.f,
+                    k15b = 1245.f / 243.f, m6 = 731.f / 2187.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const ff U2 = h ? a2 : b2, W = h ? mb : ma;
+        M[h].len = h ? ab : al;
+        M[h].m1 = h ? ff_scale(al, 0.5f) : ff_scale(ab, -0.5f);
+        M[h].m2 = ff_scale(ff_add(U2, W), 0.25f);
+        M[h].m3 = ff_mul(M[h].m1, ff_scale(ff_add(U2, ff_mulf(W, 3.f)), 0.25f));
+        const float u = M[h].m1.hi, u2 = 0.25f * U2.hi, w2 = 0.25f * (h ? b2 : a2).hi;
+        const float uu = u2 * u2, uw = u2 * w2, ww = w2 * w2;
+        M[h].m4 = fmaf(m4, ww, fmaf(k6, uw, uu));
+        M[h].m5 = u * fmaf(k5, ww, fmaf(k10, uw, uu));
+        M[h].m6 = fmaf(u2, fmaf(k15b, ww, fmaf(k15, uw, uu)), m6 * ww * w2);
+    }
+}
+
+// th moments of (sin th / sin yc) eta^n: E_0 = 1 + e0.
+struct MomT {
+    ff len, e0, e1, e2;
+    float e3, e4, e5;
+};
+
+__device__ __forceinline__ ff ff_addf(ff a, float b)      // a + b, |b| far below |a| or folded into lo
+{
+    return {a.hi, __fadd_rn(a.lo, b)};
+}
+
+// d2_2, d2_6: dth^2 / 2 and dth^2 / 6.  The cubic term of sin th, up to 10^-6
+// of the sum in the cells at the poles, is paired too.
+__device__ __forceinline__ void moments_th(const Mom M[2], ff tau, ff d2_2, ff d2_6, MomT E[2])
+{
+    const float t = tau.hi, d = 2.f * d2_2.hi;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const Mom& m = M[h];
+        E[h].len = m.len;
+        // 1 - d^2/2 + d^4/24 and tau (1 - d^2/6 + d^4/120) in powers of eta
+        const float c0 = d * d * fmaf(t * (1.f / 120.f), m.m5, (1.f / 24.f) * m.m4);
+        const ff s1 = ff_mul(tau, ff_add(m.m1, ff_neg(ff_mul(d2_6, m.m3))));
+        E[h].e0 = ff_addf(ff_add(s1, ff_neg(ff_mul(d2_2, m.m2))), c0);
+        const float c1 = -d * fmaf(-d, fmaf((1.f / 120.f) * t, m.m6, (1.f / 24.f) * m.m5),
+                                   fmaf((1.f / 6.f) * t, m.m4, 0.5f * m.m3.hi));
+        E[h].e1 = ff_addf(ff_add(m.m1, ff_mul(tau, m.m2)), c1);
+        const float c2 = -d * fmaf((1.f / 6.f) * t, m.m5, 0.5f * m.m4);
+        E[h].e2 = ff_addf(ff_add(m.m2, ff_mul(tau, m.m3)), c2);
+        E[h].e3 = fmaf(-d, fmaf((1.f / 6.f) * t, m.m6, 0.5f * m.m5), fmaf(t, m.m4, m.m3.hi));
+        E[h].e4 = fmaf(-0.5f * d, m.m6, fmaf(t, m.m5, m.m4));
+        E[h].e5 = fmaf(t, m.m6, m.m5);
+    }
+}
+
+// The four node shares (w00, w10, w01, w11: V of the opposite corner / V) of
+// a sub-grid cell from its r and th moments.
+__device__ __forceinline__ void poly_shares(const float4* __restrict__ c, const Mom X[2], const MomT Y[2], ff w[4])
+{
+    const float4 q0 = __ldg(c), q1 = __ldg(c + 1), q2 = __ldg(c + 2), q3 = __ldg(c + 3), q4 = __ldg(c + 4),
+                 q5 = __ldg(c + 5);
+    const float f05 = __ldg((const float*)(c + 6));
+    const ff f10 = {q0.x, q0.y}, f01 = {q0.z, q0.w}, f20 = {q1.x, q1.y}, f11 = {q1.z, q1.w}, f02 = {q2.x, q2.y};
+    const float f30 = q2.z, f21 = q2.w, f12 = q3.x, f03 = q3.y, f40 = q3.z, f31 = q3.w, f22 = q4.x, f13 = q4.y,
+                f04 = q4.z, f50 = q4.w, f41 = q5.x, f32 = q5.y, f23 = q5.z, f14 = q5.w;
+    ff V[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const Mom& m = X[h];
+        const ff R0 = ff_addf(ff_add(ff_mul(f10, m.m1), ff_mul(f20, m.m2)),
+                              fmaf(f30, m.m3.hi, fmaf(f40, m.m4, f50 * m.m5)));
+        const ff R1 = ff_addf(ff_add(f01, ff_mul(f11, m.m1)), fmaf(f21, m.m2.hi, fmaf(f31, m.m3.hi, f41 * m.m4)));
+        const ff R2 = ff_addf(f02, fmaf(f12, m.m1.hi, fmaf(f22, m.m2.hi, f32 * m.m3.hi)));
+        const float R3 = fmaf(f13, m.m1.hi, fmaf(f23, m.m2.hi, f03)), R4 = fmaf(f14, m.m1.hi, f04);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const MomT& e = Y[g];
+            // sum - 1 = e0 + R0 + R0 e0 + R1 e1 + R2 e2 + ...
+            ff S = ff_add(ff_add(e.e0, R0), ff_add(ff_mul(R0, e.e0), ff_mul(R1, e.e1)));
+            S = ff_add(S, ff_addf(ff_mul(R2, e.e2), fmaf(R3, e.e3, fmaf(R4, e.e4, f05 * e.e5))));
+            const ff area = ff_mul(m.len, e.len);
+            const ff v = ff_add(area, ff_mul(area, S));
+            V[h + 2 * g] = ff_fast2(v.hi, v.lo);         // normalized: S carries FP32 terms in its lo
+        }
+    }
+    const ff iV = ff_rcp(ff_add(ff_add(V[0], V[1]), ff_add(V[2], V[3])));
+    w[0] = ff_mul(V[3], iV);
+    w[1] = ff_mul(V[2], iV);
+    w[2] = ff_mul(V[1], iV);
+    w[3] = ff_mul(V[0], iV);
+}
+#endif
+
+}  // namespace fpic

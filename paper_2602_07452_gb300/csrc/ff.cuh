@@ -40,29 +40,24 @@ __device__ __forceinline__ ff ff_of(float a)
 }
 
 // The double x as hi + lo, by integer operations on its bits (the FP64
-// pipe's conversions would cost as much as FP64 arithmetic): hi takes the
-// sign, exponent and leading 23 fraction bits, lo the remaining 29 bits
-// rounded to a float (one fused multiply-add of two exact parts): within
-// 2^-47 relative for 2^-70 <= |x| < 2^127; 0 below 2^-126 (and lo 0 below
-// 2^-70), which only drops magnitudes under 2^-70 of the lattice values.
+// pipe's conversions would cost as much as FP64 arithmetic): hi is x rounded
+// to a float -- sign, exponent (the biases differ by 896 = -128 modulo 256: the
+// shifted field with its top bit flipped) and leading 23 fraction bits, one
+// up when the remaining 29 bits reach a half -- and lo what that leaves, an
+// integer of at most 2^28 rounded to a float, times 2^(e - 52): within 2^-50
+// relative for 2^-70 <= |x| < 2^127; 0 below 2^-126 (and lo 0 below 2^-70),
+// which only drops magnitudes under 2^-70 of the lattice values.
 __device__ __forceinline__ ff ff_from(double x)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
-    const int e = (int)((hw >> 20) & 0x7ffu) - 1023;
-    const unsigned sign = hw & 0x80000000u;
-    if (e < -126) return {0.f, 0.f};
-    const float h = __uint_as_float(sign | ((unsigned)(e + 127) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29));
-    if (e < -70) return {h, 0.f};
-    // remaining fraction m = lw mod 2^29 = mh 2^6 + ml; each part is a float
-    // exactly (2^23 + m - 2^23), the sum is rounded once
-    const unsigned m = lw & 0x1fffffffu;
-    const float mh = __fsub_rn(__uint_as_float(0x4b000000u | (m >> 6)), 8388608.f);
-    const float ml = __fsub_rn(__uint_as_float(0x4b000000u | (m & 63u)), 8388608.f);
-    const float s46 = __uint_as_float((unsigned)(e - 46 + 127) << 23);   // 2^(e - 46)
-    const float s52 = __uint_as_float((unsigned)(e - 52 + 127) << 23);   // 2^(e - 52)
-    const float l = __fmaf_rn(mh, s46, __fmul_rn(ml, s52));
-    return {h, __uint_as_float(__float_as_uint(l) | sign)};
+    const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+    const unsigned mag = hw & 0x7fffffffu;
+    const unsigned h = ((__funnelshift_l(lw, hw, 3) ^ 0x40000000u) & 0x7fffffffu) | (hw & 0x80000000u);
+    const float scale = __uint_as_float((h & 0xff800000u) - (52u << 23));       // +-2^(e - 52)
+    const int m = (int)(lw << 3) >> 3;                                          // bits 0..28, signed
+    const float lo = __fmul_rn(__int2float_rn(m), scale);
+    if (mag < ((1023u - 126u) << 20)) return {0.f, 0.f};
+    if (mag < ((1023u - 70u) << 20)) return {__uint_as_float(h), 0.f};
+    return {__uint_as_float(h + ((lw >> 28) & 1u)), lo};
 }
 
 // A normal float (or 0) as a double, by integer operations on its bits.
@@ -150,14 +145,17 @@ __device__ __forceinline__ ff ff_sqrt(ff a)
 }
 
 // 1/a for a > 0 in the normal float range: the FP32 estimate y of 1/a_hi
-// (relative error about 2^-23), e = 1 - a y from the exact product error of
-// a_hi y (1 - a_hi y is exact: the two are within a factor 2 of 1), and
-// 1/a = y / (1 - e) = y (1 + e + e^2 + ...) to second order: relative error
-// about 2^-46 (the rounding of y (e + e^2)); fpic_probe_math measures it.
+// (relative error about 2^-23), once corrected in FP32 (y (1 + e), e = 1 - a_hi
+// y by a fused multiply-add: half an ulp), then e = 1 - a y from the exact
+// product error of a_hi y (1 - a_hi y is exact: the two are within a factor
+// 2 of 1), and 1/a = y / (1 - e) = y (1 + e + e^2 + ...) to second order:
+// relative error about 2^-47 (the roundings of e and y (e + e^2));
+// fpic_probe_math measures it.
 __device__ __forceinline__ ff ff_rcp(ff a)
 {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a.hi));
+    y = __fmaf_rn(y, __fmaf_rn(-a.hi, y, 1.f), y);
     const float p = __fmul_rn(a.hi, y);
     const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.f, p), __fmaf_rn(a.hi, y, -p)), __fmul_rn(a.lo, y));
     return ff_fast2(y, __fmul_rn(y, __fmaf_rn(e, e, e)));

@@ -26,6 +26,11 @@ struct fpic_ctx {
     fpic::GridDev G{};
     // host copies of the node tables
     std::string h_nodes;             // raw bytes of rn, rh, tn, th
+    // per-cell polynomials of the deposit (dep_poly.cuh), built by the first
+    // fpic_deposit on a grid; poly_grid: the grid_gen they belong to
+    void* d_poly = nullptr;
+    unsigned long long poly_grid = ~0ull;
+    bool poly_ok = false;
     // metric tables at the Yee points (library-owned), see pic.cu
     double* d_metric = nullptr;
     size_t metric_stride = 0;        // elements per table

@@ -5,7 +5,8 @@
 // Deposit pipeline (no floating-point atomics, bitwise reproducible):
 //   k_dep_particle  one thread per particle (in cell order): the 4x4
 //                   trapezoidal subvolumes of sqrt(gamma) on each sub-grid
-//                   -> 16 node shares (rho, j^ph, j^r, j^th);
+//                   -> 16 node shares (rho, j^ph, j^r, j^th); on fine grids
+//                   from per-cell polynomials (dep_poly.cuh);
 //   k_dep_cell      one warp per cell, one lane per record row and
 //                   particle parity: fixed-order sums of the cell's
 //                   particles' shares into its 20 stencil slots;
@@ -13,7 +14,9 @@
 //                   (up to six) cells touching it, / (2 pi V_dual).
 // The FDTD is HBM-bound; its metric factors come from tables built once.
 #include <math.h>
+#include <string.h>
 
+#include "dep_poly.cuh"
 #include "ff.cuh"
 #include "fpic_internal.h"
 
@@ -895,6 +898,246 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
     k.code[p] = (uint32_t)(i1 - i0 + 1) | ((uint32_t)(j1 - j0 + 1) << 2);
 }
 
+// Builds the cells' polynomials (sub-grid blockIdx.z, row blockIdx.y), the
+// 1-D tables and the largest bound over the cells (as the bits of a
+// non-negative double; a NaN exceeds every tolerance).  Once per grid, about
+// 250 FP64 operations a cell: less than the first deposit saves.
+struct PolyBuild {
+    BH bh;
+    GridDev G;
+    float4* c[3];
+    float2* ir[2];
+    float4* t[2];
+    unsigned long long* bound;
+};
+
+__device__ __forceinline__ float2 pair_of(double d)
+{
+    const float h = (float)d;
+    return make_float2(h, (float)(d - (double)h));
+}
+
+__global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ PolyBuild k)
+{
+    const int sg = blockIdx.z, i = blockIdx.y, j = blockIdx.x * 128 + threadIdx.x;
+    const GridDev& G = k.G;
+    const bool hr = sg == 1, hth = sg == 2;
+    double e = 0.0;
+    if (i < G.Nr - hr && j < G.Nth - hth) {
+        const double* X = hr ? G.rh : G.rn;
+        const double* Y = hth ? G.th : G.tn;
+        const double dx = X[i + 1] - X[i], dy = Y[j + 1] - Y[j], y = 0.5 * (Y[j] + Y[j + 1]);
+        double f[7][7];
+        poly_series(k.bh.M, k.bh.a, 0.5 * (X[i] + X[i + 1]), y, dx, dy, f);
+        e = poly_bound(f);
+        float4* c = k.c[sg] + ((size_t)i * G.Nth + j) * (POLY_STRIDE / 4);
+        const float2 f10 = pair_of(f[1][0]), f01 = pair_of(f[0][1]), f20 = pair_of(f[2][0]), f11 = pair_of(f[1][1]),
+                     f02 = pair_of(f[0][2]);
+        c[0] = make_float4(f10.x, f10.y, f01.x, f01.y);
+        c[1] = make_float4(f20.x, f20.y, f11.x, f11.y);
+        c[2] = make_float4(f02.x, f02.y, (float)f[3][0], (float)f[2][1]);
+        c[3] = make_float4((float)f[1][2], (float)f[0][3], (float)f[4][0], (float)f[3][1]);
+        c[4] = make_float4((float)f[2][2], (float)f[1][3], (float)f[0][4], (float)f[5][0]);
+        c[5] = make_float4((float)f[4][1], (float)f[3][2], (float)f[2][3], (float)f[1][4]);
+        c[6] = make_float4((float)f[0][5], 0.f, 0.f, 0.f);
+        if (j == 0 && sg < 2) k.ir[sg][i] = pair_of(1.0 / dx);
+        if (i == 0 && sg != 1) {
+            double s, co;
+            sincos(y, &s, &co);
+            const double tau = dy * co / s;
+            const float2 it = pair_of(1.0 / dy), tp = pair_of(tau), d2 = pair_of(0.5 * dy * dy), d6 = pair_of(dy * dy / 6.0);
+            float4* t = k.t[hth] + 2 * j;
+            t[0] = make_float4(it.x, it.y, tp.x, tp.y);
+            t[1] = make_float4(d2.x, d2.y, d6.x, d6.y);
+            if (!(s > 0.0 && dy <= POLY_MAX_DTH && fabs(tau) <= POLY_MAX_TAU)) e = INFINITY;
+        }
+    }
+    // NaN bits sort above every number's
+    for (int o = 16; o > 0; o >>= 1) {
+        const double y = __shfl_xor_sync(0xffffffffu, e, o);
+        const unsigned long long be = (unsigned long long)__double_as_longlong(e) & ~(1ull << 63),
+                                 by = (unsigned long long)__double_as_longlong(y) & ~(1ull << 63);
+        e = __longlong_as_double((long long)(be > by ? be : by));
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(k.bound, (unsigned long long)__double_as_longlong(e) & ~(1ull << 63));
+}
+
+// The polynomials of the context's grid (built on first use, with one wait
+// for the bound); T filled and true where they may be used.  Not built while
+// the stream is being captured, nor beyond POLY_MAX_BYTES: the lattices serve.
+constexpr size_t POLY_MAX_BYTES = (size_t)16 << 30;
+
+static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
+{
+    use = false;
+    const size_t cells = (size_t)c->Nr * c->Nth, row = ((size_t)c->Nr + 31) & ~(size_t)31;
+    const size_t bytes = 3 * cells * POLY_STRIDE * 4 + 2 * row * 8 + 4 * (size_t)c->Nth * 16 + 256;
+    const bool fresh = c->poly_grid != c->grid_gen;
+    if (fresh) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        FPIC_CUDA(cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return 0;
+        c->poly_ok = false;
+        c->poly_grid = c->grid_gen;
+        retire(c, &c->d_poly);
+        if (bytes > POLY_MAX_BYTES) return 0;
+        if (cudaMalloc(&c->d_poly, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            c->d_poly = nullptr;
+            return 0;
+        }
+    }
+    if (!c->d_poly) return 0;
+    char* b = (char*)c->d_poly;
+    PolyBuild k{c->bh, c->G, {}, {}, {}, nullptr};
+    for (int q = 0; q < 3; ++q) k.c[q] = (float4*)(b + q * cells * POLY_STRIDE * 4);
+    b += 3 * cells * POLY_STRIDE * 4;
+    for (int q = 0; q < 2; ++q) k.t[q] = (float4*)b + q * 2 * (size_t)c->Nth;
+    b += 4 * (size_t)c->Nth * 16;
+    for (int q = 0; q < 2; ++q) k.ir[q] = (float2*)b + q * row;
+    k.bound = (unsigned long long*)(b + 2 * row * 8);
+    if (fresh) {
+        FPIC_CUDA(cudaMemsetAsync(k.bound, 0, 8, s));
+        k_poly_build<<<dim3((unsigned)((c->Nth + 127) / 128), c->Nr, 3), 128, 0, s>>>(k);
+        unsigned long long bits = 0;
+        FPIC_CUDA(cudaMemcpyAsync(&bits, k.bound, 8, cudaMemcpyDeviceToHost, s));
+        FPIC_CUDA(cudaStreamSynchronize(s));
+        double e;
+        memcpy(&e, &bits, 8);
+        c->poly_ok = e <= POLY_TOL;
+        if (!c->poly_ok) {
+            FPIC_CUDA(cudaFree(c->d_poly));
+            c->d_poly = nullptr;
+        }
+    }
+    if (!c->poly_ok) return 0;
+    const double* X = (const double*)c->h_nodes.data();      // rn, rh, tn, th (th with one node more)
+    const size_t m[4] = {(size_t)c->Nr + 1, (size_t)c->Nr, (size_t)c->Nth + 1, (size_t)c->Nth};
+    for (int q = 0; q < 4; ++q) {
+        T.lo[q] = X[0];
+        T.hi[q] = X[m[q] - 1];
+        X += m[q];
+    }
+    for (int q = 0; q < 3; ++q) T.c[q] = k.c[q];
+    for (int q = 0; q < 2; ++q) {
+        T.ir[q] = k.ir[q];
+        T.t[q] = k.t[q];
+    }
+    use = true;
+    return 0;
+}
+
+// The cell of x (held to [lo, hi]) on the m nodes X, est an FP32 estimate of
+// it, and the fractions of the cell below (al) and above (ab) x in paired
+// FP32, each from its own FP64 difference so that a small share keeps its
+// relative accuracy.
+__device__ __forceinline__ int cell_split(const double* __restrict__ X, int m, double lo, double hi, double x,
+                                          float est, double& d0, double& d1)
+{
+    const long long klo = okey(lo), khi = okey(hi);
+    long long kx = okey(x);
+    x = kx < klo ? lo : (kx > khi ? hi : x);
+    kx = okey(x);
+    int i = max(0, min(__float2int_rd(est), m - 2));
+    double X0 = __ldg(X + i), X1 = __ldg(X + i + 1);
+    while (i > 0 && kx < okey(X0)) {
+        X1 = X0;
+        X0 = __ldg(X + --i);
+    }
+    while (i < m - 2 && kx >= okey(X1)) {
+        X0 = X1;
+        X1 = __ldg(X + ++i + 1);
+    }
+    d0 = x - X0;
+    d1 = X1 - x;
+    return i;
+}
+
+// The per-particle pass on grids with polynomials: the same trapezoid rules'
+// node shares as k_dep_particle_ff without evaluating their 133 lattice
+// points.  FP64 keeps the particle's sin/cos th and FIDO velocity and the
+// positions' offsets in their cells.  The shares are stored as pairs of
+// floats: turning them into doubles is integer work that k_dep_cell, bound
+// by its FP64 additions, has the issue slots for.  FP64-pipe
+// bound (78 % busy, 68 instructions a particle) at 92 instead of 370
+// instructions per charge share: 1511 -> 552 us at 4.0e6 particles on
+// 512 x 512, 23.7 -> 9.4 ms at 6.4e7 on 1024 x 1024 (64 or 80 registers alike).
+__global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_constant__ DepK k,
+                                                              const __grid_constant__ PolyTab T)
+{
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (p >= k.n_alive) return;
+    const GridDev& G = k.G;
+    const double r = k.r[p], t = k.th[p];
+    const float lr = __logf(f32_est(r)), tf = f32_est(t);
+    double d0, d1;
+    const int j0 = cell_split(G.tn, G.Nth + 1, T.lo[2], T.hi[2], t, (tf - G.t0) * G.it, d0, d1);
+    Mom X[2], Y[2];
+    MomT E[2];
+    {
+        const float4 t0 = __ldg(T.t[0] + 2 * j0), t1 = __ldg(T.t[0] + 2 * j0 + 1);
+        const ff inv = {t0.x, t0.y};
+        moments(ff_mul(ff_from(d0), inv), ff_mul(ff_from(d1), inv), Y);
+        moments_th(Y, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}, E);
+    }
+    // FIDO three-velocity, as k_dep_particle_ff (sin/cos th by angle addition
+    // from the node on the side where the terms share a sign)
+    ff Q, Qr, Qt, Qp;
+    {
+        const double* sn = k.trig;
+        const double* cn = k.trig + (G.Nth + 1);
+        const int jn = j0 + (__double2hiint(cn[j0]) < 0 ? 1 : 0);
+        double sd, cm;
+        sincos_step(t - G.tn[jn], sd, cm);
+        const double s = fma(sn[jn], cm, fma(cn[jn], sd, sn[jn])), c = fma(cn[jn], cm, fma(-sn[jn], sd, cn[jn]));
+        const double ur = k.ur[p], ut = k.uth[p], up = k.uph[p];
+        Geo g;
+        geo_eval(k.bh, r, s, c, g);
+        const double Ur = fma(g.gurr, ur, g.gurp * up), Ut = g.gutt * ut, Up = fma(g.gurp, ur, g.gupp * up);
+        const double Qd = k.w[p] * k.qm[p];
+        const double QiG = Qd * rsqrt_nr(fma(ur, Ur, fma(ut, Ut, fma(up, Up, 1.0))));
+        Q = ff_from(Qd);
+        Qr = ff_from(QiG * Ur);
+        Qt = ff_from(QiG * Ut);
+        Qp = ff_from(QiG * Up);
+    }
+    const long long n = k.n_alive;
+    float2* rec = (float2*)k.rec + p;
+    auto put = [&](int row, ff q, const ff w[4]) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const ff v = ff_mul(q, w[b]);
+            rec[(row + b) * n] = make_float2(v.hi, v.lo);
+        }
+    };
+    ff w[4];
+    const int i1 = cell_split(G.rh, G.Nr, T.lo[1], T.hi[1], r, (lr - G.lrh0) * G.ilr, d0, d1);
+    {   // (i+1/2, j): j^r
+        const float2 ir = __ldg(T.ir[1] + i1);
+        moments(ff_mul(ff_from(d0), {ir.x, ir.y}), ff_mul(ff_from(d1), {ir.x, ir.y}), X);
+        poly_shares(T.c[1] + ((size_t)i1 * G.Nth + j0) * (POLY_STRIDE / 4), X, E, w);
+        put(8, Qr, w);
+    }
+    const int i0 = cell_split(G.rn, G.Nr + 1, T.lo[0], T.hi[0], r, (lr - G.lr0) * G.ilr, d0, d1);
+    {   // (i, j): rho and j^ph
+        const float2 ir = __ldg(T.ir[0] + i0);
+        moments(ff_mul(ff_from(d0), {ir.x, ir.y}), ff_mul(ff_from(d1), {ir.x, ir.y}), X);
+        poly_shares(T.c[0] + ((size_t)i0 * G.Nth + j0) * (POLY_STRIDE / 4), X, E, w);
+        put(0, Q, w);
+        put(4, Qp, w);
+    }
+    const int j1 = cell_split(G.th, G.Nth, T.lo[3], T.hi[3], t, (tf - G.th0) * G.it, d0, d1);
+    {   // (i, j+1/2): j^th
+        const float4 t0 = __ldg(T.t[1] + 2 * j1), t1 = __ldg(T.t[1] + 2 * j1 + 1);
+        const ff inv = {t0.x, t0.y};
+        moments(ff_mul(ff_from(d0), inv), ff_mul(ff_from(d1), inv), Y);
+        moments_th(Y, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}, E);
+        poly_shares(T.c[2] + ((size_t)i0 * G.Nth + j1) * (POLY_STRIDE / 4), X, E, w);
+        put(12, Qt, w);
+    }
+    k.code[p] = (uint32_t)(i1 - i0 + 1) | ((uint32_t)(j1 - j0 + 1) << 2);
+}
+
 // Slots of a cell (i0, j0): rho[a + 2b] (0..3), j^ph[a + 2b] (4..7),
 // j^r[k + 3b] at half-r node i0 - 1 + k (8..13), j^th[a + 2k] at half-th
 // node j0 - 1 + k (14..19).  A particle with offsets (ko, kt) (each 0 or 1)
@@ -922,6 +1165,12 @@ __device__ __forceinline__ double sel_bits(bool p, double a, double b)
     return r;
 }
 
+// PAIRS: the shares are pairs of floats (k_dep_particle_poly).  The high
+// floats are summed in FP64, the low ones (2^-24 of them) in FP32: 2^-48 of the
+// sum of |share|, under the shares' own rounding, at one FP64 addition a
+// share (198 -> 235 us at 4.0e6 particles in 262144 cells, for 16 conversions a
+// particle less in the FP64-bound kernel before it).
+template <bool PAIRS>
 __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* __restrict__ rec,
                                                                    const uint32_t* __restrict__ code,
                                                                    const uint32_t* __restrict__ off,
@@ -939,6 +1188,7 @@ __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* 
     const int bsh = row >= 12 ? 2 : 0;      // the offset bit this row splits on
     const uint32_t bmask = row >= 8 ? 1u : 0u;
     double acc0 = 0.0, acc1 = 0.0;
+    float lo0 = 0.f, lo1 = 0.f;
     for (uint32_t base = b0; base < b1; base += 32) {
         const uint32_t cnt = min(32u, b1 - base);
         const bool live = (uint32_t)lane < cnt;
@@ -955,8 +1205,16 @@ __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* 
         const int kend = (int)(cnt + 1) >> 1;
         for (int k = 0; k < kend; ++k) {
             const int pp = 2 * k + par;     // a particle past the group's end holds zeros
-            const double y = v[row * DEP_CELL_LD + pp];
+            double y = v[row * DEP_CELL_LD + pp];
             const bool bit = ((cw[pp] >> bsh) & bmask) != 0u;
+            if (PAIRS) {
+                const float2 f = make_float2(__uint_as_float((unsigned)__double2loint(y)),
+                                             __uint_as_float((unsigned)__double2hiint(y)));
+                y = f2d_bits(f.x);
+                const float s = (bit ? lo1 : lo0) + f.y;
+                lo1 = bit ? s : lo1;
+                lo0 = bit ? lo0 : s;
+            }
             const double s = sel_bits(bit, acc1, acc0) + y;
             acc1 = sel_bits(bit, s, acc1);
             acc0 = sel_bits(bit, acc0, s);
@@ -981,7 +1239,15 @@ __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* 
     const int la = 2 * (ra & 15), lb = 2 * (rb & 15);
     const double xa0 = __shfl_sync(0xffffffffu, acc0, la), xa1 = __shfl_sync(0xffffffffu, acc1, la);
     const double xb0 = __shfl_sync(0xffffffffu, acc0, lb);
-    if (lane < 20) part[(size_t)lane * C + cell] = (ua ? xa1 : xa0) + (rb >= 0 ? xb0 : 0.0);
+    double tot = (ua ? xa1 : xa0) + (rb >= 0 ? xb0 : 0.0);
+    if (PAIRS) {
+        lo0 += __shfl_xor_sync(0xffffffffu, lo0, 1);
+        lo1 += __shfl_xor_sync(0xffffffffu, lo1, 1);
+        const float la0 = __shfl_sync(0xffffffffu, lo0, la), la1 = __shfl_sync(0xffffffffu, lo1, la);
+        const float lb0 = __shfl_sync(0xffffffffu, lo0, lb);
+        tot += f2d_bits((ua ? la1 : la0) + (rb >= 0 ? lb0 : 0.f));
+    }
+    if (lane < 20) part[(size_t)lane * C + cell] = tot;
 }
 
 struct NodeK {
@@ -1320,17 +1586,25 @@ extern "C" int fpic_deposit(fpic_ctx* c, fpic_particles* p, double* rho, double*
     } else {
         FPIC_CUDA(cudaMemsetAsync(w.off, 0, 4 * ((size_t)C + 2), s));
     }
+    PolyTab pt;
+    bool poly = false;
+    if (n > 0 && c->dep_lattice) {
+        rc = poly_tables(c, pt, poly, s);
+        if (rc) return rc;
+    }
     // alive particles occupy [0, off[C]) after the sort; the count is read on the device
     DepK k{c->bh, bh_ff(c->bh), c->G, c->d_metric + (size_t)MT_N * c->metric_stride, p->r, p->th, p->ur, p->uth, p->uph, p->qm, p->w, n, w.rec, w.code};
     if (n > 0) {
         // rec/code for all n slots; removed particles (past off[C]) are never summed
         const int dt_ = c->dep_threads;
         const unsigned nb = (unsigned)((n + dt_ - 1) / dt_);
-        if (c->dep_lattice) k_dep_particle_ff<<<nb, dt_, 0, s>>>(k);
-        else k_dep_particle<<<nb, dt_, 0, s>>>(k);
+        if (!c->dep_lattice) k_dep_particle<<<nb, dt_, 0, s>>>(k);
+        else if (poly) k_dep_particle_poly<<<nb, dt_, 0, s>>>(k, pt);
+        else k_dep_particle_ff<<<nb, dt_, 0, s>>>(k);
     }
-    k_dep_cell<<<(unsigned)(((long long)C + DEP_CELL_WARPS - 1) / DEP_CELL_WARPS), 32 * DEP_CELL_WARPS, 0, s>>>(
-        w.rec, w.code, w.off, w.part, n > 0 ? n : 1, C);
+    const unsigned cb = (unsigned)(((long long)C + DEP_CELL_WARPS - 1) / DEP_CELL_WARPS);
+    if (poly) k_dep_cell<true><<<cb, 32 * DEP_CELL_WARPS, 0, s>>>(w.rec, w.code, w.off, w.part, n, C);
+    else k_dep_cell<false><<<cb, 32 * DEP_CELL_WARPS, 0, s>>>(w.rec, w.code, w.off, w.part, n > 0 ? n : 1, C);
     NodeK nk{c->Nr, c->Nth, c->ld, w.part, C, tabs_of(c), rho, jr, jth, jph};
     k_dep_node<<<dim3(1, c->Nr + 1), 256, 0, s>>>(nk);
     FPIC_CUDA(cudaGetLastError());
