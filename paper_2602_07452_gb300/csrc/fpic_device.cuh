@@ -216,6 +216,22 @@ __device__ __forceinline__ double fmax_nonneg(double m, double a)
     return (ba > F64_INF_BITS || ba <= bm) ? m : a;
 }
 
+// x / 2 by taking one from the exponent, off the FP64 pipe; zeros, numbers
+// near or below the normal range, infinities and NaNs go through the
+// multiplication: the product's value for every x.
+__device__ __forceinline__ double half_of(double x)
+{
+    const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
+    if (e - 0x00200000u < 0x7fd00000u) return __hiloint2double(__double2hiint(x) - 0x00100000, __double2loint(x));
+    return 0.5 * x;
+}
+
+// x == 1 by an integer compare.
+__device__ __forceinline__ bool is_one(double x)
+{
+    return __double_as_longlong(x) == 0x3ff0000000000000LL;
+}
+
 // Order-preserving integer key of a double (monotone for all non-NaN values).
 __device__ __forceinline__ long long okey(double x)
 {

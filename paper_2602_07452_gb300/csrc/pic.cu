@@ -12,7 +12,7 @@
 //                   particles' shares into its 20 stencil slots;
 //   k_dep_node      one thread per node: fixed-order sum of the slots of the
 //                   (up to six) cells touching it, / (2 pi V_dual).
-// The FDTD is HBM-bound; its metric factors come from tables built once.
+// The FDTD's metric factors come from tables built once.
 #include <math.h>
 #include <string.h>
 
@@ -25,24 +25,32 @@ namespace fpic {
 // ---------------------------------------------------------------------------
 // Metric tables
 // ---------------------------------------------------------------------------
-// type t: 0 (i, j), 1 (i+1/2, j), 2 (i, j+1/2), 3 (i+1/2, j+1/2)
-// quantity q: 0 alpha, 1 beta, 2 sqrt(gamma), 3 g_rr, 4 g_rp, 5 g_tt, 6 g_pp,
-// 7 1/sqrt(gamma) (the FDTD multiplies by it instead of dividing)
-// tables 32..34: 2 pi x dual-cell volume of the (i,j), (i+1/2,j), (i,j+1/2) grids
-// then sin/cos of the integer and half th nodes.
-enum { MT_Q = 8, MT_DUAL = 32, MT_N = 35 };
+// Points: 0 (i, j), 1 (i+1/2, j), 2 (i, j+1/2), 3 (i+1/2, j+1/2).  First what
+// cleaning and the deposits read: sqrt(gamma), lower metric components, 2 pi x
+// the dual-cell volumes; then the field update's coefficients (see the FDTD
+// section), each product of metric factors, average weights and reciprocal
+// spacings formed once: 11 FP64 operations for E or H at a node instead of
+// 35, and no factor read that is not used as it is.  Then sin/cos of the
+// integer and half th nodes.
+enum {
+    T_SG0, T_SG1, T_SG2, T_RR0, T_RP0, T_PP0, T_RR1, T_RP1, T_PP1, T_TT2, T_DUAL0, T_DUAL1, T_DUAL2,
+    // E_r = ER_D D^r + ER_P0 D^ph_i + ER_P1 D^ph_{i+1}; E_th, E_ph alike (0: row i - 1, 1: row i, held at the ends)
+    F_ER_D, F_ER_P0, F_ER_P1, F_ET_D, F_ET_B0, F_ET_B1, F_EP_D, F_EP_R0, F_EP_R1, F_EP_T0, F_EP_T1,
+    F_HR_B, F_HR_P0, F_HR_P1, F_HT_B, F_HT_D0, F_HT_D1, F_HP_B, F_HP_R0, F_HP_R1, F_HP_T0, F_HP_T1,
+    // curls: 1 / (sqrt(gamma) x spacing)
+    F_BR, F_BT, F_BPR, F_BPT, F_DR, F_DT, F_DPR, F_DPT,
+    // -4 pi J, J = alpha j - rho beta: JR j^r + JR0 rho_i + JR1 rho_{i+1}, JT j^th, JP j^ph
+    F_JR, F_JR0, F_JR1, F_JT, F_JP,
+    MT_N
+};
 
 struct Tabs {
     const double* m;   // MT_N tables of size sz, then 2 (Nth+1) + 2 Nth trig values
     size_t sz;
     int ld;
-    __device__ __forceinline__ double at(int t, int q, int i, int j) const
+    __device__ __forceinline__ double at(int t, int i, int j) const
     {
-        return m[(size_t)(t * MT_Q + q) * sz + (size_t)i * ld + j];
-    }
-    __device__ __forceinline__ double dual(int t, int i, int j) const
-    {
-        return m[(size_t)(MT_DUAL + t) * sz + (size_t)i * ld + j];
+        return m[(size_t)t * sz + (size_t)i * ld + j];
     }
 };
 
@@ -68,47 +76,150 @@ __device__ double trap16_dev(const BH& bh, double x0, double x1, double y0, doub
     return acc * hx * hy;
 }
 
-__global__ void k_metric_tables(BH bh, GridDev G, double* m, size_t sz)
+// A thread walks `rows` rows of one th column: the trigonometry of its
+// points and of the dual cells' quadrature is taken once, and each row's
+// metric serves the averages of its neighbours.
+__device__ __forceinline__ double dual_sum(const BH& bh, double x0, double x1, double dy, const double s[4],
+                                           const double A[4])
 {
-    const int i = blockIdx.y;
-    for (int j = threadIdx.x; j <= G.Nth; j += blockDim.x) {
-        for (int t = 0; t < 4; ++t) {
-            const bool ro = t & 1, to = t & 2;
-            if ((ro && i >= G.Nr) || (to && j >= G.Nth)) continue;
-            const double r = ro ? G.rh[i] : G.rn[i];
-            const double th = to ? G.th[j] : G.tn[j];
-            double s, c;
-            sincos(th, &s, &c);
-            Geo g;
-            geo_eval(bh, r, s, c, g);
-            const double v[MT_Q] = {g.alpha, g.beta, g.sqrtg, g.grr, g.grp, g.gtt, g.gpp, 1.0 / g.sqrtg};
-            for (int q = 0; q < MT_Q; ++q) m[(size_t)(t * MT_Q + q) * sz + (size_t)i * G.ld + j] = v[q];
+    const double hx = (x1 - x0) / 3.0;
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double x = x0 + k * hx, X = x * x;
+        double row = 0.0;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            const double P = X + A[l], q = P * fma(bh.twoM, x, P);
+            const double f = s[l] * (q * rsqrt_nr(q));
+            row += (l == 0 || l == 3) ? 0.5 * f : f;
         }
-        // dual-cell volumes of the (i,j), (i+1/2,j), (i,j+1/2) sub-grids
-        for (int t = 0; t < 3; ++t) {
-            const bool ro = (t == 1), to = (t == 2);
-            if ((ro && i >= G.Nr) || (to && j >= G.Nth)) continue;
-            double x0, x1, y0, y1;
-            if (ro) { x0 = G.rn[i]; x1 = G.rn[i + 1]; }
-            else { x0 = i == 0 ? G.rn[0] : G.rh[i - 1]; x1 = i == G.Nr ? G.rn[G.Nr] : G.rh[i]; }
-            if (to) { y0 = G.tn[j]; y1 = G.tn[j + 1]; }
-            else { y0 = j == 0 ? G.tn[0] : G.th[j - 1]; y1 = j == G.Nth ? G.tn[G.Nth] : G.th[j]; }
-            m[(size_t)(MT_DUAL + t) * sz + (size_t)i * G.ld + j] = 2.0 * M_PI * trap16_dev(bh, x0, x1, y0, y1);
+        acc += (k == 0 || k == 3) ? 0.5 * row : row;
+    }
+    return 2.0 * M_PI * acc * hx * (dy / 3.0);
+}
+
+__global__ void __launch_bounds__(128) k_metric_tables(BH bh, GridDev G, double* m, size_t sz, int rows)
+{
+    const int j = blockIdx.x * 128 + threadIdx.x, i0 = blockIdx.y * rows, i1 = min(i0 + rows, G.Nr + 1);
+    if (j > G.Nth) return;
+    const bool in = j < G.Nth;               // half th points exist
+    const double mfpi = -4.0 * M_PI;
+    double sn, cn, sh, ch;
+    sincos(G.tn[j], &sn, &cn);
+    sincos(G.th[j], &sh, &ch);
+    if (blockIdx.y == 0) {
+        double* trig = m + (size_t)MT_N * sz;
+        trig[j] = sn;
+        trig[(G.Nth + 1) + j] = cn;
+        if (in) {
+            trig[2 * (G.Nth + 1) + j] = sh;
+            trig[2 * (G.Nth + 1) + G.Nth + j] = ch;
         }
     }
-    if (i == 0) {
-        double* trig = m + (size_t)MT_N * sz;
-        for (int j = threadIdx.x; j <= G.Nth; j += blockDim.x) {
-            double s, c;
-            sincos(G.tn[j], &s, &c);
-            trig[j] = s;
-            trig[(G.Nth + 1) + j] = c;
-            if (j < G.Nth) {
-                sincos(G.th[j], &s, &c);
-                trig[2 * (G.Nth + 1) + j] = s;
-                trig[2 * (G.Nth + 1) + G.Nth + j] = c;
-            }
+    // th lattices of the dual cells about the integer and the half node
+    double sa[4], Aa[4], sb[4], Ab[4];
+    const double ya0 = j == 0 ? G.tn[0] : G.th[j - 1], ya1 = in ? G.th[j] : G.tn[G.Nth];
+    const double yb0 = G.tn[j], yb1 = in ? G.tn[j + 1] : yb0;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+        double s, c;
+        sincos(ya0 + l * ((ya1 - ya0) / 3.0), &s, &c);
+        sa[l] = s;
+        Aa[l] = bh.a2 * c * c;
+        sincos(yb0 + l * ((yb1 - yb0) / 3.0), &s, &c);
+        sb[l] = s;
+        Ab[l] = bh.a2 * c * c;
+    }
+    const double itn = in ? G.itn[j] : 0.0, ith = G.ith[j > 0 ? j - 1 : G.Nth - 1];
+    Geo g0, g1, g2, g3, n0, n2;
+    double s1m, s3m;                         // sqrt(gamma) of points 1 and 3 one row below (held at row 0)
+    geo_eval(bh, G.rn[i0], sn, cn, g0);
+    geo_eval(bh, G.rn[i0], sh, ch, g2);
+    {
+        const int im = max(i0 - 1, 0);
+        geo_eval(bh, G.rh[im], sn, cn, g1);
+        s1m = g1.sqrtg;
+        geo_eval(bh, G.rh[im], sh, ch, g3);
+        s3m = g3.sqrtg;
+    }
+    for (int i = i0; i < i1; ++i) {
+        const bool half = i < G.Nr;          // half r points exist
+        double* o = m + (size_t)i * G.ld + j;
+        auto put = [&](int t, double v) { o[(size_t)t * sz] = v; };
+        const double x0 = i == 0 ? G.rn[0] : G.rh[i - 1], x1 = half ? G.rh[i] : G.rn[G.Nr];
+        if (half) {
+            geo_eval(bh, G.rh[i], sn, cn, g1);
+            geo_eval(bh, G.rh[i], sh, ch, g3);
+            geo_eval(bh, G.rn[i + 1], sn, cn, n0);
+            geo_eval(bh, G.rn[i + 1], sh, ch, n2);
         }
+        const double s1 = half ? g1.sqrtg : s1m, s3 = half ? g3.sqrtg : s3m;    // held at the last row
+        const double irn = half ? G.irn[i] : 0.0, irh = (i >= 1 && half) ? G.irh[i - 1] : 0.0;
+        {   // (i, j)
+            const double is = 1.0 / g0.sqrtg, k = 0.5 * g0.alpha * g0.grp * is;
+            put(T_SG0, g0.sqrtg);
+            put(T_RR0, g0.grr);
+            put(T_RP0, g0.grp);
+            put(T_PP0, g0.gpp);
+            put(T_DUAL0, dual_sum(bh, x0, x1, ya1 - ya0, sa, Aa));
+            put(F_EP_D, g0.alpha * g0.gpp);
+            put(F_EP_R0, k * s1m);
+            put(F_EP_R1, k * s1);
+            put(F_EP_T0, 0.5 * g0.beta * s1m);
+            put(F_EP_T1, 0.5 * g0.beta * s1);
+            put(F_DPR, irh * is);
+            put(F_DPT, ith * is);
+            put(F_JP, mfpi * g0.alpha);
+        }
+        if (in) {   // (i, j+1/2)
+            const double is = 1.0 / g2.sqrtg, k = 0.5 * g2.alpha * g2.grp * is;
+            put(T_SG2, g2.sqrtg);
+            put(T_TT2, g2.gtt);
+            put(T_DUAL2, dual_sum(bh, x0, x1, yb1 - yb0, sb, Ab));
+            put(F_ET_D, g2.alpha * g2.gtt);
+            put(F_ET_B0, -0.5 * g2.beta * s3m);
+            put(F_ET_B1, -0.5 * g2.beta * s3);
+            put(F_HR_B, g2.alpha * g2.grr);
+            put(F_HR_P0, k * s3m);
+            put(F_HR_P1, k * s3);
+            put(F_BR, itn * is);
+            put(F_DT, irh * is);
+            put(F_JT, mfpi * g2.alpha);
+        }
+        if (half) {   // (i+1/2, j)
+            const double is = 1.0 / g1.sqrtg, k = 0.5 * g1.alpha * g1.grp * is;
+            put(T_SG1, g1.sqrtg);
+            put(T_RR1, g1.grr);
+            put(T_RP1, g1.grp);
+            put(T_PP1, g1.gpp);
+            put(T_DUAL1, dual_sum(bh, G.rn[i], G.rn[i + 1], ya1 - ya0, sa, Aa));
+            put(F_ER_D, g1.alpha * g1.grr);
+            put(F_ER_P0, k * g0.sqrtg);
+            put(F_ER_P1, k * n0.sqrtg);
+            put(F_HT_B, g1.alpha * g1.gtt);
+            put(F_HT_D0, 0.5 * g1.beta * g0.sqrtg);
+            put(F_HT_D1, 0.5 * g1.beta * n0.sqrtg);
+            put(F_BT, irn * is);
+            put(F_DR, ith * is);
+            put(F_JR, mfpi * g1.alpha);
+            put(F_JR0, -0.5 * mfpi * g1.beta * is * g0.sqrtg);
+            put(F_JR1, -0.5 * mfpi * g1.beta * is * n0.sqrtg);
+        }
+        if (half && in) {   // (i+1/2, j+1/2)
+            const double is = 1.0 / g3.sqrtg, k = 0.5 * g3.alpha * g3.grp * is;
+            put(F_HP_B, g3.alpha * g3.gpp);
+            put(F_HP_R0, k * g2.sqrtg);
+            put(F_HP_R1, k * n2.sqrtg);
+            put(F_HP_T0, -0.5 * g3.beta * g2.sqrtg);
+            put(F_HP_T1, -0.5 * g3.beta * n2.sqrtg);
+            put(F_BPR, irn * is);
+            put(F_BPT, itn * is);
+        }
+        s1m = s1;
+        s3m = s3;
+        g0 = n0;
+        g2 = n2;
     }
 }
 
@@ -119,8 +230,12 @@ int build_metric_tables(fpic_ctx* c)
     retire(c, (void**)&c->d_metric);
     FPIC_CUDA(cudaMalloc(&c->d_metric, tot * sizeof(double)));
     c->metric_stride = sz;
-    dim3 grid(1, c->Nr + 1);
-    k_metric_tables<<<grid, 128>>>(c->bh, c->G, c->d_metric, sz);
+    // the trigonometry of a thread costs about two rows: as few rows as keep
+    // two blocks on every SM, 16 at most
+    const long long cols = c->Nth / 128 + 1;
+    int rows = 16;
+    while (rows > 1 && cols * (c->Nr / rows + 1) < 2LL * c->sm_count) rows >>= 1;
+    k_metric_tables<<<dim3((unsigned)cols, (unsigned)(c->Nr / rows + 1)), 128>>>(c->bh, c->G, c->d_metric, sz, rows);
     FPIC_CUDA(cudaGetLastError());
     return 0;
 }
@@ -1276,8 +1391,8 @@ __global__ void k_dep_node(NodeK k)
                 sr += P(a + 2 * b, ci, cj);
                 sp += P(4 + a + 2 * b, ci, cj);
             }
-        k.rho[o] = sr / k.T.dual(0, i, j);
-        k.jp[o] = sp / k.T.dual(0, i, j);
+        k.rho[o] = sr / k.T.at(T_DUAL0, i, j);
+        k.jp[o] = sp / k.T.at(T_DUAL0, i, j);
         // j^r at (i+1/2, j): cells (i + 1 - kk, j - b), slot kk + 3b
         if (i < Nr) {
             double sj = 0.0;
@@ -1287,7 +1402,7 @@ __global__ void k_dep_node(NodeK k)
                     if (ci < 0 || ci >= Nr || cj < 0 || cj >= Nth) continue;
                     sj += P(8 + kk + 3 * b, ci, cj);
                 }
-            k.jr[o] = sj / k.T.dual(1, i, j);
+            k.jr[o] = sj / k.T.at(T_DUAL1, i, j);
         }
         // j^th at (i, j+1/2): cells (i - a, j + 1 - kk), slot a + 2 kk
         if (j < Nth) {
@@ -1298,7 +1413,7 @@ __global__ void k_dep_node(NodeK k)
                     if (ci < 0 || ci >= Nr || cj < 0 || cj >= Nth) continue;
                     sj += P(14 + a + 2 * kk, ci, cj);
                 }
-            k.jt[o] = sj / k.T.dual(2, i, j);
+            k.jt[o] = sj / k.T.at(T_DUAL2, i, j);
         }
     }
 }
@@ -1306,226 +1421,273 @@ __global__ void k_dep_node(NodeK k)
 // ---------------------------------------------------------------------------
 // FDTD (Sec. 2.1, Eqs. m3, m4, Ei; Sec. 2.5)
 // ---------------------------------------------------------------------------
+// Four launches a step, k_step_B twice in stage 1 and k_step_D twice in stage
+// 2, each an auxiliary field and the update by its curl in one pass:
+//   E_r (i+1/2,j) = alpha (g_rr D^r + g_rp <D^ph>),  E_th (i,j+1/2) = alpha g_tt
+//   D^th - sqrtg beta <B^ph>,  E_ph (i,j) = alpha (g_rp <D^r> + g_pp D^ph) +
+//   sqrtg beta <B^th>  (Eq. Ei; <.> the sqrtg-weighted mean of the two rows);
+//   H_r (i,j+1/2) = alpha (g_rr B^r + g_rp <B^ph>),  H_th (i+1/2,j) = alpha g_tt
+//   B^th + sqrtg beta <D^ph>,  H_ph (i+1/2,j+1/2) = alpha (g_rp <B^r> + g_pp
+//   B^ph) - sqrtg beta <D^th>.
+// A warp owns 31 adjacent columns (its 32nd lane holds the neighbour column
+// the th differences need, exchanged by shuffles) and walks down `rows` rows
+// with the neighbouring rows' values in registers: every array is read once
+// and E, H go to memory only where the caller gets them (sub-steps 3 and 9).
+// Bound by the FP64 pipe (75-78 % busy on about 160 operations a node and
+// step; halvings and the tests for a factor of one are integer operations),
+// with 140 doubles a node of traffic behind it.  Before, with E, H and the
+// averages as arrays of their own, their metric products per node and the
+// absorbing layer's exp and pow in every thread, it was 13 launches: a step
+// on 1024 x 1024 809 -> 400 us, 4196 x 1024 full-theta 2645 -> 1433 us.
 struct FK {
-    int Nr, Nth, ld;
+    int rows;           // rows of a warp, at most 16
     GridDev G;
     Tabs T;
     double dt, chi0, lam, r_abs, r_max;
     int conserving;     // sources are coordinate currents J (fpic_deposit_conserving)
 };
 
+struct P3 {
+    double* p[3];
+};
+
+struct C3 {
+    const double* p[3];
+};
+
+constexpr int FD_THREADS = 128, FD_COLS = 31;    // columns of a warp
+
+// x^n with the products' rounding errors carried along: within an ulp.
+__device__ __forceinline__ double powi_acc(double x, int n)
+{
+    double h = x, l = 0.0;
+    for (int k = 1; k < n; ++k) {
+        const double t = h * x, e = fma(h, x, -t);
+        l = fma(l, x, e);
+        h = t;
+    }
+    return h + l;
+}
+
+// Absorbing-layer factor exp(-chi dt), chi = chi0 ((r - r_abs)/(r_max -
+// r_abs))^lambda beyond r_abs (Eqs. abs0-abs2).  A small whole lambda by
+// multiplications: pow's latency would be most of a short launch.
 __device__ __forceinline__ double damp(const FK& k, double r)
 {
     if (k.chi0 <= 0.0 || r <= k.r_abs) return 1.0;
     const double x = (r - k.r_abs) / (k.r_max - k.r_abs);
-    return exp(-k.chi0 * pow(x, k.lam) * k.dt);
+    const int n = (int)k.lam;
+    const double y = (k.lam == (double)n && n >= 1 && n <= 8) ? powi_acc(x, n) : pow(x, k.lam);
+    return exp(-k.chi0 * y * k.dt);
 }
 
-// metric-weighted average of F (staggering ro, to) to the point of the other
-// r staggering at index i2 (zero-gradient beyond the ends)
-__device__ __forceinline__ double avg_r(const FK& k, const double* F, int ro, int to, int i2, int j)
+// The factors of rows i0 .. i0 + 15, integer (lanes 0-15) and half (16-31).
+__device__ __forceinline__ double damp_rows(const FK& k, int i0, int lane)
 {
-    int ia = ro ? i2 - 1 : i2, ib = ro ? i2 : i2 + 1;
-    const int m = ro ? k.Nr : k.Nr + 1;
-    if (ia < 0) ia = ib;
-    if (ib > m - 1) ib = ia;
-    const int tF = (ro ? 1 : 0) | (to ? 2 : 0), tT = (ro ? 0 : 1) | (to ? 2 : 0);
-    const double sa = k.T.at(tF, 2, ia, j), sb = k.T.at(tF, 2, ib, j), ist = k.T.at(tT, 7, i2, j);
-    return fma(sa, F[(size_t)ia * k.ld + j], sb * F[(size_t)ib * k.ld + j]) * (0.5 * ist);
+    const int i = i0 + (lane & 15);
+    if (lane < 16) return i <= k.G.Nr ? damp(k, k.G.rn[i]) : 1.0;
+    return i < k.G.Nr ? damp(k, k.G.rh[i]) : 1.0;
 }
 
-struct F3 {
-    const double *a[3], *b[3];   // value = b ? 0.5 (a + b) : a  (pointwise level average)
-    __device__ __forceinline__ double v(int c, size_t o) const
-    {
-        return b[c] ? 0.5 * (a[c][o] + b[c][o]) : a[c][o];
-    }
-};
-
-struct O3 {
-    double* p[3];
-};
-
-__global__ void k_avg3(F3 in, O3 out, size_t sz)
-{
-    for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < sz; o += (size_t)gridDim.x * blockDim.x)
-        for (int c = 0; c < 3; ++c) out.p[c][o] = in.v(c, o);
-}
-
-// Eq. (Ei): E_r (i+1/2,j) = alpha (g_rr D^r + g_rp <D^ph>);
-// E_th (i,j+1/2) = alpha g_tt D^th - sqrtg beta <B^ph>;
-// E_ph (i,j) = alpha (g_rp <D^r> + g_pp D^ph) + sqrtg beta <B^th>.
 // Full-theta domain (Sec. 2.5, periodic in th): columns 0..Nth-1 are the
 // distinct points; the thread of column 0 also stores its values in column
 // Nth, the image the seam's stencils and the push's gather read.
-__device__ __forceinline__ void put(double* F, size_t o, int j, const FK& k, double v)
+__device__ __forceinline__ void put(double* F, size_t o, int j, const GridDev& G, double v)
 {
     F[o] = v;
-    if (k.G.full && j == 0) F[o + k.Nth] = v;
+    if (G.full && j == 0) F[o + G.Nth] = v;
 }
 
-__global__ void k_make_E(FK k, F3 D, F3 B, O3 E)
+// Eq. (m4) + (abs0): Bout = (Bin - dt curl E / sqrtg) exp(-chi dt).  FIRST
+// (sub-steps 1, 2): E from D = (D0 + D1) / 2 and B1, Bin = (B0 + B1) / 2; else
+// (sub-steps 3, 4) E from D1 and Bh, stored, and Bin = B1.
+template <bool FIRST>
+__global__ void __launch_bounds__(FD_THREADS) k_step_B(const __grid_constant__ FK k, C3 D0, C3 D1, C3 B0, C3 B1,
+                                                       C3 Bh, P3 E, P3 Bout)
 {
-    const int i = blockIdx.y;
-    const int jend = k.G.full ? k.Nth - 1 : k.Nth;
-    for (int j = threadIdx.x; j <= jend; j += blockDim.x) {
-        const size_t o = (size_t)i * k.ld + j;
-        if (i < k.Nr) {
-            const double Dp = avg_r(k, D.a[2], 0, 0, i, j);
-            put(E.p[0], o, j, k, k.T.at(1, 0, i, j) * fma(k.T.at(1, 3, i, j), D.a[0][o], k.T.at(1, 4, i, j) * Dp));
-        }
-        if (j < k.Nth) {
-            const double Bp = avg_r(k, B.a[2], 1, 1, i, j);
-            put(E.p[1], o, j, k, fma(k.T.at(2, 0, i, j) * k.T.at(2, 5, i, j), D.a[1][o],
-                                     -k.T.at(2, 2, i, j) * k.T.at(2, 1, i, j) * Bp));
-        }
-        const double Dr = avg_r(k, D.a[0], 1, 0, i, j);
-        const double Bt = avg_r(k, B.a[1], 1, 0, i, j);
-        put(E.p[2], o, j, k, fma(k.T.at(0, 0, i, j), fma(k.T.at(0, 4, i, j), Dr, k.T.at(0, 6, i, j) * D.a[2][o]),
-                                 k.T.at(0, 2, i, j) * k.T.at(0, 1, i, j) * Bt));
-    }
-}
-
-// H_r (i,j+1/2) = alpha (g_rr B^r + g_rp <B^ph>);  H_th (i+1/2,j) = alpha g_tt
-// B^th + sqrtg beta <D^ph>;  H_ph (i+1/2,j+1/2) = alpha (g_rp <B^r> + g_pp B^ph)
-// - sqrtg beta <D^th>.
-__global__ void k_make_H(FK k, F3 D, F3 B, O3 H)
-{
-    const int i = blockIdx.y;
-    const int jend = k.G.full ? k.Nth - 1 : k.Nth;
-    for (int j = threadIdx.x; j <= jend; j += blockDim.x) {
-        const size_t o = (size_t)i * k.ld + j;
-        if (j < k.Nth) {
-            const double Bp = avg_r(k, B.a[2], 1, 1, i, j);
-            put(H.p[0], o, j, k, k.T.at(2, 0, i, j) * fma(k.T.at(2, 3, i, j), B.a[0][o], k.T.at(2, 4, i, j) * Bp));
-        }
-        if (i < k.Nr) {
-            const double Dp = avg_r(k, D.a[2], 0, 0, i, j);
-            put(H.p[1], o, j, k, fma(k.T.at(1, 0, i, j) * k.T.at(1, 5, i, j), B.a[1][o],
-                                     k.T.at(1, 2, i, j) * k.T.at(1, 1, i, j) * Dp));
-        }
-        if (i < k.Nr && j < k.Nth) {
-            const double Br = avg_r(k, B.a[0], 0, 1, i, j);
-            const double Dt = avg_r(k, D.a[1], 0, 1, i, j);
-            put(H.p[2], o, j, k, fma(k.T.at(3, 0, i, j), fma(k.T.at(3, 4, i, j), Br, k.T.at(3, 6, i, j) * B.a[2][o]),
-                                     -k.T.at(3, 2, i, j) * k.T.at(3, 1, i, j) * Dt));
-        }
-    }
-}
-
-// Eq. (m4) + (abs0): B_out = (B_in - dt curl E / sqrtg) exp(-chi dt).
-// The forward th differences at j = Nth-1 read column Nth: the image of
-// column 0 in the full-theta domain.
-__global__ void k_update_B(FK k, F3 Bin, O3 E, O3 Bout)
-{
-    const int i = blockIdx.y;
     const GridDev& G = k.G;
-    const int jend = G.full ? k.Nth - 1 : k.Nth;
-    // the damping factor depends on the row only; 1/dr of the row
-    const double dn = damp(k, G.rn[i]), dh = i < k.Nr ? damp(k, G.rh[i]) : 1.0;
-    const double idr = i < k.Nr ? G.irn[i] : 0.0;
-    for (int j = threadIdx.x; j <= jend; j += blockDim.x) {
-        const size_t o = (size_t)i * k.ld + j;
-        if (j < k.Nth) {   // B^r (i, j+1/2)
-            const double curl = (E.p[2][o + 1] - E.p[2][o]) * G.itn[j];
-            put(Bout.p[0], o, j, k, (Bin.v(0, o) - k.dt * curl * k.T.at(2, 7, i, j)) * dn);
+    const int lane = threadIdx.x & 31;
+    const int Nr = G.Nr, Nth = G.Nth;
+    const int j = (blockIdx.x * (FD_THREADS / 32) + (threadIdx.x >> 5)) * FD_COLS + lane;
+    if (j - lane > Nth) return;              // whole warps
+    const int i0 = blockIdx.y * k.rows, i1 = min(i0 + k.rows, Nr + 1);
+    const int jend = G.full ? Nth - 1 : Nth;
+    const bool out = lane < FD_COLS && j <= jend;
+    const bool in = j < Nth;                 // half th points
+    // column read: the image column is column 0 itself, idle lanes read the last
+    const int jj = (G.full && j == Nth) ? 0 : min(j, Nth);
+    const double dmp = damp_rows(k, i0, lane);
+    const size_t ld = (size_t)G.ld, sz = k.T.sz;
+    const C3& Be = FIRST ? B1 : Bh;
+    auto mean = [](double x, double y) { return half_of(x + y); };
+    auto D = [&](int c, size_t o) { return FIRST ? mean(__ldg(D0.p[c] + o), __ldg(D1.p[c] + o)) : __ldg(D1.p[c] + o); };
+    size_t o = (size_t)i0 * ld + jj;
+    const double* T = k.T.m + o;
+    auto tab = [&](int t) { return __ldg(T + (size_t)t * sz); };
+    // row i0's E_th, E_ph
+    double Dr, Dp = D(2, o), Bt, Bp, Et, Ep;
+    {
+        const size_t om = i0 > 0 ? o - ld : o, oc = i0 < Nr ? o : o - ld;
+        const double Drm = D(0, om), Btm = __ldg(Be.p[1] + om), Bpm = __ldg(Be.p[2] + om);
+        Dr = D(0, oc);
+        Bt = __ldg(Be.p[1] + oc);
+        Bp = __ldg(Be.p[2] + oc);
+        Et = fma(tab(F_ET_D), D(1, o), fma(tab(F_ET_B0), Bpm, tab(F_ET_B1) * Bp));
+        Ep = fma(tab(F_EP_D), Dp, fma(tab(F_EP_R0), Drm, tab(F_EP_R1) * Dr));
+        Ep = fma(tab(F_EP_T0), Btm, fma(tab(F_EP_T1), Bt, Ep));
+    }
+    for (int i = i0; i < i1; ++i, o += ld, T += ld) {
+        const double dn = __shfl_sync(0xffffffffu, dmp, i - i0), dh = __shfl_sync(0xffffffffu, dmp, 16 + i - i0);
+        const double EpR = __shfl_down_sync(0xffffffffu, Ep, 1);
+        if (!FIRST && out) {
+            if (in) put(E.p[1], o, j, G, Et);
+            put(E.p[2], o, j, G, Ep);
         }
-        if (i < k.Nr) {    // B^th (i+1/2, j)
-            const double curl = -(E.p[2][o + k.ld] - E.p[2][o]) * idr;
-            put(Bout.p[1], o, j, k, (Bin.v(1, o) - k.dt * curl * k.T.at(1, 7, i, j)) * dh);
+        if (out && in) {   // B^r (i, j+1/2)
+            const double b = FIRST ? mean(__ldg(B0.p[0] + o), __ldg(B1.p[0] + o)) : __ldg(B1.p[0] + o);
+            double v = fma(-k.dt, tab(F_BR) * (EpR - Ep), b);
+            if (!is_one(dn)) v *= dn;
+            put(Bout.p[0], o, j, G, v);
         }
-        if (i < k.Nr && j < k.Nth) {   // B^ph (i+1/2, j+1/2)
-            const double dEt = (E.p[1][o + k.ld] - E.p[1][o]) * idr;
-            const double dEr = (E.p[0][o + 1] - E.p[0][o]) * G.itn[j];
-            put(Bout.p[2], o, j, k, (Bin.v(2, o) - k.dt * (dEt - dEr) * k.T.at(3, 7, i, j)) * dh);
+        if (i == Nr) break;
+        // row i+1 (its own half row held at Nr - 1)
+        const size_t on = o + ld, oc = i + 1 < Nr ? on : o;
+        const double Dpn = D(2, on), Drn = D(0, oc), Btn = __ldg(Be.p[1] + oc), Bpn = __ldg(Be.p[2] + oc);
+        const double Er = fma(tab(F_ER_D), Dr, fma(tab(F_ER_P0), Dp, tab(F_ER_P1) * Dpn));
+        auto tabn = [&](int t) { return __ldg(T + ld + (size_t)t * sz); };
+        const double Etn = fma(tabn(F_ET_D), D(1, on), fma(tabn(F_ET_B0), Bp, tabn(F_ET_B1) * Bpn));
+        double Epn = fma(tabn(F_EP_D), Dpn, fma(tabn(F_EP_R0), Dr, tabn(F_EP_R1) * Drn));
+        Epn = fma(tabn(F_EP_T0), Bt, fma(tabn(F_EP_T1), Btn, Epn));
+        const double ErR = __shfl_down_sync(0xffffffffu, Er, 1);
+        if (out) {
+            if (!FIRST) put(E.p[0], o, j, G, Er);
+            {   // B^th (i+1/2, j)
+                const double b = FIRST ? mean(__ldg(B0.p[1] + o), Bt) : __ldg(B1.p[1] + o);
+                double v = fma(k.dt, tab(F_BT) * (Epn - Ep), b);
+                if (!is_one(dh)) v *= dh;
+                put(Bout.p[1], o, j, G, v);
+            }
+            if (in) {   // B^ph (i+1/2, j+1/2)
+                const double b = FIRST ? mean(__ldg(B0.p[2] + o), Bp) : __ldg(B1.p[2] + o);
+                double v = fma(-k.dt, fma(tab(F_BPR), Etn - Et, -tab(F_BPT) * (ErR - Er)), b);
+                if (!is_one(dh)) v *= dh;
+                put(Bout.p[2], o, j, G, v);
+            }
         }
+        Et = Etn;
+        Ep = Epn;
+        Dr = Drn;
+        Dp = Dpn;
+        Bt = Btn;
+        Bp = Bpn;
     }
 }
 
 struct Src {
     const double *j[3], *rho;
-    double w;
 };
 
-// J = alpha j - rho beta at the J^k point (rho averaged to J^r's point)
-__device__ __forceinline__ double jsrc(const FK& k, const Src& S, int comp, int i, int j)
+// Eq. (m3) + (abs1): Dout = (Din + dt [curl H / sqrtg - 4 pi J]) exp(-chi dt).
+// FIRST (sub-steps 7, 8): H from B and D = D1, Din = (D0 + D1) / 2, J the mean
+// of both levels; else (9, 10) H from B and D = Dw, stored, Din = D1, J = S1.
+// Interior points; the boundaries follow from them (Sec. 2.5, reading: zero
+// gradient where a stencil is one-sided, D^ph = 0 on the axis) and are stored
+// by the threads of the rows and columns they copy.  Full-theta domain: D^r
+// and D^ph at j = 0 too, their backward th difference across the seam (half
+// node Nth-1), no th boundary.
+template <bool FIRST>
+__global__ void __launch_bounds__(FD_THREADS) k_step_D(const __grid_constant__ FK k, C3 D0, C3 D1, C3 D, C3 B, Src S0,
+                                                       Src S1, P3 H, P3 Dout)
 {
-    if (S.w == 0.0) return 0.0;
-    const size_t o = (size_t)i * k.ld + j;
-    if (k.conserving) return S.w * S.j[comp][o];
-    if (comp == 0) {
-        const double rb = avg_r(k, S.rho, 0, 0, i, j);
-        return S.w * fma(k.T.at(1, 0, i, j), S.j[0][o], -rb * k.T.at(1, 1, i, j));
-    }
-    if (comp == 1) return S.w * (k.T.at(2, 0, i, j) * S.j[1][o]);
-    return S.w * (k.T.at(0, 0, i, j) * S.j[2][o]);
-}
-
-// Eq. (m3) + (abs1): D_out = (D_in + dt [curl H / sqrtg - 4 pi J]) exp(-chi dt),
-// interior points only (boundaries: k_bc_D).  Full-theta domain: D^r and D^ph
-// at j = 0 too, their backward th difference across the seam (half node
-// Nth-1, one period below: spacing th[Nth] - th[Nth-1], th[Nth] = th[0] + P).
-__global__ void k_update_D(FK k, F3 Din, O3 H, Src S0, Src S1, O3 Dout)
-{
-    const int i = blockIdx.y;
     const GridDev& G = k.G;
-    const double fpi = 4.0 * M_PI;
-    const int jlo = G.full ? 0 : 1;
-    // the damping factor depends on the row only; 1/dr of the row
-    const double dn = damp(k, G.rn[i]), dh = i < k.Nr ? damp(k, G.rh[i]) : 1.0;
-    const double idr = (i >= 1 && i < k.Nr) ? G.irh[i - 1] : 0.0;
-    for (int j = threadIdx.x; j < k.Nth; j += blockDim.x) {
-        const size_t o = (size_t)i * k.ld + j;
-        const size_t om = j > 0 ? o - 1 : o + (k.Nth - 1);
-        const double idth = G.ith[j > 0 ? j - 1 : k.Nth - 1];     // 1/(th[j] - th[j-1]), across the seam at j = 0
-        if (i < k.Nr && j >= jlo) {    // D^r (i+1/2, j)
-            const double curl = (H.p[2][o] - H.p[2][om]) * idth;
-            const double J = jsrc(k, S0, 0, i, j) + jsrc(k, S1, 0, i, j);
-            put(Dout.p[0], o, j, k, (Din.v(0, o) + k.dt * fma(curl, k.T.at(1, 7, i, j), -fpi * J)) * dh);
-        }
-        if (i >= 1 && i < k.Nr) {    // D^th (i, j+1/2)
-            const double curl = -(H.p[2][o] - H.p[2][o - k.ld]) * idr;
-            const double J = jsrc(k, S0, 1, i, j) + jsrc(k, S1, 1, i, j);
-            put(Dout.p[1], o, j, k, (Din.v(1, o) + k.dt * fma(curl, k.T.at(2, 7, i, j), -fpi * J)) * dn);
-        }
-        if (i >= 1 && i < k.Nr && j >= jlo) {   // D^ph (i, j)
-            const double dHt = (H.p[1][o] - H.p[1][o - k.ld]) * idr;
-            const double dHr = (H.p[0][o] - H.p[0][om]) * idth;
-            const double J = jsrc(k, S0, 2, i, j) + jsrc(k, S1, 2, i, j);
-            put(Dout.p[2], o, j, k, (Din.v(2, o) + k.dt * fma(dHt - dHr, k.T.at(0, 7, i, j), -fpi * J)) * dn);
-        }
-    }
-}
-
-// Sec. 2.5 (reading): zero gradient where a stencil is one-sided, D^ph = 0 on
-// the axis rows (k_axis_D).  Full-theta domain: no th boundary; the radial
-// boundary rows copy every column, the image column Nth included.
-__global__ void k_bc_D(FK k, O3 D)
-{
-    const int i = blockIdx.y;
-    const int Nr = k.Nr, Nth = k.Nth, ld = k.ld;
-    const bool full = k.G.full;
-    if (threadIdx.x == 0 && !full) {
+    const int lane = threadIdx.x & 31;
+    const int Nr = G.Nr, Nth = G.Nth;
+    const int j = (blockIdx.x * (FD_THREADS / 32) + (threadIdx.x >> 5)) * FD_COLS + lane - 1;
+    if (j - lane + 1 > Nth) return;          // whole warps
+    const int i0 = blockIdx.y * k.rows, i1 = min(i0 + k.rows, Nr + 1);
+    const bool out = lane > 0 && j <= (G.full ? Nth - 1 : Nth);
+    const bool in = j < Nth;                 // half th points
+    const bool mid = out && in && (G.full || j >= 1);            // D^r, D^ph updated
+    // column read: below column 0 the period's last, idle lanes the last
+    const int jj = j < 0 ? (G.full ? Nth - 1 : 0) : min(j, Nth);
+    const double dmp = damp_rows(k, i0, lane);
+    const size_t ld = (size_t)G.ld, sz = k.T.sz;
+    const double mfpi = -4.0 * M_PI;
+    auto mean = [](double x, double y) { return half_of(x + y); };
+    auto Din = [&](int c, size_t o, double d1) { return FIRST ? mean(__ldg(D0.p[c] + o), d1) : __ldg(D1.p[c] + o); };
+    auto src = [&](int c, size_t o) { return FIRST ? mean(__ldg(S0.j[c] + o), __ldg(S1.j[c] + o)) : __ldg(S1.j[c] + o); };
+    auto rho = [&](size_t o) { return FIRST ? mean(__ldg(S0.rho + o), __ldg(S1.rho + o)) : __ldg(S1.rho + o); };
+    const int is = max(i0 - 1, 0);           // row i0 - 1's H_th, H_ph come first
+    size_t o = (size_t)is * ld + jj;
+    const double* T = k.T.m + o;
+    auto tab = [&](int t) { return __ldg(T + (size_t)t * sz); };
+    double Br = __ldg(B.p[0] + o), Dt = __ldg(D.p[1] + o), Dp = __ldg(D.p[2] + o), Bp = is > 0 ? __ldg(B.p[2] + o - ld) : __ldg(B.p[2] + o);
+    double Htm = 0.0, Hpm = 0.0, rh = k.conserving ? 0.0 : rho((size_t)i0 * ld + jj);
+    for (int i = is; i < i1; ++i, o += ld, T += ld) {
+        const bool own = i >= i0;
+        double Ht = 0.0, Hp = 0.0, Bpi = Bp, Brn = 0.0, Dtn = 0.0, Dpn = 0.0, Bt = 0.0;
         if (i < Nr) {
-            D.p[0][(size_t)i * ld + 0] = D.p[0][(size_t)i * ld + 1];
-            D.p[0][(size_t)i * ld + Nth] = D.p[0][(size_t)i * ld + Nth - 1];
+            const size_t on = o + ld;
+            Bpi = __ldg(B.p[2] + o);
+            Bt = __ldg(B.p[1] + o);
+            Brn = __ldg(B.p[0] + on);
+            Dtn = __ldg(D.p[1] + on);
+            Dpn = __ldg(D.p[2] + on);
+            Ht = fma(tab(F_HT_B), Bt, fma(tab(F_HT_D0), Dp, tab(F_HT_D1) * Dpn));
+            Hp = fma(tab(F_HP_B), Bpi, fma(tab(F_HP_R0), Br, tab(F_HP_R1) * Brn));
+            Hp = fma(tab(F_HP_T0), Dt, fma(tab(F_HP_T1), Dtn, Hp));
         }
-    }
-    const int jt = full ? Nth : Nth - 1, jp0 = full ? 0 : 1, jp1 = full ? Nth : Nth - 1;
-    for (int j = threadIdx.x; j <= Nth; j += blockDim.x) {
-        if (i == 0 && j <= jt) D.p[1][j] = D.p[1][(size_t)ld + j];
-        if (i == Nr && j <= jt) D.p[1][(size_t)Nr * ld + j] = D.p[1][(size_t)(Nr - 1) * ld + j];
-        if (i == 0 && j >= jp0 && j <= jp1) D.p[2][j] = D.p[2][(size_t)ld + j];
-        if (i == Nr && j >= jp0 && j <= jp1) D.p[2][(size_t)Nr * ld + j] = D.p[2][(size_t)(Nr - 1) * ld + j];
-    }
-}
-
-__global__ void k_axis_D(FK k, O3 D)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i <= k.Nr) {
-        D.p[2][(size_t)i * k.ld + 0] = 0.0;
-        D.p[2][(size_t)i * k.ld + k.Nth] = 0.0;
+        if (own) {
+            // Bp: row i - 1 (row 0 at the lower end), Bpi: row i (row Nr - 1 at the upper end)
+            const double Hr = fma(tab(F_HR_B), Br, fma(tab(F_HR_P0), Bp, tab(F_HR_P1) * Bpi));
+            const double dn = __shfl_sync(0xffffffffu, dmp, i - i0), dh = __shfl_sync(0xffffffffu, dmp, 16 + i - i0);
+            const double HrL = __shfl_up_sync(0xffffffffu, Hr, 1), HpL = __shfl_up_sync(0xffffffffu, Hp, 1);
+            if (!FIRST && out) {
+                if (in) put(H.p[0], o, j, G, Hr);
+                if (i < Nr) put(H.p[1], o, j, G, Ht);
+                if (i < Nr && in) put(H.p[2], o, j, G, Hp);
+            }
+            if (mid && i < Nr) {   // D^r (i+1/2, j)
+                double J = (k.conserving ? mfpi : tab(F_JR)) * src(0, o);
+                if (!k.conserving) {
+                    const double rn = rho(o + ld);
+                    J = fma(tab(F_JR0), rh, fma(tab(F_JR1), rn, J));
+                    rh = rn;
+                }
+                const double d = FIRST ? __ldg(D1.p[0] + o) : 0.0;
+                double v = fma(k.dt, fma(tab(F_DR), Hp - HpL, J), Din(0, o, d));
+                if (!is_one(dh)) v *= dh;
+                put(Dout.p[0], o, j, G, v);
+                if (!G.full) {
+                    if (j == 1) Dout.p[0][o - 1] = v;
+                    if (j == Nth - 1) Dout.p[0][o + 1] = v;
+                }
+            }
+            if (i >= 1 && i < Nr && out && in) {   // D^th (i, j+1/2)
+                const double J = (k.conserving ? mfpi : tab(F_JT)) * src(1, o);
+                double v = fma(k.dt, fma(-tab(F_DT), Hp - Hpm, J), Din(1, o, Dt));
+                if (!is_one(dn)) v *= dn;
+                put(Dout.p[1], o, j, G, v);
+                if (i == 1) put(Dout.p[1], o - ld, j, G, v);
+                if (i == Nr - 1) put(Dout.p[1], o + ld, j, G, v);
+            }
+            if (i >= 1 && i < Nr && mid) {   // D^ph (i, j)
+                const double J = (k.conserving ? mfpi : tab(F_JP)) * src(2, o);
+                const double c = fma(tab(F_DPR), Ht - Htm, fma(-tab(F_DPT), Hr - HrL, J));
+                double v = fma(k.dt, c, Din(2, o, Dp));
+                if (!is_one(dn)) v *= dn;
+                put(Dout.p[2], o, j, G, v);
+                if (i == 1) put(Dout.p[2], o - ld, j, G, v);
+                if (i == Nr - 1) put(Dout.p[2], o + ld, j, G, v);
+            }
+            if (!G.full && out && (j == 0 || j == Nth)) Dout.p[2][o] = 0.0;
+        }
+        Htm = Ht;
+        Hpm = Hp;
+        Bp = Bpi;
+        Br = Brn;
+        Dt = Dtn;
+        Dp = Dpn;
     }
 }
 
@@ -1805,12 +1967,12 @@ __global__ void k_cdep_node(CDepK k, Tabs T, const double* __restrict__ part, ui
                 if (y < 2) Ft += part[(size_t)(CD_T + 2 * x + y) * C + cell];
             }
         const double drd = cd_dual_r(G, i), dtd = cd_dual_t(G, j);
-        const double vol = 2.0 * M_PI * T.at(0, 2, i, j) * drd * dtd;
+        const double vol = 2.0 * M_PI * T.at(T_SG0, i, j) * drd * dtd;
         rho[o] = vol > 0.0 ? Q / vol : 0.0;
         Jp[o] = vol > 0.0 ? Pp / vol : 0.0;
-        if (i < k.Nr) Jr[o] = Fr / (dt * 2.0 * M_PI * T.at(1, 2, i, j) * dtd);
+        if (i < k.Nr) Jr[o] = Fr / (dt * 2.0 * M_PI * T.at(T_SG1, i, j) * dtd);
         else Jr[o] = 0.0;
-        if (j < k.Nth) Jt[o] = Ft / (dt * 2.0 * M_PI * T.at(2, 2, i, j) * drd);
+        if (j < k.Nth) Jt[o] = Ft / (dt * 2.0 * M_PI * T.at(T_SG2, i, j) * drd);
         else Jt[o] = 0.0;
     }
 }
@@ -1885,15 +2047,15 @@ struct CleanK {
 
 // Inverse spatial metric from the tabulated lower one: the th block is
 // diagonal, the (r, ph) block a 2 x 2 inverse.
-__device__ __forceinline__ double tab_gu_rr(const Tabs& T, int t, int i, int j)
+__device__ __forceinline__ double tab_gu_rr(const Tabs& T, int i, int j)       // at (i+1/2, j)
 {
-    const double grr = T.at(t, 3, i, j), grp = T.at(t, 4, i, j), gpp = T.at(t, 6, i, j);
+    const double grr = T.at(T_RR1, i, j), grp = T.at(T_RP1, i, j), gpp = T.at(T_PP1, i, j);
     return gpp / fma(grr, gpp, -grp * grp);
 }
 
-__device__ __forceinline__ double tab_gu_rp(const Tabs& T, int t, int i, int j)
+__device__ __forceinline__ double tab_gu_rp(const Tabs& T, int i, int j)       // at (i, j)
 {
-    const double grr = T.at(t, 3, i, j), grp = T.at(t, 4, i, j), gpp = T.at(t, 6, i, j);
+    const double grr = T.at(T_RR0, i, j), grp = T.at(T_RP0, i, j), gpp = T.at(T_PP0, i, j);
     return -grp / fma(grr, gpp, -grp * grp);
 }
 
@@ -1908,15 +2070,15 @@ __global__ void k_clean_setup(CleanK k, const double* __restrict__ Dr, const dou
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= k.Nth; j += gridDim.x * blockDim.x) {
         const size_t o = (size_t)i * k.ld + j;
         const double dth = (j < k.Nth ? G.th[j] : M_PI) - (j > 0 ? G.th[j - 1] : 0.0);
-        const double sr1 = T.at(1, 2, i, j), sr0 = T.at(1, 2, i - 1, j);
-        const double st1 = j < k.Nth ? T.at(2, 2, i, j) : 0.0, st0 = j > 0 ? T.at(2, 2, i, j - 1) : 0.0;
+        const double sr1 = T.at(T_SG1, i, j), sr0 = T.at(T_SG1, i - 1, j);
+        const double st1 = j < k.Nth ? T.at(T_SG2, i, j) : 0.0, st0 = j > 0 ? T.at(T_SG2, i, j - 1) : 0.0;
         const double rhs = (sr1 * Dr[o] - sr0 * Dr[o - k.ld]) / dr +
                            ((j < k.Nth ? st1 * Dt[o] : 0.0) - (j > 0 ? st0 * Dt[o - 1] : 0.0)) / dth -
-                           4.0 * M_PI * T.at(0, 2, i, j) * rho[o];
-        const double cr1 = sr1 * tab_gu_rr(T, 1, i, j) * ir1;
-        const double cr0 = sr0 * tab_gu_rr(T, 1, i - 1, j) * ir0;
-        const double ct1 = j < k.Nth ? st1 / (T.at(2, 5, i, j) * (G.tn[j + 1] - G.tn[j]) * dth) : 0.0;
-        const double ct0 = j > 0 ? st0 / (T.at(2, 5, i, j - 1) * (G.tn[j] - G.tn[j - 1]) * dth) : 0.0;
+                           4.0 * M_PI * T.at(T_SG0, i, j) * rho[o];
+        const double cr1 = sr1 * tab_gu_rr(T, i, j) * ir1;
+        const double cr0 = sr0 * tab_gu_rr(T, i - 1, j) * ir0;
+        const double ct1 = j < k.Nth ? st1 / (T.at(T_TT2, i, j) * (G.tn[j + 1] - G.tn[j]) * dth) : 0.0;
+        const double ct0 = j > 0 ? st0 / (T.at(T_TT2, i, j - 1) * (G.tn[j] - G.tn[j - 1]) * dth) : 0.0;
         const double inv = 1.0 / (cr1 + cr0 + ct1 + ct0);
         k.c_r1[o] = cr1 * inv;
         k.c_r0[o] = cr0 * inv;
@@ -1967,9 +2129,9 @@ __global__ void k_clean_correct(CleanK k, const double* __restrict__ phi, double
         const double up = i < k.Nr ? (phi[o + k.ld] - phi[o]) * iu : 0.0;
         const double dn = i > 0 ? (phi[o] - phi[o - k.ld]) * id : 0.0;
         const double mean = (i > 0 && i < k.Nr) ? 0.5 * (up + dn) : up + dn;
-        if (i < k.Nr) Dr[o] -= tab_gu_rr(T, 1, i, j) * up;
-        if (j < k.Nth) Dt[o] -= (phi[o + 1] - phi[o]) / (T.at(2, 5, i, j) * (G.tn[j + 1] - G.tn[j]));
-        Dp[o] -= tab_gu_rp(T, 0, i, j) * mean;
+        if (i < k.Nr) Dr[o] -= tab_gu_rr(T, i, j) * up;
+        if (j < k.Nth) Dt[o] -= (phi[o + 1] - phi[o]) / (T.at(T_TT2, i, j) * (G.tn[j + 1] - G.tn[j]));
+        Dp[o] -= tab_gu_rp(T, i, j) * mean;
     }
 }
 
@@ -2246,43 +2408,30 @@ extern "C" int fpic_fdtd_step(fpic_ctx* c, fpic_fields* f, const fpic_fdtd_param
     if (!f->rho0 || !f->rho1) return set_error(FPIC_EINVAL, "fpic_fdtd_step: NULL rho array");
     FPIC_CUDA(cudaSetDevice(c->device));
     cudaStream_t s = (cudaStream_t)stream;
-    FK k{c->Nr, c->Nth, c->ld, c->G, tabs_of(c), prm->dt, prm->chi0, prm->lambda, prm->r_abs, prm->r_max,
-         prm->conserving};
-    const size_t sz = (size_t)(c->Nr + 1) * c->ld;
-    const dim3 g2(1, c->Nr + 1);
-    const int TB = 256;
-    auto f3 = [](double* const a[3], double* const b[3]) {
-        F3 r;
-        for (int q = 0; q < 3; ++q) { r.a[q] = a[q]; r.b[q] = b ? b[q] : nullptr; }
-        return r;
-    };
-    auto o3 = [](double* const a[3]) { O3 r; for (int q = 0; q < 3; ++q) r.p[q] = a[q]; return r; };
+    // rows a warp walks: the first row's auxiliary field is worked out twice,
+    // so as many as keep 16 warps on every SM, 16 at most
+    const long long cols = (c->Nth + FD_COLS) / FD_COLS;
+    int rows = 16;
+    while (rows > 1 && cols * ((c->Nr + rows) / rows) < 16LL * c->sm_count) rows >>= 1;
+    const FK k{rows, c->G, tabs_of(c), prm->dt, prm->chi0, prm->lambda, prm->r_abs, prm->r_max, prm->conserving};
+    const dim3 grid((unsigned)((cols + FD_THREADS / 32 - 1) / (FD_THREADS / 32)), (unsigned)((c->Nr + rows) / rows));
+    auto c3 = [](double* const a[3]) { return C3{{a[0], a[1], a[2]}}; };
+    auto p3 = [](double* const a[3]) { return P3{{a[0], a[1], a[2]}}; };
     if (stage == 1) {
-        // [1] E^{n+1} = alpha <D>^{n+1} + beta x B^{n+1}, <D> materialised in Dw
-        k_avg3<<<1024, TB, 0, s>>>(f3(f->D0, f->D1), o3(f->Dw), sz);
-        k_make_E<<<g2, TB, 0, s>>>(k, f3(f->Dw, nullptr), f3(f->B1, nullptr), o3(f->E));
-        // [2] B^{n+3/2} = <B>^{n+1/2} - dt curl E^{n+1}
-        k_update_B<<<g2, TB, 0, s>>>(k, f3(f->B0, f->B1), o3(f->E), o3(f->Bh));
-        // [3] E^{n+3/2}
-        k_make_E<<<g2, TB, 0, s>>>(k, f3(f->D1, nullptr), f3(f->Bh, nullptr), o3(f->E));
-        // [4] B^{n+2} = B^{n+1} - dt curl E^{n+3/2}  (into B0)
-        k_update_B<<<g2, TB, 0, s>>>(k, f3(f->B1, nullptr), o3(f->E), o3(f->B0));
+        // [1] E^{n+1} = alpha <D>^{n+1} + beta x B^{n+1}, [2] B^{n+3/2} = <B>^{n+1/2} - dt curl E^{n+1}
+        k_step_B<true><<<grid, FD_THREADS, 0, s>>>(k, c3(f->D0), c3(f->D1), c3(f->B0), c3(f->B1), c3(f->B1),
+                                                   p3(f->E), p3(f->Bh));
+        // [3] E^{n+3/2}, [4] B^{n+2} = B^{n+1} - dt curl E^{n+3/2}  (into B0)
+        k_step_B<false><<<grid, FD_THREADS, 0, s>>>(k, c3(f->D0), c3(f->D1), c3(f->B0), c3(f->B1), c3(f->Bh),
+                                                    p3(f->E), p3(f->B0));
     } else {
-        // [7] H^{n+3/2} = alpha B^{n+3/2} - beta x D^{n+3/2}
-        k_make_H<<<g2, TB, 0, s>>>(k, f3(f->D1, nullptr), f3(f->Bh, nullptr), o3(f->H));
-        // [8] D^{n+2} = <D>^{n+1} + dt [curl H - 4 pi <J>^{n+3/2}]  (into Dw)
-        Src S0{{f->j0[0], f->j0[1], f->j0[2]}, f->rho0, 0.5}, S1{{f->j1[0], f->j1[1], f->j1[2]}, f->rho1, 0.5};
-        k_update_D<<<g2, TB, 0, s>>>(k, f3(f->D0, f->D1), o3(f->H), S0, S1, o3(f->Dw));
-        k_bc_D<<<g2, TB, 0, s>>>(k, o3(f->Dw));
-        if (!c->G.full) k_axis_D<<<(c->Nr + 1 + 255) / 256, 256, 0, s>>>(k, o3(f->Dw));
-        // [9] H^{n+2} = alpha B^{n+2} - beta x D^{n+2}
-        k_make_H<<<g2, TB, 0, s>>>(k, f3(f->Dw, nullptr), f3(f->B0, nullptr), o3(f->H));
-        // [10] D^{n+5/2} = D^{n+3/2} + dt [curl H - 4 pi J^{n+2}]  (into D0)
-        S0.w = 0.0;
-        S1.w = 1.0;
-        k_update_D<<<g2, TB, 0, s>>>(k, f3(f->D1, nullptr), o3(f->H), S0, S1, o3(f->D0));
-        k_bc_D<<<g2, TB, 0, s>>>(k, o3(f->D0));
-        if (!c->G.full) k_axis_D<<<(c->Nr + 1 + 255) / 256, 256, 0, s>>>(k, o3(f->D0));
+        const Src S0{{f->j0[0], f->j0[1], f->j0[2]}, f->rho0}, S1{{f->j1[0], f->j1[1], f->j1[2]}, f->rho1};
+        // [7] H^{n+3/2} = alpha B^{n+3/2} - beta x D^{n+3/2}, [8] D^{n+2} = <D>^{n+1} + dt [curl H - 4 pi <J>^{n+3/2}]
+        k_step_D<true><<<grid, FD_THREADS, 0, s>>>(k, c3(f->D0), c3(f->D1), c3(f->D1), c3(f->Bh), S0, S1, p3(f->H),
+                                                   p3(f->Dw));
+        // [9] H^{n+2} = alpha B^{n+2} - beta x D^{n+2}, [10] D^{n+5/2} = D^{n+3/2} + dt [curl H - 4 pi J^{n+2}]  (into D0)
+        k_step_D<false><<<grid, FD_THREADS, 0, s>>>(k, c3(f->D0), c3(f->D1), c3(f->Dw), c3(f->B0), S0, S1, p3(f->H),
+                                                    p3(f->D0));
     }
     FPIC_CUDA(cudaGetLastError());
     return FPIC_OK;
