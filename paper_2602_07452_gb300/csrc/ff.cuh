@@ -18,8 +18,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
-
-#include "fpic_device.cuh"
+#include <stdint.h>
 
 namespace fpic {
 
@@ -45,18 +44,20 @@ __device__ __forceinline__ ff ff_of(float a)
 // shifted field with its top bit flipped) and leading 23 fraction bits, one
 // up when the remaining 29 bits reach a half -- and lo what that leaves, an
 // integer of at most 2^28 rounded to a float, times 2^(e - 52): within 2^-50
-// relative for 2^-70 <= |x| < 2^127; 0 below 2^-126 (and lo 0 below 2^-70),
-// which only drops magnitudes under 2^-70 of the lattice values.
+// relative for 2^-98 <= |x| < 2^127; 0 below 2^-126 (and lo 0 below 2^-98),
+// which only drops magnitudes far under the values this is used on.
+constexpr unsigned F64_HI_2M126 = (1023u - 126u) << 20, F64_HI_2M98 = (1023u - 98u) << 20;
+
 __device__ __forceinline__ ff ff_from(double x)
 {
     const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
     const unsigned mag = hw & 0x7fffffffu;
     const unsigned h = ((__funnelshift_l(lw, hw, 3) ^ 0x40000000u) & 0x7fffffffu) | (hw & 0x80000000u);
-    const float scale = __uint_as_float((h & 0xff800000u) - (52u << 23));       // +-2^(e - 52)
+    const float scale = __uint_as_float((h & 0xff800000u) - (28u << 23));       // +-2^(e - 28)
     const int m = (int)(lw << 3) >> 3;                                          // bits 0..28, signed
-    const float lo = __fmul_rn(__int2float_rn(m), scale);
-    if (mag < ((1023u - 126u) << 20)) return {0.f, 0.f};
-    if (mag < ((1023u - 70u) << 20)) return {__uint_as_float(h), 0.f};
+    const float lo = __fmul_rn(__fmul_rn(__int2float_rn(m), 5.9604644775390625e-8f), scale);
+    if (mag < F64_HI_2M126) return {0.f, 0.f};
+    if (mag < F64_HI_2M98) return {__uint_as_float(h), 0.f};
     return {__uint_as_float(h + ((lw >> 28) & 1u)), lo};
 }
 
@@ -73,6 +74,22 @@ __device__ __forceinline__ double f2d_bits(float f)
 __device__ __forceinline__ double ff_to(ff a)
 {
     return f2d_bits(a.hi) + f2d_bits(a.lo);
+}
+
+// The pair's sum as a double by integer operations, off the FP64 pipe: h,
+// the sum rounded towards zero, leaves a remainder of its own sign below one
+// of its last places, which in units of the last place of h's double (2^(e -
+// 52)) is an integer added to that double's bits; to 2^-47 relative.
+__device__ __forceinline__ double ff_to_bits(ff a)
+{
+    const float h = __fadd_rz(a.hi, a.lo), l = __fadd_rn(__fsub_rn(a.hi, h), a.lo);
+    const unsigned u = __float_as_uint(h), ex = u & 0x7f800000u;
+    // l sign(h) 2^-e: the reciprocal power of two has the exponent field 254 - e8
+    const float s = __uint_as_float((u & 0x80000000u) | ((254u << 23) - ex));
+    const int off = __float2int_rn(__fmul_rn(__fmul_rn(l, s), 4503599627370496.f));
+    const unsigned hw = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20));
+    const long long b = (long long)(((unsigned long long)hw << 32) | (u << 29)) + off;
+    return ex ? __longlong_as_double(b) : 0.0;
 }
 
 __device__ __forceinline__ ff ff_add(ff a, ff b)
@@ -159,36 +176,6 @@ __device__ __forceinline__ ff ff_rcp(ff a)
     const float p = __fmul_rn(a.hi, y);
     const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.f, p), __fmaf_rn(a.hi, y, -p)), __fmul_rn(a.lo, y));
     return ff_fast2(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
-}
-
-// sin h and cos h - 1 of a step h in paired FP32 (the deposit's th
-// lattice rotations).  Below 2^-7 by the Maclaurin series: h - h^3/6 and
-// -h^2/2 in paired arithmetic, the next terms (h^5/120; h^4/24 - h^6/720),
-// below 2^-28 relative, in FP32, the omitted ones below 2^-48 of the
-// result: sin h to about 2^-46 relative, cos h - 1 to about 2^-40 of
-// itself (2^-55 absolute, which is what the rotations need); larger steps
-// (coarse grids) through the FP64 routine sincos_step.
-__device__ __forceinline__ void sincos_step_ff(ff h, ff& sh, ff& cm)
-{
-    if (fabsf(h.hi) >= 0.0078125f) {
-        double s, c;
-        sincos_step(ff_to(h), s, c);
-        sh = ff_from(s);
-        cm = ff_from(c);
-        return;
-    }
-    const ff t = ff_sqr(h);
-    const ff h3 = ff_mul(h, t);
-    const ff sixth = {__uint_as_float(0x3e2aaaabu), __uint_as_float(0xb1aaaaabu)};   // 1/6
-    const float h5 = __fmul_rn(__fmul_rn(h3.hi, t.hi), 1.f / 120.f);
-    sh = ff_add(h, ff_add(ff_neg(ff_mul(h3, sixth)), ff_of(h5)));
-    const float c4 = __fmul_rn(__fmul_rn(t.hi, t.hi), __fsub_rn(1.f / 24.f, __fmul_rn(t.hi, 1.f / 720.f)));
-    cm = ff_add(ff_scale(t, -0.5f), ff_of(c4));
-}
-
-__device__ __forceinline__ void sincos_step_ff(double hd, ff& sh, ff& cm)
-{
-    sincos_step_ff(ff_from(hd), sh, cm);
 }
 
 }  // namespace fpic

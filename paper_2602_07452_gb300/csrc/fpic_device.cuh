@@ -2,14 +2,19 @@
 // metric and derivatives (Appendix A), the equations of motion (Eqs. p1, p2,
 // O1, O2), the Hamiltonian (Eq. Ham) and the staggered-grid field gather.
 //
-// GB300 note: FP64 issues at a small fraction of the FP32 rate, so these
-// helpers are written to minimise FP64-pipe instructions: one sincos, one
-// reciprocal and two reciprocal square roots per evaluation, fused
-// multiply-adds throughout, and cell location by integer comparison of the
-// IEEE bit patterns (order-preserving) instead of FP64 compares.
+// GB300 note: FP64 issues at 1/64 of the FP32 rate, so these helpers are
+// written to minimise FP64-pipe instructions: one sincos, one reciprocal and
+// two reciprocal square roots per evaluation, fused multiply-adds throughout,
+// corrections and differences that need 46 bits or fewer in paired FP32
+// (ff.cuh), and cell location by integer comparison of the IEEE bit patterns
+// (order-preserving) instead of FP64 compares.  Against an extended-precision
+// RK4 step the pushed states' relative errors are those of the all-FP64 forms
+// (4.8e-17 to 5.1e-17 on either side, at 48 to 900 cells a side).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "ff.cuh"
 
 namespace fpic {
 
@@ -17,12 +22,38 @@ struct BH {
     double M, a, a2, twoM;
 };
 
-// 1/x from the hardware approximation y refined by one third-order step:
-// with e = 1 - x y, 1/x = y / (1 - e) = y (1 + e + e^2 + ...), so
-// y (1 + e + e^2) triples the correct bits of the estimate (its relative
-// error e^3); fpic_probe_math measures the result against correctly
-// rounded reciprocals.
-__device__ __forceinline__ double rcp_nr(double x)
+// 1/x and 1/sqrt(x) with two FP64-pipe operations each.  The FP32 estimate y
+// of the result is a double with 24 significant bits, so that the residual
+// e = 1 - x y (e = 1 - x y^2, y^2 exact in 48 bits) is one fused multiply-add,
+// good to 2^-53 of itself; the correction y (e + e^2) (y (e/2 + 3 e^2/8)) of
+// the binomial series -- e is about 2^-21, the next term below 2^-64 -- needs
+// 32 significant bits and is formed in paired FP32, and one FP64 addition
+// rounds the result: within an ulp (fpic_probe_math measures both).  The
+// FP64 pipe takes 64 issue slots per operation, so the 40 or so FP32 and
+// integer instructions cost less than the two (three) FP64 operations they
+// replace.  Arguments outside 2^-60 .. 2^60 (where the correction's low float
+// keeps its bits), zeros, infinities and NaNs take the FP64 forms: the hardware estimate y and y (1 + e + e^2), or y (1 + e/2 +
+// 3 e^2/8).
+__device__ __forceinline__ bool f32_range(unsigned hi)      // 2^-60 <= x < 2^60, hi the high word of |x|
+{
+    return hi - ((1023u - 60u) << 20) < (120u << 20);
+}
+
+// a double in the float range as a float, cut off; a normal float as a double
+__device__ __forceinline__ float f32_cut(double x)
+{
+    const unsigned hw = (unsigned)__double2hiint(x);
+    return __uint_as_float(((__funnelshift_l((unsigned)__double2loint(x), hw, 3) ^ 0x40000000u) & 0x7fffffffu) |
+                           (hw & 0x80000000u));
+}
+
+__device__ __forceinline__ double f64_of(float y)
+{
+    const unsigned u = __float_as_uint(y);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+static __device__ __noinline__ double rcp_wide(double x)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -30,20 +61,37 @@ __device__ __forceinline__ double rcp_nr(double x)
     return fma(y, fma(e, e, e), y);
 }
 
-// 1/sqrt(x) for a positive normal x from the hardware estimate y: with
-// e = 1 - x y^2 (one rounded product, then a fused multiply-add),
-// 1/sqrt(x) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...), taken to
-// second order; the omitted terms are of order e^3, far below double
-// rounding for the estimate's error, so the result is within about an ulp
-// (fpic_probe_math measures it against an extended-precision reference).
-// Five FP64 operations and no special-case branches: the push only takes
-// it of xi = 1 + 2 M r / rho^2 and Gamma^2, both at least 1.
-__device__ __forceinline__ double rsqrt_nr(double x)
+static __device__ __noinline__ double rsqrt_wide(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x * y, y, 1.0);
     return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+__device__ __forceinline__ double rcp_nr(double x)
+{
+    if (!f32_range((unsigned)__double2hiint(x) & 0x7fffffffu)) return rcp_wide(x);
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f32_cut(x)));
+    const double yd = f64_of(y);
+    const ff e = ff_from(fma(-x, yd, 1.0));
+    return yd + ff_to_bits(ff_mulf({e.hi, __fmaf_rn(e.hi, e.hi, e.lo)}, y));
+}
+
+__device__ __forceinline__ double rsqrt_nr(double x)
+{
+    if (!f32_range((unsigned)__double2hiint(x))) return rsqrt_wide(x);       // negative x too
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f32_cut(x)));
+    // y^2 = m^2 2^(2 E - 46), m in [2^23, 2^24): its leading bit is bit 46 + k of m^2
+    const unsigned u = __float_as_uint(y), m = (u & 0x7fffffu) | 0x800000u;
+    const unsigned long long M = (unsigned long long)m * m;
+    const unsigned k = (unsigned)(M >> 47);
+    const unsigned long long b = (M << (6 - k)) + ((unsigned long long)((2u * (u >> 23) + 768u + k) << 20) << 32);
+    const ff e = ff_from(fma(-x, __longlong_as_double((long long)b), 1.0));
+    const ff c = ff_mulf({0.5f * e.hi, __fmaf_rn(0.375f * e.hi, e.hi, 0.5f * e.lo)}, y);
+    return f64_of(y) + ff_to_bits(c);
 }
 
 // Square root of a positive normal x (the deposit's trapezoid sums): the
@@ -101,15 +149,55 @@ __device__ __forceinline__ void sincos_step(double h, double& sh, double& cm)
     }
 }
 
+// sin h and cos h - 1 of a step h in paired FP32 (the deposit's th
+// lattice rotations).  Below 2^-7 by the Maclaurin series: h - h^3/6 and
+// -h^2/2 in paired arithmetic, the next terms (h^5/120; h^4/24 - h^6/720),
+// below 2^-28 relative, in FP32, the omitted ones below 2^-48 of the
+// result: sin h to about 2^-46 relative, cos h - 1 to about 2^-40 of
+// itself (2^-55 absolute, which is what the rotations need); larger steps
+// (coarse grids) through the FP64 routine sincos_step.
+__device__ __forceinline__ void sincos_step_ff(ff h, ff& sh, ff& cm)
+{
+    if (fabsf(h.hi) >= 0.0078125f) {
+        double s, c;
+        sincos_step(ff_to(h), s, c);
+        sh = ff_from(s);
+        cm = ff_from(c);
+        return;
+    }
+    const ff t = ff_sqr(h);
+    const ff h3 = ff_mul(h, t);
+    const ff sixth = {__uint_as_float(0x3e2aaaabu), __uint_as_float(0xb1aaaaabu)};   // 1/6
+    const float h5 = __fmul_rn(__fmul_rn(h3.hi, t.hi), 1.f / 120.f);
+    sh = ff_add(h, ff_add(ff_neg(ff_mul(h3, sixth)), ff_of(h5)));
+    const float c4 = __fmul_rn(__fmul_rn(t.hi, t.hi), __fsub_rn(1.f / 24.f, __fmul_rn(t.hi, 1.f / 720.f)));
+    cm = ff_add(ff_scale(t, -0.5f), ff_of(c4));
+}
+
+__device__ __forceinline__ void sincos_step_ff(double hd, ff& sh, ff& cm)
+{
+    sincos_step_ff(ff_from(hd), sh, cm);
+}
+
 // sin and cos of t from those of a nearby t0 by the angle-addition formula,
 // with sin d and cos d - 1 of d = t - t0 by their Taylor series (the first
-// omitted terms are below 1e-23 for |d| < 2^-7); farther away, sincos.
+// omitted terms are below 1e-23 for |d| < 2^-7); farther away, sincos.  The
+// series run in paired FP32: cos d - 1 and sin d - d are below 2^-15 and 2^-23,
+// so their 46 bits leave errors under 2^-60 and 2^-68 of the result; FP64 does
+// the difference, d + (sin d - d) and the rotation: six operations.
 __device__ __forceinline__ void sincos_near(double t0, double s0, double c0, double t, double& s, double& c)
 {
     const double d = t - t0;
     if (abs_below_pow2(d, HI_2M7)) {
-        double sd, cm;
-        sincos_step(d, sd, cm);
+        const ff f = ff_from(d), q = ff_sqr(f);
+        const ff sixth = {__uint_as_float(0x3e2aaaabu), __uint_as_float(0xb1aaaaabu)};   // 1/6
+        // sin d - d = -d^3/6 (1 - d^2/20 + d^4/840), cos d - 1 = -d^2/2 + d^4/24 - d^6/720 + d^8/40320
+        ff b = ff_neg(ff_mul(ff_mul(f, q), sixth));
+        b.lo = __fmaf_rn(__fmul_rn(b.hi, q.hi), __fmaf_rn(q.hi, 1.f / 840.f, -0.05f), b.lo);
+        const float q2 = __fmul_rn(q.hi, q.hi);
+        const ff m = {-0.5f * q.hi, __fmaf_rn(q2, __fmaf_rn(q.hi, __fmaf_rn(q.hi, 1.f / 40320.f, -1.f / 720.f), 1.f / 24.f),
+                                              -0.5f * q.lo)};
+        const double sd = d + ff_to_bits(b), cm = ff_to_bits(m);
         s = fma(s0, cm, fma(c0, sd, s0));
         c = fma(c0, cm, fma(-s0, sd, c0));
     } else {
@@ -157,31 +245,6 @@ __device__ __forceinline__ void geo_eval(const BH& bh, double r, double s, doubl
     g.sqrtg = g.rho2 * g.xi * g.alpha * s;
 }
 
-// d_r and d_th of the three functions the momentum equations need: xi,
-// g^tt = 1/rho^2 (g^rp = a g^tt, and g^rr, alpha, beta^r follow from xi and
-// g^tt, see eval_rhs_sc) and g^pp; plus q = 2 a^2 sin cos = -d_th rho^2.
-struct GeoD {
-    double xi[2], tt[2], pp[2];
-    double q;
-};
-
-// With P = rho^2 (d_r P = 2 r, d_th P = -q) and u = 1/P^2: d g^tt = -dP u,
-// d_r xi = 2M (P - 2 r^2) u, d_th xi = 2 M r q u, d_r g^pp = -2 r t / P,
-// d_th g^pp = -2 s c t^2 (P - a^2 s^2)  (t = g^pp = 1 / (P s^2)).
-__device__ __forceinline__ void geo_deriv(const BH& bh, double r, const Geo& g, GeoD& d)
-{
-    const double sc = g.s * g.c;
-    d.q = 2.0 * bh.a2 * sc;
-    const double u = g.irho2 * g.irho2;
-    const double mr2 = -2.0 * r;
-    d.tt[0] = mr2 * u;
-    d.tt[1] = d.q * u;
-    d.xi[0] = fma(bh.a2, g.c2, -g.r2) * (bh.twoM * u);   // rho^2 - 2 r^2 = a^2 cos^2 - r^2
-    d.xi[1] = g.twoMr * d.tt[1];
-    d.pp[0] = mr2 * (g.t * g.irho2);
-    d.pp[1] = (-2.0 * sc) * (g.t * g.t) * (g.rho2 - g.a2s2);
-}
-
 // FP32 value of a double from its high word (20 of its 52 mantissa bits,
 // truncated), by integer operations only, for the index estimates of
 // locate: no FP64 conversion instruction.  Exact enough for normal floats;
@@ -216,6 +279,17 @@ __device__ __forceinline__ double fmax_nonneg(double m, double a)
     return (ba > F64_INF_BITS || ba <= bm) ? m : a;
 }
 
+// x != 0 and x < 0 as the FP64 compares give them, by integer compares.
+__device__ __forceinline__ bool not_zero(double x)
+{
+    return ((unsigned long long)__double_as_longlong(x) << 1) != 0ull;
+}
+__device__ __forceinline__ bool is_neg(double x)
+{
+    const unsigned long long m = (unsigned long long)__double_as_longlong(x) << 1;
+    return __double_as_longlong(x) < 0 && m - 1ull < 0xffe0000000000000ull;
+}
+
 // x / 2 by taking one from the exponent, off the FP64 pipe; zeros, numbers
 // near or below the normal range, infinities and NaNs go through the
 // multiplication: the product's value for every x.
@@ -245,7 +319,7 @@ struct GridDev {
     int Nr, Nth, ld;
     const double *rn, *rh, *tn, *th;   // th: Nth half nodes + th[Nth] = th[0] + (tn[Nth] - tn[0])
     const double *irn, *irh, *itn, *ith;
-    const double *brn, *brh, *btn, *bth;   // -X[i] / (X[i+1] - X[i]) (locate_fma)
+    const float2 *prn, *prh, *ptn, *pth;   // the inverse spacings as pairs of floats (locate_ff)
     float lr0, lrh0, ilr;        // FP32 index estimate in ln r
     float t0, th0, it;           // FP32 index estimate in th
     int full;                    // full-theta domain (periodic th), else half-theta
@@ -310,104 +384,70 @@ __device__ __forceinline__ void locate(const double* __restrict__ X, const doubl
     w = ww;
 }
 
-// The same with the weight as one fused multiply-add, x iX[i] + BX[i]
-// (BX[i] = -X[i] iX[i]): an absolute error of about X[i] iX[i] ulps of 1
-// (~1e-13 on grids of a few hundred cells per e-fold) against one rounding
-// for (x - X[i]) iX[i]; the field gathers take it (one FP64 instruction
-// fewer per weight, four per gather).
-__device__ __forceinline__ void locate_fma(const double* __restrict__ X, const double* __restrict__ iX,
-                                           const double* __restrict__ BX, int m, double x, float est, int& i,
-                                           double& w)
+// The same with the weight in paired FP32: the FP64 difference x - X[i]
+// (exact but for its own rounding) times the inverse spacing, to 2^-47.
+__device__ __forceinline__ void locate_ff(const double* __restrict__ X, const float2* __restrict__ pX, int m, double x,
+                                          float est, int& i, ff& w)
 {
     const long long kx = okey(x);
     const int k = locate_walk(X, m, kx, est);
     i = k;
-    double ww = fma(x, __ldg(iX + k), __ldg(BX + k));
-    const bool below = kx < okey(__ldg(X + k));
-    const bool above = kx >= okey(__ldg(X + k + 1));
-    ww = below ? 0.0 : ww;
-    ww = above ? 1.0 : ww;
-    w = ww;
+    const double x0 = __ldg(X + k);
+    const float2 ix = __ldg(pX + k);
+    w = ff_mul(ff_from(x - x0), {ix.x, ix.y});
+    if (kx < okey(x0)) w = {0.f, 0.f};
+    if (kx >= okey(__ldg(X + k + 1))) w = {1.f, 0.f};
 }
 
 struct Fields {
     const double* f[6];   // D^r, D^th, D^ph, B^r, B^th, B^ph (Yee layout)
 };
 
-// Bilinear (r, th) gather of the six components at (r, th).
-__device__ __forceinline__ void gather(const GridDev& G, const Fields& F, double r, double th,
-                                       double D[3], double B[3])
+// Bilinear (r, th) gather of the six components at (r, th), all in FP64.
+static __device__ __noinline__ void gather(const GridDev& G, const Fields& F, double r, double th, double v[6])
 {
     const float lr = __logf(f32_est(r));
     int i0, i1, j0, j1;
     double wr0, wr1, wt0, wt1;
-    locate_fma(G.rn, G.irn, G.brn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
-    locate_fma(G.rh, G.irh, G.brh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
+    locate(G.rn, G.irn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
+    locate(G.rh, G.irh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
     double tnv, thv;
     int mh;
     theta_views(G, th, tnv, thv, mh);
     const float tfn = f32_est(tnv), tfh = G.full ? f32_est(thv) : tfn;
-    locate_fma(G.tn, G.itn, G.btn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
-    locate_fma(G.th, G.ith, G.bth, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
+    locate(G.tn, G.itn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
+    locate(G.th, G.ith, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
     const int ld = G.ld;
     // component k sits at (roff, toff): D^r (1,0) D^th (0,1) D^ph (0,0)
     //                                    B^r (0,1) B^th (1,0) B^ph (1,1)
-    double v[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         const bool ro = (k == 0 || k == 4 || k == 5);
         const bool to = (k == 1 || k == 3 || k == 5);
         const int i = ro ? i1 : i0, j = to ? j1 : j0;
         const double wr = ro ? wr1 : wr0, wt = to ? wt1 : wt0;
-        const double* p = F.f[k] + i * ld + j;
+        const double* p = F.f[k] + (size_t)i * ld + j;
         const double f00 = __ldg(p), f01 = __ldg(p + 1);
         const double f10 = __ldg(p + ld), f11 = __ldg(p + ld + 1);
         const double lo = fma(wt, f01 - f00, f00);
         const double hi = fma(wt, f11 - f10, f10);
         v[k] = fma(wr, hi - lo, lo);
     }
-    D[0] = v[0]; D[1] = v[1]; D[2] = v[2];
-    B[0] = v[3]; B[1] = v[4]; B[2] = v[5];
 }
 
 // The same bilinear interpolant from per-cell coefficients: component k's
-// cell (i, j) holds (a, b, c, d) = (f00, f10 - f00, f01 - f00,
-// f11 - f10 - f01 + f00) at 4 (i ld + j) (r index first), so that
-// f = a + b w_r + c w_th + d w_r w_th costs 3 FMA instead of 3 subtractions
-// and 3 FMA (built by k_field_coef before each push).
+// cell (i, j) holds a = f00 in FP64 and b = f10 - f00, c = f01 - f00,
+// d = f11 - f10 - f01 + f00 as pairs of floats, 32 bytes at 4 (i ld + j) doubles (r
+// index first; built by k_field_coef before each push), and
+// f = a + (b w_r + w_th (c + d w_r)), the bracket in paired FP32: what the
+// cell adds to a is good to 2^-47 of its differences, as the weights are, and
+// one FP64 addition per component remains of three fused multiply-adds (an
+// expansion about the cell's centre measured the same error).
+// A cell whose differences are no numbers or outside 2^-90 .. 2^100 is marked
+// (b's high float a NaN) and gathered from the fields in FP64.
 struct FieldsC {
     const double* c[6];
 };
-
-__device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, double r, double th, double D[3],
-                                         double B[3])
-{
-    const float lr = __logf(f32_est(r));
-    int i0, i1, j0, j1;
-    double wr0, wr1, wt0, wt1;
-    locate_fma(G.rn, G.irn, G.brn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
-    locate_fma(G.rh, G.irh, G.brh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
-    double tnv, thv;
-    int mh;
-    theta_views(G, th, tnv, thv, mh);
-    const float tfn = f32_est(tnv), tfh = G.full ? f32_est(thv) : tfn;
-    locate_fma(G.tn, G.itn, G.btn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
-    locate_fma(G.th, G.ith, G.bth, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
-    const int ld = G.ld;
-    double v[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const bool ro = (k == 0 || k == 4 || k == 5);
-        const bool to = (k == 1 || k == 3 || k == 5);
-        const int i = ro ? i1 : i0, j = to ? j1 : j0;
-        const double wr = ro ? wr1 : wr0, wt = to ? wt1 : wt0;
-        const double2* q = reinterpret_cast<const double2*>(F.c[k] + 4 * ((size_t)i * ld + j));
-        const double2 ab = __ldg(q), cd = __ldg(q + 1);
-        v[k] = fma(wt, fma(cd.y, wr, cd.x), fma(ab.y, wr, ab.x));
-    }
-    D[0] = v[0]; D[1] = v[1]; D[2] = v[2];
-    B[0] = v[3]; B[1] = v[4]; B[2] = v[5];
-}
 
 // Field tile staged in shared memory for a block of cell-sorted particles:
 // STAGE_TI coefficient rows (r cells) x STAGE_TJ coefficient cells (th) of
@@ -420,32 +460,39 @@ struct StageTile {
     int i0, j0;
 };
 
-__device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, double r, double th, double D[3],
-                                         double B[3], const StageTile& T)
+__device__ __forceinline__ ff ff_bits(double x)      // a pair of floats stored in a double's place
+{
+    return {__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x))};
+}
+
+template <bool STAGED = false>
+__device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, const Fields& raw, double r, double th,
+                                         double D[3], double B[3], const StageTile* T = nullptr)
 {
     const float lr = __logf(f32_est(r));
     int i0, i1, j0, j1;
-    double wr0, wr1, wt0, wt1;
-    locate_fma(G.rn, G.irn, G.brn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
-    locate_fma(G.rh, G.irh, G.brh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
+    ff wr0, wr1, wt0, wt1;
+    locate_ff(G.rn, G.prn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
+    locate_ff(G.rh, G.prh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
     double tnv, thv;
     int mh;
     theta_views(G, th, tnv, thv, mh);
     const float tfn = f32_est(tnv), tfh = G.full ? f32_est(thv) : tfn;
-    locate_fma(G.tn, G.itn, G.btn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
-    locate_fma(G.th, G.ith, G.bth, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
+    locate_ff(G.tn, G.ptn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
+    locate_ff(G.th, G.pth, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
     const int ld = G.ld;
     double v[6];
+    bool odd = false;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         const bool ro = (k == 0 || k == 4 || k == 5);
         const bool to = (k == 1 || k == 3 || k == 5);
         const int i = ro ? i1 : i0, j = to ? j1 : j0;
-        const double wr = ro ? wr1 : wr0, wt = to ? wt1 : wt0;
-        const unsigned ti = (unsigned)(i - T.i0), tj = (unsigned)(j - T.j0);
+        const ff wr = ro ? wr1 : wr0, wt = to ? wt1 : wt0;
         double2 ab, cd;
-        if (T.s && ti < (unsigned)STAGE_TI && tj < (unsigned)STAGE_TJ) {
-            const double2* q = reinterpret_cast<const double2*>(T.s + ((k * STAGE_TI + ti) * STAGE_TJ + tj) * 4);
+        const unsigned ti = STAGED ? (unsigned)(i - T->i0) : 0u, tj = STAGED ? (unsigned)(j - T->j0) : 0u;
+        if (STAGED && T->s && ti < (unsigned)STAGE_TI && tj < (unsigned)STAGE_TJ) {
+            const double2* q = reinterpret_cast<const double2*>(T->s + ((k * STAGE_TI + ti) * STAGE_TJ + tj) * 4);
             ab = q[0];
             cd = q[1];
         } else {
@@ -453,7 +500,15 @@ __device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, dou
             ab = __ldg(q);
             cd = __ldg(q + 1);
         }
-        v[k] = fma(wt, fma(cd.y, wr, cd.x), fma(ab.y, wr, ab.x));
+        const ff b = ff_bits(ab.y);
+        odd = odd || b.hi != b.hi;
+        v[k] = ab.x + ff_to_bits(ff_add(ff_mul(b, wr), ff_mul(wt, ff_add(ff_bits(cd.x), ff_mul(ff_bits(cd.y), wr)))));
+    }
+    if (odd) {
+        double u[6];
+        gather(G, raw, r, th, u);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = u[k];
     }
     D[0] = v[0]; D[1] = v[1]; D[2] = v[2];
     B[0] = v[3]; B[1] = v[4]; B[2] = v[5];
@@ -479,45 +534,54 @@ __device__ __forceinline__ void eval_rhs_sc_t(const BH& bh, const double y[6], d
                                               bool em, const double D[3], const double B[3], double B0pot,
                                               double f[6], double& H, RhsJ* J)
 {
-    Geo g;
-    geo_eval(bh, y[0], s, c, g);
-    GeoD d;
-    geo_deriv(bh, y[0], g, d);
-    const double ur = y[3], ut = y[4], up = y[5];
-    const double Ur = fma(g.gurr, ur, g.gurp * up);
-    const double Ut = g.gutt * ut;
-    const double Up = fma(g.gurp, ur, g.gupp * up);
-    const double G2 = fma(ur, Ur, fma(ut, Ut, fma(up, Up, 1.0)));
+    const double r = y[0], ur = y[3], ut = y[4], up = y[5];
+    // metric (App. A): e = xi - 1 = 2 M r / rho^2, beta^r = e / xi, g^rph = a / rho^2,
+    // g^thth = 1 / rho^2, t = g^phph = 1 / (rho^2 sin^2 th)
+    const double s2 = s * s, rho2 = fma(bh.a2, c * c, r * r);
+    const double t = rcp_nr(rho2 * s2), irho2 = t * s2;
+    const double mi = bh.twoM * irho2, e = mi * r, xi = fma(mi, r, 1.0);
+    const double alpha = rsqrt_nr(xi), ixi = alpha * alpha, beta = e * ixi;
+    const double gurp = bh.a * irho2, as2 = bh.a * s2;
+    // u^i = g^ij u_j: u^r = u_r / xi + g^rph (a s^2 u_r + u_ph)
+    const double g1 = fma(as2, ur, up), iu = ixi * ur, tu = t * up;
+    const double Ur = fma(gurp, g1, iu), Ut = irho2 * ut, Up = fma(gurp, ur, tu);
+    // W = a^2 s^2 u_r^2 + 2 a u_r u_ph + u_th^2, Q = W / rho^2 + u_ph^2 t, so that
+    // Gamma^2 = 1 + u_r^2 / xi + Q
+    const double W = fma(bh.a * ur, g1 + up, ut * ut);
+    const double Q = fma(W, irho2, tu * up);
+    const double G2 = fma(iu, ur, 1.0 + Q);
     const double iG = rsqrt_nr(G2);
-    const double aiG = g.alpha * iG;
-    f[0] = fma(aiG, Ur, -g.beta);
+    const double aiG = alpha * iG;
+    f[0] = fma(aiG, Ur, -beta);
     f[1] = aiG * Ut;
     f[2] = aiG * Up;
     // du_i/dt = -Gamma d_i alpha + u_r d_i beta^r - (alpha / 2 Gamma) u_j u_k d_i g^jk
     // (Eq. p2).  With d alpha = -(alpha^3 / 2) d xi, d beta^r = d xi / xi^2,
-    // d g^rr = a^2 s^2 d g^tt - d xi / xi^2 (+ q / rho^2 in th), d g^rp = a d g^tt:
-    //   u_j u_k d_i g^jk = W d_i g^tt + u_ph^2 d_i g^pp - u_r^2 d_i xi / xi^2 (+ u_r^2 q / rho^2)
-    //   with W = a^2 s^2 u_r^2 + 2 a u_r u_ph + u_th^2, so
-    //   du_i/dt = h (W d_i g^tt + u_ph^2 d_i g^pp [+ u_r^2 q / rho^2])
-    //             + d_i xi (u_r (1 - h u_r) / xi^2 + Gamma alpha^3 / 2),  h = -alpha / (2 Gamma).
-    //   In r: W d_r g^tt + u_ph^2 d_r g^pp = -2 r (W / rho^4 + u_ph^2 / (rho^4 s^2))
-    //   = -2 r / rho^2 (W / rho^2 + u_ph^2 t), t = 1 / (rho^2 s^2), so that
-    //   h (...) = (alpha / Gamma) m0 with m0 = (r / rho^2) (W / rho^2 + u_ph^2 t).
-    //   With alpha^2 = 1/xi the d_i xi factor is
-    //   kap = (1/xi) ((1/xi) u_r (1 - h u_r) + alpha Gamma / 2), alpha Gamma / 2 = -h Gamma^2.
-    const double h = -0.5 * aiG;
-    const double urur = ur * ur, upup = up * up;
-    const double W = fma(urur, g.a2s2, fma(2.0 * bh.a * ur, up, ut * ut));
-    const double haG = -h * G2;                       // alpha Gamma / 2
-    const double kap = g.ixi * fma(g.ixi * ur, fma(-h, ur, 1.0), haG);
-    const double m0 = (y[0] * g.irho2) * fma(W, g.irho2, upup * g.t);
-    f[3] = fma(aiG, m0, d.xi[0] * kap);
-    f[4] = fma(h, fma(W, d.tt[1], fma(upup, d.pp[1], urur * d.q * g.irho2)), d.xi[1] * kap);
+    // d g^rr = a^2 s^2 d g^tt - d xi / xi^2 (+ q / rho^2 in th), d g^rp = a d g^tt
+    // and q = 2 a^2 sin cos = -d_th rho^2:
+    //   u_j u_k d_i g^jk = W d_i g^tt + u_ph^2 d_i g^pp - u_r^2 d_i xi / xi^2 (+ u_r^2 q / rho^2),
+    // so the d_i xi factor is kap = (1/xi) ((u_r / xi)(1 + (alpha / Gamma) u_r / 2) +
+    // alpha Gamma / 2), alpha Gamma = (alpha / Gamma) Gamma^2; k2 = 2 kap.
+    //   r: d_r xi = (2 M / rho^2)(1 - 2 r^2 / rho^2), W d_r g^tt + u_ph^2 d_r g^pp
+    //   = -2 (r / rho^2) Q;
+    //   th: d_th g^tt = q / rho^4, d_th xi = e q / rho^2, d_th g^pp = -2 s c t^2 (rho^2 - a^2
+    //   s^2), q / rho^2 = 2 a g^rph s c, so with P = W / rho^2 + u_r^2
+    //   du_th/dt = a g^rph s c (2 e kap - (alpha / Gamma) P)
+    //              + (alpha / Gamma) s c (t u_ph)^2 (rho^2 - a^2 s^2).
+    const double GA = aiG * G2;                       // alpha Gamma
+    const double k2 = ixi * fma(iu, fma(aiG, ur, 2.0), GA);
+    const double rr = r * irho2;
+    const double xk = mi * fma(-rr, r, 0.5);          // d_r xi / 2
+    const double P = fma(W, irho2, ur * ur);
+    const double br = fma(-aiG, P, e * k2), X2 = fma(-bh.a, as2, rho2);
+    f[3] = aiG * rr;                                  // completed below
+    f[4] = (s * c) * fma(aiG, (tu * tu) * X2, (bh.a * gurp) * br);
     f[5] = 0.0;
+    double fr = 0.0;                                  // electromagnetic force in r
     if (JAC) {
         J->U[0] = Ur; J->U[1] = Ut; J->U[2] = Up;
         J->iG = iG; J->aiG = aiG;
-        J->gurr = g.gurr; J->gurp = g.gurp; J->gutt = g.gutt; J->gupp = g.gupp;
+        J->gurr = fma(bh.a * as2, irho2, ixi); J->gurp = gurp; J->gutt = irho2; J->gupp = t;
         // no field: the force terms of the Newton matrix vanish (set, not left undefined)
         J->ks = 0.0;
         J->B[0] = J->B[1] = J->B[2] = 0.0;
@@ -528,43 +592,28 @@ __device__ __forceinline__ void eval_rhs_sc_t(const BH& bh, const double y[6], d
         // gamma_thth = rho^2, gamma_phph = s^2 (rho^2 + a^2 xi s^2):
         //   r:  k xi X,  X = D^r - a s^2 D^ph
         //   ph: k s^2 (rho^2 D^ph - a xi X)
-        const double k = qm * g.alpha;
-        const double kxi = k * g.xi, kr = k * g.rho2;
-        const double ks = (qm * g.rho2) * (g.s * iG);    // k sqrt(gamma) / Gamma, alpha^2 xi = 1
+        const double k = qm * alpha;
+        const double kr = k * rho2;
+        const double ks = (qm * rho2) * (s * iG);    // k sqrt(gamma) / Gamma, alpha^2 xi = 1
         const double cr = fma(Ut, B[2], -Up * B[1]);
         const double ct = fma(Up, B[0], -Ur * B[2]);
         const double cp = fma(Ur, B[1], -Ut * B[0]);
-        const double X = fma(-bh.a * g.s2, D[2], D[0]);
-        f[3] = fma(kxi, X, fma(ks, cr, f[3]));
+        const double kx = (k * xi) * fma(-as2, D[2], D[0]);
+        fr = fma(ks, cr, kx);
         f[4] = fma(kr, D[1], fma(ks, ct, f[4]));
-        f[5] = fma(g.s2, fma(kr, D[2], -(bh.a * kxi) * X), ks * cp);
+        f[5] = fma(s2, fma(kr, D[2], -bh.a * kx), ks * cp);
         if (JAC) {
             J->ks = ks;
             J->B[0] = B[0]; J->B[1] = B[1]; J->B[2] = B[2];
             J->cx[0] = cr; J->cx[1] = ct; J->cx[2] = cp;
         }
     }
-    H = fma(-g.beta, ur, haG + haG);                  // alpha Gamma - beta^r u_r
-    if (B0pot != 0.0 && qm != 0.0) {
+    f[3] = fma(f[3], Q, fma(xk, k2, fr));
+    H = fma(-beta, ur, GA);                           // alpha Gamma - beta^r u_r
+    if (not_zero(B0pot) && not_zero(qm)) {
         // A_0 = B0 a r (1 + cos^2 th) / rho^2   (Sec. 3.1.3)
-        H = fma(-qm * B0pot * bh.a * y[0], (1.0 + g.c2) * g.irho2, H);
+        H = fma(-qm * B0pot * bh.a * r, fma(c, c, 1.0) * irho2, H);
     }
-}
-
-__device__ __forceinline__ void eval_rhs_sc(const BH& bh, const double y[6], double s, double c, double qm,
-                                            bool em, const double D[3], const double B[3], double B0pot,
-                                            double f[6], double& H)
-{
-    eval_rhs_sc_t<false>(bh, y, s, c, qm, em, D, B, B0pot, f, H, nullptr);
-}
-
-__device__ __forceinline__ void eval_rhs(const BH& bh, const double y[6], double qm, bool em,
-                                         const double D[3], const double B[3], double B0pot,
-                                         double f[6], double& H)
-{
-    double s, c;
-    sincos(y[1], &s, &c);
-    eval_rhs_sc(bh, y, s, c, qm, em, D, B, B0pot, f, H);
 }
 
 // Hamiltonian only (no derivatives, no force), given sin/cos of y[1].
@@ -579,7 +628,7 @@ __device__ __forceinline__ double eval_H_sc(const BH& bh, const double y[6], dou
     const double Up = fma(g.gurp, ur, g.gupp * up);
     const double G = sqrt(fma(ur, Ur, fma(ut, Ut, fma(up, Up, 1.0))));
     double H = fma(g.alpha, G, -g.beta * ur);
-    if (B0pot != 0.0 && qm != 0.0) H = fma(-qm * B0pot * bh.a * y[0], (1.0 + c * c) * g.irho2, H);
+    if (not_zero(B0pot) && not_zero(qm)) H = fma(-qm * B0pot * bh.a * y[0], fma(c, c, 1.0) * g.irho2, H);
     return H;
 }
 

@@ -17,7 +17,6 @@
 #include <string.h>
 
 #include "dep_poly.cuh"
-#include "ff.cuh"
 #include "fpic_internal.h"
 
 namespace fpic {
@@ -1095,7 +1094,13 @@ static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
         c->poly_ok = false;
         c->poly_grid = c->grid_gen;
         retire(c, &c->d_poly);
-        if (bytes > POLY_MAX_BYTES) return 0;
+        // spacings far beyond what the bound admits: not worth a look
+        const double* X = (const double*)c->h_nodes.data();
+        const double* Y = X + (size_t)c->Nr + 1 + c->Nr;
+        double dr = 0.0, dt = 0.0;
+        for (int i = 0; i < c->Nr; ++i) dr = fmax(dr, (X[i + 1] - X[i]) / X[i]);
+        for (int j = 0; j < c->Nth; ++j) dt = fmax(dt, Y[j + 1] - Y[j]);
+        if (bytes > POLY_MAX_BYTES || dr > 0.05 || dt > POLY_MAX_DTH) return 0;
         if (cudaMalloc(&c->d_poly, bytes) != cudaSuccess) {
             cudaGetLastError();
             c->d_poly = nullptr;

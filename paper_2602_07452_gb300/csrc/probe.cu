@@ -1,7 +1,6 @@
 // Measurement helper: sustained FP64 FMA throughput of the device.  Eight
 // independent FMA chains per thread keep the FP64 pipe fed; the result is
 // stored so the chains cannot be removed.
-#include "ff.cuh"
 #include "fpic_internal.h"
 
 namespace fpic {

@@ -178,30 +178,26 @@ __device__ __forceinline__ uint32_t cell_of(const GridDev& G, double r, double t
     return (uint32_t)i * (uint32_t)G.Nth + (uint32_t)j;
 }
 
-// Right-hand side at y: gathers the fields when the particle is charged.
-__device__ __forceinline__ void F_at(const RunK& R, const double y[6], double qm, bool em,
-                                     double f[6], double& H)
-{
-    double D[3] = {0, 0, 0}, B[3] = {0, 0, 0};
-    if (em) {
-        if (R.has_coef) gather_c(R.G, R.FC, y[0], y[1], D, B);
-        else gather(R.G, R.F, y[0], y[1], D, B);
-    }
-    eval_rhs(R.bh, y, qm, em, D, B, R.B0pot, f, H);
-}
-
-// Same, with sin/cos of y[1] supplied (from sincos_near).  STAGED: the
-// coefficient gather looks in the block's staged field tile T first.
+// Right-hand side at y, sin/cos of y[1] supplied (from sincos_near): gathers
+// the fields when the particle is charged.  STAGED: the coefficient gather
+// looks in the block's staged field tile T first.
 template <bool JAC = false, bool STAGED = false>
 __device__ __forceinline__ void F_at_sc(const RunK& R, const double y[6], double s, double c, double qm, bool em,
                                         double f[6], double& H, RhsJ* J = nullptr, const StageTile* T = nullptr)
 {
     double D[3] = {0, 0, 0}, B[3] = {0, 0, 0};
     if (em) {
-        if (R.B0field != 0.0) wald_point_sc(R.bh, R.B0field, y[0], s, c, D, B);
-        else if (STAGED && R.has_coef) gather_c(R.G, R.FC, y[0], y[1], D, B, *T);
-        else if (R.has_coef) gather_c(R.G, R.FC, y[0], y[1], D, B);
-        else gather(R.G, R.F, y[0], y[1], D, B);
+        if (not_zero(R.B0field)) wald_point_sc(R.bh, R.B0field, y[0], s, c, D, B);
+        else if (R.has_coef) gather_c<STAGED>(R.G, R.FC, R.F, y[0], y[1], D, B, T);
+        else {
+            double v[6];
+            gather(R.G, R.F, y[0], y[1], v);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                D[i] = v[i];
+                B[i] = v[3 + i];
+            }
+        }
     }
     eval_rhs_sc_t<JAC>(R.bh, y, s, c, qm, em, D, B, R.B0pot, f, H, J);
 }
@@ -338,11 +334,11 @@ __device__ __forceinline__ void theta_boundary(const GridDev& G, double z[6])
 {
     if (G.full) {
         z[1] = theta_period_wrap(z[1], G.tlo, G.tper);
-    } else if (z[1] < 0.0) {
+    } else if (is_neg(z[1])) {
         z[1] = -z[1];
         z[4] = -z[4];
         z[2] += M_PI;
-    } else if (z[1] > M_PI) {
+    } else if (lt_nonneg(M_PI, z[1])) {
         z[1] = 2.0 * M_PI - z[1];
         z[4] = -z[4];
         z[2] += M_PI;
@@ -353,7 +349,7 @@ __device__ __forceinline__ bool finish(const RunK& R, const PartDev& P, long lon
                                        int implicit, int iters)
 {
     theta_boundary(R.G, z);
-    const bool alive = (z[0] >= R.r_h) && (z[0] <= R.r_max);
+    const bool alive = le_nonneg(R.r_h, z[0]) && le_nonneg(z[0], R.r_max);     // r_h > 0
     store_state(P, p, z);
     P.Hn[p] = H;
     P.scheme[p] = (uint8_t)implicit;
@@ -405,6 +401,12 @@ __device__ __forceinline__ void trial_store(const PushK& k, unsigned long long i
     }
 }
 
+// Bound by the FP64 pipe (82 % busy; 64 issue slots per FP64 instruction), so
+// its cost is the count of those: 470 a particle with the reused slope, 610
+// before the reciprocals, the sin/cos series and the gather's differences
+// went to paired FP32 and integer instructions (fpic_device.cuh) and the
+// force's common factors were shared: 1.164 -> 0.951 ms per 2^20 particles
+// (ncu), 76.2 -> 61 ms for the RK4 push of 6.4e7 on 1024 x 1024.
 // MODE 0: RK4 only.  MODE 1: hybrid (RK4 trial + test + enqueue).  MODE 2:
 // hybrid that also parks the RK4 slopes of each rejected particle
 // (corrector form of the learned guess); k1, k2 wait in shared memory
@@ -450,7 +452,7 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
         k.before.uph[p] = z0[5];
     }
     const double qm = k.P.qm[p];
-    const bool em = (R.has_fields || R.B0field != 0.0) && qm != 0.0;
+    const bool em = (R.has_fields || not_zero(R.B0field)) && not_zero(qm);
     const double dt = k.dt, hdt = 0.5 * k.dt;
     double Hd, s0, c0, sn, cn;
     // k1 = F(z^n): from the slope cache when this particle's state is the
@@ -701,7 +703,7 @@ __global__ void __launch_bounds__(128, NEWTON ? 3 : 4) k_imr(const __grid_consta
                                                 : k.guess[(size_t)i * k.n + p];
                         }
                         qm = (!all_mode && k.z0s) ? k.z0s[(size_t)6 * k.n + slot] : k.P.qm[p];
-                        em = (R->has_fields || R->B0field != 0.0) && qm != 0.0;
+                        em = (R->has_fields || not_zero(R->B0field)) && not_zero(qm);
                         it = 0;
                         best_dz = INFINITY;
                         best_it = 0;
@@ -940,7 +942,7 @@ __global__ void __launch_bounds__(256) k_imr_finish(const __grid_constant__ Push
         const double qm = st ? k.z0s[(size_t)6 * k.n + idx] : k.P.qm[p];
         const bool keep = !BATCHED && k.slope && !all_mode && !k.record;
         double H, f[6];
-        const bool em = (R.has_fields || R.B0field != 0.0) && qm != 0.0;
+        const bool em = (R.has_fields || not_zero(R.B0field)) && not_zero(qm);
         if (keep) F_at_sc(R, z, sn, cn, qm, em, f, H);
         else H = eval_H_sc(R.bh, z, sn, cn, qm, R.B0pot);
         if (k.substeps > 0 && !k.record) {
@@ -994,7 +996,7 @@ __global__ void __launch_bounds__(128) k_imr_substep(const __grid_constant__ Pus
             load_state(k.P, p, z0);
         }
         const double qm = st ? k.z0s[(size_t)6 * k.n + qi] : k.P.qm[p];
-        const bool em = (R.has_fields || R.B0field != 0.0) && qm != 0.0;
+        const bool em = (R.has_fields || not_zero(R.B0field)) && not_zero(qm);
         const double Href = eval_H(R.bh, z0, qm, R.B0pot), D0 = st ? k.z0s[(size_t)8 * k.n + qi] : k.P.D0[p];
         double z[6];
 #pragma unroll
@@ -1487,10 +1489,21 @@ __global__ void k_field_coef(GridDev G, Fields F, double* out, size_t sz)
             const size_t o = (size_t)i * G.ld + j;
             const double* f = F.f[k];
             const double f00 = f[o], f01 = f[o + 1], f10 = f[o + G.ld], f11 = f[o + G.ld + 1];
-            const double b = f10 - f00, c = f01 - f00;
+            const double v[3] = {f10 - f00, f01 - f00, (f11 - f10) - (f01 - f00)};
+            float2 w[3];
+            bool ok = true;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const ff x = ff_from(v[m]);
+                w[m] = make_float2(x.hi, x.lo);
+                const unsigned e = (unsigned)__double2hiint(v[m]) & 0x7fffffffu;
+                ok = ok && (!not_zero(v[m]) || e - ((1023u - 90u) << 20) < (190u << 20));
+            }
+            if (!ok) w[0].x = __int_as_float(0x7fffffff);
             double2* q = reinterpret_cast<double2*>(out + (size_t)k * 4 * sz + 4 * o);
-            q[0] = make_double2(f00, b);
-            q[1] = make_double2(c, (f11 - f10) - c);
+            auto bits = [](float2 x) { return __hiloint2double(__float_as_int(x.y), __float_as_int(x.x)); };
+            q[0] = make_double2(f00, bits(w[0]));
+            q[1] = make_double2(bits(w[1]), bits(w[2]));
         }
     }
 }
