@@ -25,14 +25,14 @@ namespace fpic {
 // Metric tables
 // ---------------------------------------------------------------------------
 // Points: 0 (i, j), 1 (i+1/2, j), 2 (i, j+1/2), 3 (i+1/2, j+1/2).  First what
-// cleaning and the deposits read: sqrt(gamma), lower metric components, 2 pi x
-// the dual-cell volumes; then the field update's coefficients (see the FDTD
+// cleaning and the deposits read: sqrt(gamma), g^rph, g^rr, g^thth, 2 pi x the
+// dual-cell volumes; then the field update's coefficients (see the FDTD
 // section), each product of metric factors, average weights and reciprocal
 // spacings formed once: 11 FP64 operations for E or H at a node instead of
 // 35, and no factor read that is not used as it is.  Then sin/cos of the
 // integer and half th nodes.
 enum {
-    T_SG0, T_SG1, T_SG2, T_RR0, T_RP0, T_PP0, T_RR1, T_RP1, T_PP1, T_TT2, T_DUAL0, T_DUAL1, T_DUAL2,
+    T_SG0, T_SG1, T_SG2, T_URP0, T_URR1, T_UTT2, T_DUAL0, T_DUAL1, T_DUAL2,
     // E_r = ER_D D^r + ER_P0 D^ph_i + ER_P1 D^ph_{i+1}; E_th, E_ph alike (0: row i - 1, 1: row i, held at the ends)
     F_ER_D, F_ER_P0, F_ER_P1, F_ET_D, F_ET_B0, F_ET_B1, F_EP_D, F_EP_R0, F_EP_R1, F_EP_T0, F_EP_T1,
     F_HR_B, F_HR_P0, F_HR_P1, F_HT_B, F_HT_D0, F_HT_D1, F_HP_B, F_HP_R0, F_HP_R1, F_HP_T0, F_HP_T1,
@@ -158,9 +158,7 @@ __global__ void __launch_bounds__(128) k_metric_tables(BH bh, GridDev G, double*
         {   // (i, j)
             const double is = 1.0 / g0.sqrtg, k = 0.5 * g0.alpha * g0.grp * is;
             put(T_SG0, g0.sqrtg);
-            put(T_RR0, g0.grr);
-            put(T_RP0, g0.grp);
-            put(T_PP0, g0.gpp);
+            put(T_URP0, g0.gurp);
             put(T_DUAL0, dual_sum(bh, x0, x1, ya1 - ya0, sa, Aa));
             put(F_EP_D, g0.alpha * g0.gpp);
             put(F_EP_R0, k * s1m);
@@ -174,7 +172,7 @@ __global__ void __launch_bounds__(128) k_metric_tables(BH bh, GridDev G, double*
         if (in) {   // (i, j+1/2)
             const double is = 1.0 / g2.sqrtg, k = 0.5 * g2.alpha * g2.grp * is;
             put(T_SG2, g2.sqrtg);
-            put(T_TT2, g2.gtt);
+            put(T_UTT2, g2.gutt);
             put(T_DUAL2, dual_sum(bh, x0, x1, yb1 - yb0, sb, Ab));
             put(F_ET_D, g2.alpha * g2.gtt);
             put(F_ET_B0, -0.5 * g2.beta * s3m);
@@ -189,9 +187,7 @@ __global__ void __launch_bounds__(128) k_metric_tables(BH bh, GridDev G, double*
         if (half) {   // (i+1/2, j)
             const double is = 1.0 / g1.sqrtg, k = 0.5 * g1.alpha * g1.grp * is;
             put(T_SG1, g1.sqrtg);
-            put(T_RR1, g1.grr);
-            put(T_RP1, g1.grp);
-            put(T_PP1, g1.gpp);
+            put(T_URR1, g1.gurr);
             put(T_DUAL1, dual_sum(bh, G.rn[i], G.rn[i + 1], ya1 - ya0, sa, Aa));
             put(F_ER_D, g1.alpha * g1.grr);
             put(F_ER_P0, k * g0.sqrtg);
@@ -522,9 +518,9 @@ struct Work {
 };
 
 static int work_layout(fpic_ctx* c, long long n, bool deposit, Work& w, size_t extra_bytes = 0,
-                       void** extra = nullptr)
+                       void** extra = nullptr, int buckets_per_cell = 1)
 {
-    const long long C = (long long)c->Nr * c->Nth;
+    const long long C = (long long)c->Nr * c->Nth * buckets_per_cell;
     const long long nbs = (n > C + 2 ? n : C + 2) / (SCAN_B * SCAN_PER) + 2;
     size_t bytes = 0;
     auto take = [&](size_t b) { size_t o = bytes; bytes += (b + 255) & ~(size_t)255; return o; };
@@ -1789,12 +1785,24 @@ namespace fpic {
 // and new), charge crossing the dual face between window nodes x and x+1 in
 // +r: -Q sum_{x' <= x} W_r(x', y) (alike in th).  Window partials (30 per
 // particle: Q S^new and Q <S> (dph/dt)_mid on 3 x 3 nodes, 2 x 3 r faces,
-// 3 x 2 th faces) are summed per window-base cell by one warp over the cell's
-// particles in index order (fixed shuffle tree), then gathered per node /
-// face in a fixed order: bitwise reproducible.  Normalised by the Yee cell
-// (2 pi sqrtg dr_dual dth_dual) so that sqrtg (rho^{n+1} - rho^n) + dt
-// Yee-div(sqrtg J) = 0 at every node.
+// 3 x 2 th faces) are summed per window-base cell in particle-index order,
+// then gathered per node / face in a fixed order: bitwise reproducible.
+// Normalised by the Yee cell (2 pi sqrtg dr_dual dth_dual) so that sqrtg
+// (rho^{n+1} - rho^n) + dt Yee-div(sqrtg J) = 0 at every node.
+//
+// A move inside one cell (all but a few per cent at a PIC step) has only 12
+// partials that are not zero, products of the two positions' cell fractions;
+// it is keyed to its cell, a move across a boundary to a second set of
+// buckets, so that k_cdep_particle works through each kind densely, one
+// thread per particle, and k_cdep_cell adds the records up.  FP64-pipe
+// bound: with one warp per cell, its 30 partials by every lane and a
+// reduction tree, a cell of 16 particles left half the lanes idle:
+// 4.0e6 particles on 512 x 512 3604 us, now 842 (particles, 86 % of the pipe,
+// 113 FP64 operations each) + 188 (cells).
 enum { CD_Q = 0, CD_P = 9, CD_R = 18, CD_T = 24, CD_SLOTS = 30 };
+// rows of a move inside its cell: Q and P at node (x, y) in row x + 2 y, the r
+// face's charge at th node y, the th face's at r node x
+enum { CI_Q = 0, CI_P = 4, CI_R = 8, CI_T = 10, CI_ROWS = 12 };
 
 struct CDepK {
     int Nr, Nth, ld;
@@ -1814,132 +1822,171 @@ __device__ __forceinline__ void cd_lin(const GridDev& G, double r, double t, int
     locate(G.tn, G.itn, G.Nth + 1, t, (f32_est(t) - G.t0) * G.it, j, ft);
 }
 
-// window base cell of each particle alive before the move (C: skipped / removed)
+// Bucket of each particle alive before the move: its cell, or C + the window
+// base cell of a move across a boundary (2 C: skipped / removed).
 __global__ void k_cdep_keys(CDepK k, uint32_t* key, uint32_t* count, uint32_t C, long long* n_skip)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool valid = p < k.n;
-    uint32_t kk = C;
+    uint32_t kk = 2 * C;
     if (valid && k.alive0[p]) {
         int ia, ja, ib, jb;
         double f;
         cd_lin(k.G, k.r0[p], k.t0[p], ia, f, ja, f);
         cd_lin(k.G, k.r1[p], k.t1[p], ib, f, jb, f);
         if (abs(ia - ib) > 1 || abs(ja - jb) > 1) atomicAdd((unsigned long long*)n_skip, 1ull);
-        else kk = (uint32_t)min(ia, ib) * (uint32_t)k.Nth + (uint32_t)min(ja, jb);
+        else kk = (uint32_t)min(ia, ib) * (uint32_t)k.Nth + (uint32_t)min(ja, jb) + (ia == ib && ja == jb ? 0u : C);
     }
     if (valid) key[p] = kk;
     count_key(count, kk, valid);
 }
 
-// coordinate dph/dt = alpha gamma^{ph j} u_j / Gamma.  sin/cos th by angle
-// addition from the tabulated node tn[j] of the particle's cell (the step
-// t - tn[j] is under a cell, so its sin / cos - 1 come from the series), and
-// 1/Gamma as one reciprocal square root.
+// coordinate dph/dt = alpha gamma^{ph j} u_j / Gamma, sin/cos th by angle
+// addition from the tabulated node tn[j] of the particle's cell; the metric
+// as in eval_rhs_sc_t.
 __device__ __forceinline__ double cd_phdot(const BH& bh, const GridDev& G, const double* trig, int j, double r,
                                            double t, double ur, double ut, double up)
 {
-    double sh, cm;
-    sincos_step(t - G.tn[j], sh, cm);
-    const double s0 = trig[j], c0 = trig[G.Nth + 1 + j];
-    const double s = fma(s0, cm, fma(c0, sh, s0)), c = fma(c0, cm, fma(-s0, sh, c0));
-    Geo g;
-    geo_eval(bh, r, s, c, g);
-    const double iG = rsqrt_nr(fma(g.gurr * ur, ur, fma(2.0 * g.gurp * ur, up, fma(g.gutt * ut, ut, fma(g.gupp * up, up, 1.0)))));
-    return g.alpha * fma(g.gurp, ur, g.gupp * up) * iG;
+    double s, c;
+    sincos_near(G.tn[j], trig[j], trig[G.Nth + 1 + j], t, s, c);
+    const double s2 = s * s, rho2 = fma(bh.a2, c * c, r * r);
+    const double gpp = rcp_nr(rho2 * s2), irho2 = gpp * s2;
+    const double alpha = rsqrt_nr(fma(bh.twoM * irho2, r, 1.0));
+    const double iu = (alpha * alpha) * ur, tu = gpp * up, g1 = fma(bh.a * s2, ur, up);
+    const double Q = fma(fma(bh.a * ur, g1 + up, ut * ut), irho2, tu * up);
+    const double iG = rsqrt_nr(fma(iu, ur, 1.0 + Q));
+    return alpha * fma(bh.a * irho2, ur, tu) * iG;
 }
 
-// one warp per window-base cell: its particles' 30 window partials, summed
-__global__ void k_cdep_cell(CDepK k, const uint32_t* __restrict__ off, const uint32_t* __restrict__ perm,
-                            double* __restrict__ part, uint32_t C)
+// One thread per sorted entry: entries below off[C] are moves inside their
+// cell (CI_ROWS records), the rest up to off[2 C] the general ones (CD_SLOTS).
+__global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ CDepK k,
+                                                       const uint32_t* __restrict__ off,
+                                                       const uint32_t* __restrict__ perm, double* __restrict__ rec,
+                                                       uint32_t C)
 {
-    const long long cell = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (cell >= C) return;
-    const uint32_t b0 = off[cell], b1 = off[cell + 1];
-    const int i0 = (int)(cell / k.Nth), j0 = (int)(cell - (long long)i0 * k.Nth);
-    double acc = 0.0;           // lane q: slot q of the cell (q < CD_SLOTS)
-    for (uint32_t base = b0; base < b1; base += 32) {
-        double v[32];
-#pragma unroll
-        for (int q = 0; q < 32; ++q) v[q] = 0.0;
-        const uint32_t a = base + lane;
-        if (a < b1) {
-            const uint32_t p = perm[a];
-            int ia, ja, ib, jb;
-            double fra, fta, frb, ftb;
-            cd_lin(k.G, k.r0[p], k.t0[p], ia, fra, ja, fta);
-            cd_lin(k.G, k.r1[p], k.t1[p], ib, frb, jb, ftb);
-            // window weights by selects (registers, no indexed local arrays)
-            const int da = ia - i0, db = ib - i0, ea = ja - j0, eb = jb - j0;
-            double Sra[3], Srb[3], Sta[3], Stb[3];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                Sra[x] = x == da ? 1.0 - fra : (x == da + 1 ? fra : 0.0);
-                Srb[x] = x == db ? 1.0 - frb : (x == db + 1 ? frb : 0.0);
-                Sta[x] = x == ea ? 1.0 - fta : (x == ea + 1 ? fta : 0.0);
-                Stb[x] = x == eb ? 1.0 - ftb : (x == eb + 1 ? ftb : 0.0);
-            }
-            const double Q = k.w[p] * k.qm[p];
-            const double phd = 0.5 * (cd_phdot(k.bh, k.G, k.trig, ja, k.r0[p], k.t0[p], k.ur0[p], k.ut0[p], k.up0[p]) +
-                                      cd_phdot(k.bh, k.G, k.trig, jb, k.r1[p], k.t1[p], k.ur1[p], k.ut1[p], k.up1[p]));
-            // factors shared by the slots: Q S_r^{n+1}, Q (dph/dt) / 2, the
-            // half differences and sums of the weights
-            const double Qh = 0.5 * Q * phd;
-            double QSrb[3], dSr[2], aSr[3], dSt[2], sSt[3];
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                QSrb[x] = Q * Srb[x];
-                aSr[x] = 0.5 * (Sra[x] + Srb[x]);
-                sSt[x] = Sta[x] + Stb[x];
-            }
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                dSr[x] = 0.5 * (Srb[x] - Sra[x]);
-                dSt[x] = Stb[x] - Sta[x];
-            }
-#pragma unroll
-            for (int x = 0; x < 3; ++x)
-#pragma unroll
-                for (int y = 0; y < 3; ++y) {
-                    v[CD_Q + 3 * x + y] = QSrb[x] * Stb[y];
-                    v[CD_P + 3 * x + y] = Qh * fma(Sra[x], Sta[y], Srb[x] * Stb[y]);
-                }
-#pragma unroll
-            for (int y = 0; y < 3; ++y) {
-                double s_ = 0.0;
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    s_ = fma(dSr[x], sSt[y], s_);
-                    v[CD_R + 3 * x + y] = -Q * s_;
-                }
-            }
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                double s_ = 0.0;
-#pragma unroll
-                for (int y = 0; y < 2; ++y) {
-                    s_ = fma(aSr[x], dSt[y], s_);
-                    v[CD_T + 2 * x + y] = -Q * s_;
-                }
-            }
-        }
-        // reduce-scatter across the warp (recursive halving): each step a lane
-        // keeps half of its slots and adds its partner's copy of them; after
-        // five steps lane q holds the warp's sum of slot q (31 adds per lane)
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            const bool upper = (lane & o) != 0;
-#pragma unroll
-            for (int q = 0; q < o; ++q) {
-                const double send = upper ? v[q] : v[q + o];
-                const double keep = upper ? v[q + o] : v[q];
-                v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-        }
-        acc += v[0];
+    const long long a = blockIdx.x * 128LL + threadIdx.x;
+    if (a >= (long long)off[2 * (size_t)C]) return;
+    const uint32_t p = perm[a];
+    const bool inside = a < (long long)off[C];
+    int ia, ja, ib, jb;
+    double fra, fta, frb, ftb;
+    const double r0 = k.r0[p], t0 = k.t0[p], r1 = k.r1[p], t1 = k.t1[p];
+    cd_lin(k.G, r0, t0, ia, fra, ja, fta);
+    cd_lin(k.G, r1, t1, ib, frb, jb, ftb);
+    const double Q = k.w[p] * k.qm[p];
+    const double ph = cd_phdot(k.bh, k.G, k.trig, ja, r0, t0, k.ur0[p], k.ut0[p], k.up0[p]) +
+                      cd_phdot(k.bh, k.G, k.trig, jb, r1, t1, k.ur1[p], k.ut1[p], k.up1[p]);
+    const double Qh = 0.25 * Q * ph;         // Q (dph/dt)_mid / 2
+    rec += a;
+    auto put = [&](int row, double v) { rec[row * k.n] = v; };
+    if (inside) {
+        const double qx = Q * frb, qc = Q - qx, q11 = qx * ftb, q01 = qc * ftb;
+        put(CI_Q + 0, qc - q01);
+        put(CI_Q + 1, qx - q11);
+        put(CI_Q + 2, q01);
+        put(CI_Q + 3, q11);
+        const double sx = fra + frb, sy = fta + ftb, px = Qh * sx;
+        const double p11 = Qh * fma(fra, fta, frb * ftb), p01 = fma(Qh, sy, -p11);
+        put(CI_P + 0, fma(2.0, Qh, -px) - p01);
+        put(CI_P + 1, px - p11);
+        put(CI_P + 2, p01);
+        put(CI_P + 3, p11);
+        const double qr = Q * (frb - fra), qt = Q * (ftb - fta);
+        const double r1h = half_of(qr) * sy, t1h = half_of(qt) * sx;
+        put(CI_R + 0, qr - r1h);
+        put(CI_R + 1, r1h);
+        put(CI_T + 0, qt - t1h);
+        put(CI_T + 1, t1h);
+        return;
     }
-    if (lane < CD_SLOTS) part[(size_t)lane * C + cell] = acc;
+    // window weights by selects (registers, no indexed local arrays)
+    const int da = ia - min(ia, ib), db = ib - min(ia, ib), ea = ja - min(ja, jb), eb = jb - min(ja, jb);
+    double Sra[3], Srb[3], Sta[3], Stb[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        Sra[x] = x == da ? 1.0 - fra : (x == da + 1 ? fra : 0.0);
+        Srb[x] = x == db ? 1.0 - frb : (x == db + 1 ? frb : 0.0);
+        Sta[x] = x == ea ? 1.0 - fta : (x == ea + 1 ? fta : 0.0);
+        Stb[x] = x == eb ? 1.0 - ftb : (x == eb + 1 ? ftb : 0.0);
+    }
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        const double q = Q * Srb[x];
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            put(CD_Q + 3 * x + y, q * Stb[y]);
+            put(CD_P + 3 * x + y, Qh * fma(Sra[x], Sta[y], Srb[x] * Stb[y]));
+        }
+    }
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+        const double sSt = Sta[y] + Stb[y];
+        double s_ = 0.0;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            s_ = fma(0.5 * (Srb[x] - Sra[x]), sSt, s_);
+            put(CD_R + 3 * x + y, -Q * s_);
+        }
+    }
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        const double aSr = 0.5 * (Sra[x] + Srb[x]);
+        double s_ = 0.0;
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            s_ = fma(aSr, Stb[y] - Sta[y], s_);
+            put(CD_T + 2 * x + y, -Q * s_);
+        }
+    }
+}
+
+// One warp per cell: the 12 rows of its inside moves (32 particles at a time
+// through shared memory, lane 2 row + parity sums its row over the particles
+// of its parity, as in k_dep_cell), then lane q < 30 slot q of its general
+// moves; both in a fixed order.
+constexpr int CDEP_WARPS = 8;
+__global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __restrict__ rec,
+                                                               const uint32_t* __restrict__ off, long long n,
+                                                               double* __restrict__ part, uint32_t C)
+{
+    __shared__ double sv[CDEP_WARPS][CI_ROWS * DEP_CELL_LD];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long cell = blockIdx.x * (long long)CDEP_WARPS + wid;
+    if (cell >= C) return;                  // whole warps
+    double* v = sv[wid];
+    const uint32_t b0 = off[cell], b1 = off[cell + 1], c0 = off[(size_t)C + cell], c1 = off[(size_t)C + cell + 1];
+    const int row = min(lane >> 1, CI_ROWS - 1), par = lane & 1;
+    double acc = 0.0;
+    for (uint32_t base = b0; base < b1; base += 32) {
+        const uint32_t cnt = min(32u, b1 - base);
+        const bool live = (uint32_t)lane < cnt;
+        double x[CI_ROWS];
+#pragma unroll
+        for (int q = 0; q < CI_ROWS; ++q) x[q] = live ? __ldg(rec + (size_t)q * n + base + lane) : 0.0;
+        __syncwarp();                       // the previous group's reads are done
+#pragma unroll
+        for (int q = 0; q < CI_ROWS; ++q) v[q * DEP_CELL_LD + lane] = x[q];
+        __syncwarp();
+        const int kend = (int)(cnt + 1) >> 1;
+        for (int k = 0; k < kend; ++k) acc += v[row * DEP_CELL_LD + 2 * k + par];
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    double g = 0.0;
+    const int slot = min(lane, CD_SLOTS - 1);
+    for (uint32_t a = c0; a < c1; ++a) g += __ldg(rec + (size_t)slot * n + a);
+    // the inside row that belongs to this lane's slot, if any
+    int src = -1;
+    if (slot < CD_R) {
+        const int q = slot % 9, x = q / 3, y = q % 3;
+        if (x < 2 && y < 2) src = (slot < CD_P ? CI_Q : CI_P) + x + 2 * y;
+    } else if (slot < CD_T) {
+        if (slot - CD_R < 2) src = CI_R + (slot - CD_R);
+    } else if (slot == CD_T || slot == CD_T + 2) {
+        src = CI_T + ((slot - CD_T) >> 1);
+    }
+    const double in = __shfl_sync(0xffffffffu, acc, 2 * max(src, 0));
+    if (lane < CD_SLOTS) part[(size_t)lane * C + cell] = src >= 0 ? in + g : g;
 }
 
 __device__ __forceinline__ double cd_dual_r(const GridDev& G, int i)
@@ -2002,23 +2049,27 @@ extern "C" int fpic_deposit_conserving(fpic_ctx* c, const fpic_particles* before
     cudaStream_t s = (cudaStream_t)stream;
     const long long C = (long long)c->Nr * c->Nth;
     Work w;
-    void* part_v = nullptr;     // per-cell window partials, CD_SLOTS x C doubles
-    int rc = work_layout(c, n > 0 ? n : 1, false, w, (size_t)CD_SLOTS * C * sizeof(double), &part_v);
+    void* part_v = nullptr;     // per-cell window partials (CD_SLOTS x C), the particles' records (CD_SLOTS x n)
+    const long long nn = n > 0 ? n : 1;
+    int rc = work_layout(c, nn, false, w, (size_t)CD_SLOTS * (C + nn) * sizeof(double), &part_v, 2);
     if (rc) return rc;
     double* part = (double*)part_v;
+    double* rec = part + (size_t)CD_SLOTS * C;
     CDepK k{c->Nr, c->Nth, c->ld, c->G, c->bh, n, before->r, before->th, before->ur, before->uth, before->uph,
             before->alive, after->r, after->th, after->ur, after->uth, after->uph, after->qm, after->w,
             c->d_metric + (size_t)MT_N * c->metric_stride};
-    FPIC_CUDA(cudaMemsetAsync(w.count, 0, 4 * ((size_t)C + 2), s));
-    FPIC_CUDA(cudaMemsetAsync(w.cursor, 0, 4 * ((size_t)C + 2), s));
+    FPIC_CUDA(cudaMemsetAsync(w.count, 0, 4 * (2 * (size_t)C + 2), s));
+    FPIC_CUDA(cudaMemsetAsync(w.cursor, 0, 4 * (2 * (size_t)C + 2), s));
     FPIC_CUDA(cudaMemsetAsync(c->d_cnt + CNT_ERR, 0, sizeof(long long), s));
     const unsigned nb = (unsigned)((n + 255) / 256);
     if (n > 0) k_cdep_keys<<<nb, 256, 0, s>>>(k, w.key, w.count, (uint32_t)C, c->d_cnt + CNT_ERR);
-    rc = scan_u32(w.count, w.off, w.bsum, C + 1, s);
+    rc = scan_u32(w.count, w.off, w.bsum, 2 * C + 1, s);
     if (rc) return rc;
     if (n > 0) k_scatter<<<nb, 256, 0, s>>>(w.key, w.off, w.cursor, w.perm, n);
-    k_bucket_rank<<<(unsigned)((C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, (uint32_t)C);
-    k_cdep_cell<<<(unsigned)((C * 32 + 255) / 256), 256, 0, s>>>(k, w.off, w.perm2, part, (uint32_t)C);
+    k_bucket_rank<<<(unsigned)((2 * C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, 2 * (uint32_t)C);
+    if (n > 0) k_cdep_particle<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(k, w.off, w.perm2, rec, (uint32_t)C);
+    k_cdep_cell<<<(unsigned)((C + CDEP_WARPS - 1) / CDEP_WARPS), 32 * CDEP_WARPS, 0, s>>>(rec, w.off, nn, part,
+                                                                                         (uint32_t)C);
     k_cdep_node<<<dim3((unsigned)((c->Nth + 1 + 255) / 256), c->Nr + 1), 256, 0, s>>>(k, tabs_of(c), part,
                                                                                      (uint32_t)C, dt, rho, jr,
                                                                                      jth, jph);
@@ -2046,23 +2097,10 @@ namespace fpic {
 struct CleanK {
     int Nr, Nth, ld;
     GridDev G;
-    Tabs T;                                  // metric tables at the Yee points
-    double *c_r1, *c_r0, *c_t1, *c_t0, *b;   // per node (library scratch)
+    Tabs T;                  // metric tables at the Yee points
+    double2 *cr, *ct;        // per node (library scratch): (c_r1, c_r0), (c_t1, c_t0)
+    double *nb;              // and -b
 };
-
-// Inverse spatial metric from the tabulated lower one: the th block is
-// diagonal, the (r, ph) block a 2 x 2 inverse.
-__device__ __forceinline__ double tab_gu_rr(const Tabs& T, int i, int j)       // at (i+1/2, j)
-{
-    const double grr = T.at(T_RR1, i, j), grp = T.at(T_RP1, i, j), gpp = T.at(T_PP1, i, j);
-    return gpp / fma(grr, gpp, -grp * grp);
-}
-
-__device__ __forceinline__ double tab_gu_rp(const Tabs& T, int i, int j)       // at (i, j)
-{
-    const double grr = T.at(T_RR0, i, j), grp = T.at(T_RP0, i, j), gpp = T.at(T_PP0, i, j);
-    return -grp / fma(grr, gpp, -grp * grp);
-}
 
 __global__ void k_clean_setup(CleanK k, const double* __restrict__ Dr, const double* __restrict__ Dt,
                               const double* __restrict__ rho)
@@ -2070,53 +2108,61 @@ __global__ void k_clean_setup(CleanK k, const double* __restrict__ Dr, const dou
     const int i = blockIdx.y + 1;                   // 1 .. Nr-1
     const GridDev& G = k.G;
     const Tabs& T = k.T;
-    const double dr = G.rh[i] - G.rh[i - 1];
-    const double ir1 = 1.0 / ((G.rn[i + 1] - G.rn[i]) * dr), ir0 = 1.0 / ((G.rn[i] - G.rn[i - 1]) * dr);
+    const double idr = G.irh[i - 1], ir1 = G.irn[i] * idr, ir0 = G.irn[i - 1] * idr;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= k.Nth; j += gridDim.x * blockDim.x) {
         const size_t o = (size_t)i * k.ld + j;
-        const double dth = (j < k.Nth ? G.th[j] : M_PI) - (j > 0 ? G.th[j - 1] : 0.0);
+        const bool up = j < k.Nth, dn = j > 0;
+        const double idth = up && dn ? G.ith[j - 1] : rcp_nr((up ? G.th[j] : M_PI) - (dn ? G.th[j - 1] : 0.0));
         const double sr1 = T.at(T_SG1, i, j), sr0 = T.at(T_SG1, i - 1, j);
-        const double st1 = j < k.Nth ? T.at(T_SG2, i, j) : 0.0, st0 = j > 0 ? T.at(T_SG2, i, j - 1) : 0.0;
-        const double rhs = (sr1 * Dr[o] - sr0 * Dr[o - k.ld]) / dr +
-                           ((j < k.Nth ? st1 * Dt[o] : 0.0) - (j > 0 ? st0 * Dt[o - 1] : 0.0)) / dth -
+        const double st1 = up ? T.at(T_SG2, i, j) : 0.0, st0 = dn ? T.at(T_SG2, i, j - 1) : 0.0;
+        const double rhs = (sr1 * Dr[o] - sr0 * Dr[o - k.ld]) * idr +
+                           ((up ? st1 * Dt[o] : 0.0) - (dn ? st0 * Dt[o - 1] : 0.0)) * idth -
                            4.0 * M_PI * T.at(T_SG0, i, j) * rho[o];
-        const double cr1 = sr1 * tab_gu_rr(T, i, j) * ir1;
-        const double cr0 = sr0 * tab_gu_rr(T, i - 1, j) * ir0;
-        const double ct1 = j < k.Nth ? st1 / (T.at(T_TT2, i, j) * (G.tn[j + 1] - G.tn[j]) * dth) : 0.0;
-        const double ct0 = j > 0 ? st0 / (T.at(T_TT2, i, j - 1) * (G.tn[j] - G.tn[j - 1]) * dth) : 0.0;
-        const double inv = 1.0 / (cr1 + cr0 + ct1 + ct0);
-        k.c_r1[o] = cr1 * inv;
-        k.c_r0[o] = cr0 * inv;
-        k.c_t1[o] = ct1 * inv;
-        k.c_t0[o] = ct0 * inv;
-        k.b[o] = rhs * inv;
+        const double cr1 = sr1 * T.at(T_URR1, i, j) * ir1;
+        const double cr0 = sr0 * T.at(T_URR1, i - 1, j) * ir0;
+        const double ct1 = up ? st1 * T.at(T_UTT2, i, j) * (G.itn[j] * idth) : 0.0;
+        const double ct0 = dn ? st0 * T.at(T_UTT2, i, j - 1) * (G.itn[j - 1] * idth) : 0.0;
+        const double inv = rcp_nr(cr1 + cr0 + ct1 + ct0);
+        k.cr[o] = make_double2(cr1 * inv, cr0 * inv);
+        k.ct[o] = make_double2(ct1 * inv, ct0 * inv);
+        k.nb[o] = -rhs * inv;
     }
 }
 
 // One Jacobi sweep over the interior nodes (phi_in -> phi_out); the radial
-// end rows stay zero in both buffers.  A thread walks JAC_ROWS rows of one
-// theta column keeping the column's three radial neighbours in registers,
-// so each phi value comes from L2 about once per sweep; the theta
-// neighbours are the same row's loads of the adjacent threads (L1).
-constexpr int JAC_ROWS = 8, JAC_THREADS = 128;
-__global__ void __launch_bounds__(JAC_THREADS) k_jacobi(CleanK k, const double* __restrict__ phi_in,
-                                                        double* __restrict__ phi_out)
+// end rows stay zero in both buffers.  A warp takes two rows of 32 theta
+// columns; neighbours come from L1 and L2.  Four fused multiply-adds a node
+// (the sum starts from -b): FP64-pipe bound at best, 6.7 us a sweep on 1024 x
+// 1024.  What stands in the way is latency: a sweep is a few microseconds of
+// work between two launches.  Hence short blocks (3 to 16 rows a warp measured
+// 5 to 30 % slower), the coefficients loaded before the wait for the previous
+// sweep (programmatic dependent launch inside the graph of sweeps): a
+// cleaning of 500 sweeps 6564 -> 4360 us on 1024 x 1024, 2195 -> 727 us on
+// 64 x 64.
+constexpr int JAC_WARPS = 4, JAC_ROWS = 2;          // warps of a block, rows of a warp
+__global__ void __launch_bounds__(32 * JAC_WARPS, 7) k_jacobi(CleanK k, const double* phi_in, double* phi_out)
 {
-    const int j = blockIdx.x * JAC_THREADS + threadIdx.x;
-    if (j > k.Nth) return;
-    const int i0 = 1 + blockIdx.y * JAC_ROWS;
-    const int i1 = min(i0 + JAC_ROWS, k.Nr);        // exclusive
-    size_t o = (size_t)i0 * k.ld + j;
-    double dn = phi_in[o - k.ld], mid = phi_in[o];
-    for (int i = i0; i < i1; ++i, o += k.ld) {
-        const double up = phi_in[o + k.ld];
-        double s = fma(k.c_r1[o], up, k.c_r0[o] * dn);
-        if (j < k.Nth) s = fma(k.c_t1[o], phi_in[o + 1], s);
-        if (j > 0) s = fma(k.c_t0[o], phi_in[o - 1], s);
-        phi_out[o] = s - k.b[o];
-        dn = mid;
-        mid = up;
-    }
+    const int j = min((int)(blockIdx.x * 32 + (threadIdx.x & 31)), k.Nth);       // idle lanes repeat the last column
+    const int i = 1 + ((int)blockIdx.y * JAC_WARPS + (int)(threadIdx.x >> 5)) * JAC_ROWS;
+    if (i >= k.Nr) return;
+    const size_t ld = k.ld, o0 = (size_t)i * ld + j, o1 = i + 1 < k.Nr ? o0 + ld : o0;   // a last odd row twice
+    const double2 cr0 = __ldg(k.cr + o0), ct0 = __ldg(k.ct + o0), cr1 = __ldg(k.cr + o1), ct1 = __ldg(k.ct + o1);
+    const double nb0 = __ldg(k.nb + o0), nb1 = __ldg(k.nb + o1);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // neighbours beyond the poles: any finite value, their coefficients are zero
+    const int jl = j > 0 ? 1 : 0, jr = j < k.Nth ? 1 : 0;
+    const double dn0 = phi_in[o0 - ld], up0 = phi_in[o0 + ld], l0 = phi_in[o0 - jl], r0 = phi_in[o0 + jr];
+    const double dn1 = phi_in[o1 - ld], up1 = phi_in[o1 + ld], l1 = phi_in[o1 - jl], r1 = phi_in[o1 + jr];
+    double v0 = fma(cr0.y, dn0, nb0), v1 = fma(cr1.y, dn1, nb1);
+    v0 = fma(cr0.x, up0, v0);
+    v1 = fma(cr1.x, up1, v1);
+    v0 = fma(ct0.x, r0, v0);
+    v1 = fma(ct1.x, r1, v1);
+    v0 = fma(ct0.y, l0, v0);
+    v1 = fma(ct1.y, l1, v1);
+    phi_out[o0] = v0;
+    phi_out[o1] = v1;
 }
 
 // D^i -= gamma^ij d_j phi: D^r at (i+1/2, j), D^th at (i, j+1/2), D^ph at
@@ -2127,16 +2173,15 @@ __global__ void k_clean_correct(CleanK k, const double* __restrict__ phi, double
     const int i = blockIdx.y;                       // 0 .. Nr
     const GridDev& G = k.G;
     const Tabs& T = k.T;
-    const double iu = i < k.Nr ? 1.0 / (G.rn[i + 1] - G.rn[i]) : 0.0;
-    const double id = i > 0 ? 1.0 / (G.rn[i] - G.rn[i - 1]) : 0.0;
+    const double iu = i < k.Nr ? G.irn[i] : 0.0, id = i > 0 ? G.irn[i - 1] : 0.0;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= k.Nth; j += gridDim.x * blockDim.x) {
         const size_t o = (size_t)i * k.ld + j;
         const double up = i < k.Nr ? (phi[o + k.ld] - phi[o]) * iu : 0.0;
         const double dn = i > 0 ? (phi[o] - phi[o - k.ld]) * id : 0.0;
         const double mean = (i > 0 && i < k.Nr) ? 0.5 * (up + dn) : up + dn;
-        if (i < k.Nr) Dr[o] -= tab_gu_rr(T, i, j) * up;
-        if (j < k.Nth) Dt[o] -= (phi[o + 1] - phi[o]) / (T.at(T_TT2, i, j) * (G.tn[j + 1] - G.tn[j]));
-        Dp[o] -= tab_gu_rp(T, i, j) * mean;
+        if (i < k.Nr) Dr[o] -= T.at(T_URR1, i, j) * up;
+        if (j < k.Nth) Dt[o] -= T.at(T_UTT2, i, j) * ((phi[o + 1] - phi[o]) * G.itn[j]);
+        Dp[o] -= T.at(T_URP0, i, j) * mean;
     }
 }
 
@@ -2340,28 +2385,39 @@ extern "C" int fpic_div_clean(fpic_ctx* c, double* const D[3], const double* rho
     int rc = ensure_scratch2(c, 7 * sz * sizeof(double) + 256);
     if (rc) return rc;
     double* base = (double*)c->d_scratch2;
-    CleanK k{c->Nr, c->Nth, c->ld, c->G, tabs_of(c), base, base + sz, base + 2 * sz, base + 3 * sz, base + 4 * sz};
+    CleanK k{c->Nr, c->Nth, c->ld, c->G, tabs_of(c), (double2*)base, (double2*)base + sz, base + 4 * sz};
     double* pa = base + 5 * sz;
     double* pb = base + 6 * sz;
     FPIC_CUDA(cudaMemsetAsync(pa, 0, 2 * sz * sizeof(double), s));
     if (c->Nr >= 2) {
         const unsigned gx = (unsigned)((c->Nth + 1 + 255) / 256);
         k_clean_setup<<<dim3(gx, c->Nr - 1), 256, 0, s>>>(k, D[0], D[1], rho);
-        const dim3 jg((unsigned)((c->Nth + 1 + JAC_THREADS - 1) / JAC_THREADS),
-                      (unsigned)((c->Nr - 1 + JAC_ROWS - 1) / JAC_ROWS));
-        auto sweeps = [&](cudaStream_t st) {
+        const dim3 jg((unsigned)((c->Nth + 32) / 32),
+                      (unsigned)((c->Nr - 1 + JAC_WARPS * JAC_ROWS - 1) / (JAC_WARPS * JAC_ROWS)));
+        auto sweeps = [&](cudaStream_t st, bool chained) -> int {
             double *x = base + 5 * sz, *y = base + 6 * sz;
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at.val.programmaticStreamSerializationAllowed = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = jg;
+            cfg.blockDim = dim3(32 * JAC_WARPS);
+            cfg.stream = st;
+            cfg.attrs = &at;
             for (int it = 0; it < n_iter; ++it) {
-                k_jacobi<<<jg, JAC_THREADS, 0, st>>>(k, x, y);
+                cfg.numAttrs = chained && it > 0 ? 1 : 0;    // a sweep after a sweep of the same graph
+                FPIC_CUDA(cudaLaunchKernelEx(&cfg, k_jacobi, k, (const double*)x, y));
                 double* t = x;
                 x = y;
                 y = t;
             }
+            return 0;
         };
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         FPIC_CUDA(cudaStreamIsCapturing(s, &cap));
         if (n_iter < 8 || cap != cudaStreamCaptureStatusNone) {
-            sweeps(s);       // short chains, or the caller is recording a graph itself
+            rc = sweeps(s, false);  // short chains, or the caller is recording a graph itself
+            if (rc) return rc;
         } else {
             // hundreds of short launches: replay them as one graph
             if (!c->clean_exec || c->clean_key_base != base || c->clean_key_Nr != c->Nr ||
@@ -2372,8 +2428,13 @@ extern "C" int fpic_div_clean(fpic_ctx* c, double* const D[3], const double* rho
                 if (rc2) return rc2;
                 cudaGraph_t g = nullptr;
                 FPIC_CUDA(cudaStreamBeginCapture(c->copy_stream, cudaStreamCaptureModeThreadLocal));
-                sweeps(c->copy_stream);
-                FPIC_CUDA(cudaStreamEndCapture(c->copy_stream, &g));
+                rc = sweeps(c->copy_stream, true);
+                const cudaError_t ec = cudaStreamEndCapture(c->copy_stream, &g);
+                if (rc) {
+                    if (g) cudaGraphDestroy(g);
+                    return rc;
+                }
+                FPIC_CUDA(ec);
                 cudaError_t e = cudaGraphInstantiate(&c->clean_exec, g, 0);
                 cudaGraphDestroy(g);
                 FPIC_CUDA(e);
