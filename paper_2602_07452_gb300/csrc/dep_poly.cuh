@@ -31,71 +31,105 @@ constexpr int POLY_STRIDE = 28;      // floats of a cell (25 used): seven 16-byt
 constexpr double POLY_TOL = 2e-14;
 constexpr double POLY_MAX_DTH = 0.03, POLY_MAX_TAU = 4.0;     // limits of the sin th series
 
-// f_mn (m + n <= 6, f[m][n]) of the cell of centre (x, y) and size (dx, dy).
-__host__ __device__ inline void poly_series(double M, double a, double x, double y, double dx, double dy,
-                                            double f[7][7])
+// What a th cell of centre yc (sin, cos given) and size dy brings to its cells'
+// series: P1 = r^2 + a^2 cos^2 th = r^2 + sum_n p[n] eta^n.
+struct PolyTheta {
+    double p[7];
+};
+
+__host__ __device__ inline void poly_theta(double a, double s, double c, double dy, PolyTheta& t)
 {
-    constexpr int D = 6;
-    // P1 = r^2 + a^2 cos^2 th = sum_n p[n] eta^n + p1 xi + p2 xi^2
-    double p[D + 1];
-    const double c = cos(y), s2y = 2.0 * sin(y) * c, c2y = 2.0 * c * c - 1.0;
+    const double s2y = 2.0 * s * c, c2y = 2.0 * c * c - 1.0;
     double h = 0.5 * a * a;
 #pragma unroll
-    for (int n = 1; n <= D; ++n) {
-        h *= 2.0 * dy / n;
-        const double t = (n & 1) ? s2y : c2y;
-        p[n] = ((n & 3) == 1 || (n & 3) == 2) ? -h * t : h * t;
+    for (int n = 1; n <= 6; ++n) {
+        h *= 2.0 * dy * (1.0 / n);
+        const double v = (n & 1) ? s2y : c2y;
+        t.p[n] = ((n & 3) == 1 || (n & 3) == 2) ? -h * v : h * v;
     }
-    p[0] = x * x + a * a * c * c;
-    const double p1 = 2.0 * x * dx, p2 = dx * dx;
-    // g = P1 (P1 + 2 M r) / g_00, then f = sqrt(g)
-    const double q0 = 2.0 * M * x, q1 = 2.0 * M * dx;
+    t.p[0] = a * a * c * c;
+}
+
+// Coefficient (m, n) of g = P1 (P1 + 2 M r), P1 = x^2 + sum p[n] eta^n + p1 xi + p2 xi^2.
+template <typename R>
+__host__ __device__ inline R poly_g(int m, int n, const R* p, R p1, R p2, R q0, R q1)
+{
+    R g = R(0);
+    if (m == 0) {
+        g = q0 * p[n];
+#pragma unroll
+        for (int j = 0; j <= n; ++j) g += p[j] * p[n - j];
+    } else if (m == 1) {
+        g = (R(2) * p1 + q1) * p[n] + (n == 0 ? q0 * p1 : R(0));
+    } else if (m == 2) {
+        g = R(2) * p2 * p[n] + (n == 0 ? p1 * p1 + q0 * p2 + q1 * p1 : R(0));
+    } else if (n == 0 && m == 3) {
+        g = R(2) * p1 * p2 + q1 * p2;
+    } else if (n == 0 && m == 4) {
+        g = p2 * p2;
+    }
+    return g;
+}
+
+// f_mn of a cell of centre r = x and size dx: f = sqrt(g / g_00), to degree 3 in
+// FP64 (f[m][n]), to degree 6 in FP32 (q): those terms are used in FP32 and, at
+// degree 6, only bound the error.
+__host__ __device__ inline void poly_series(double M, double x, double dx, const PolyTheta& th, double f[4][4],
+                                            float q[7][7])
+{
+    double p[7];
+#pragma unroll
+    for (int n = 0; n < 7; ++n) p[n] = th.p[n];
+    p[0] += x * x;
+    const double p1 = 2.0 * x * dx, p2 = dx * dx, q0 = 2.0 * M * x, q1 = 2.0 * M * dx;
     const double ig = 1.0 / (p[0] * (p[0] + q0));
 #pragma unroll
-    for (int d = 0; d <= D; ++d)
+    for (int d = 0; d <= 3; ++d)
 #pragma unroll
         for (int m = 0; m <= d; ++m) {
             const int n = d - m;
-            double g = 0.0;
-            if (m == 0) {
-                g = q0 * p[n];
-#pragma unroll
-                for (int j = 0; j <= n; ++j) g += p[j] * p[n - j];
-            } else if (m == 1) {
-                g = (2.0 * p1 + q1) * p[n] + (n == 0 ? q0 * p1 : 0.0);
-            } else if (m == 2) {
-                g = 2.0 * p2 * p[n] + (n == 0 ? p1 * p1 + q0 * p2 + q1 * p1 : 0.0);
-            } else if (n == 0 && m == 3) {
-                g = 2.0 * p1 * p2 + q1 * p2;
-            } else if (n == 0 && m == 4) {
-                g = p2 * p2;
-            }
-            if (d == 0) {
-                f[0][0] = 1.0;
-                continue;
-            }
-            double t = g * ig;
+            double t = poly_g<double>(m, n, p, p1, p2, q0, q1) * ig;
 #pragma unroll
             for (int i = 0; i <= m; ++i)
 #pragma unroll
                 for (int j = 0; j <= n; ++j)
                     if (i + j > 0 && i + j < d) t -= f[i][j] * f[m - i][n - j];
-            f[m][n] = 0.5 * t;
+            f[m][n] = d == 0 ? 1.0 : 0.5 * t;
+            q[m][n] = (float)f[m][n];
+        }
+    // normalized by g_00 = (1 / ig): the float factors stay in range
+    const double is = sqrt(ig);
+    float pf[7];
+#pragma unroll
+    for (int n = 0; n < 7; ++n) pf[n] = (float)(p[n] * is);
+    const float p1f = (float)(p1 * is), p2f = (float)(p2 * is), q0f = (float)(q0 * is), q1f = (float)(q1 * is);
+#pragma unroll
+    for (int d = 4; d <= 6; ++d)
+#pragma unroll
+        for (int m = 0; m <= d; ++m) {
+            const int n = d - m;
+            float t = poly_g<float>(m, n, pf, p1f, p2f, q0f, q1f);
+#pragma unroll
+            for (int i = 0; i <= m; ++i)
+#pragma unroll
+                for (int j = 0; j <= n; ++j)
+                    if (i + j > 0 && i + j < d) t -= q[i][j] * q[m - i][n - j];
+            q[m][n] = 0.5f * t;
         }
 }
 
 // Bound on the error of a node share (a fraction of the cell): the terms of
 // degree 6 that are left out and the FP32 rounding of those of degree 3 to 5,
 // an interval's share of a cell's moment of xi^m being at most 2^-m / (2 m + 1).
-__host__ __device__ inline double poly_bound(const double f[7][7])
+__host__ __device__ inline float poly_bound(const float f[7][7])
 {
-    double e = 0.0;
+    float e = 0.f;
 #pragma unroll
     for (int d = 3; d <= 6; ++d)
 #pragma unroll
         for (int m = 0; m <= d; ++m) {
             const int n = d - m;
-            e += fabs(f[m][n]) * (d == 6 ? 1.0 : 5.9604644775390625e-8) / ((1 << d) * (2.0 * m + 1.0) * (2.0 * n + 1.0));
+            e += fabsf(f[m][n]) * (d == 6 ? 1.f : 5.9604644775390625e-8f) / (float)((1 << d) * (2 * m + 1) * (2 * n + 1));
         }
     return e;
 }

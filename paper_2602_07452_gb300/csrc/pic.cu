@@ -717,7 +717,7 @@ __device__ __forceinline__ void sincos_from_node(double s0, double c0, double d,
 {
     ff sh, cm;
     sincos_step_ff(d, sh, cm);
-    rotate_ff(ff_from(s0), ff_from(c0), sh, cm, s, c);
+    rotate_ff(ff_cut(s0), ff_cut(c0), sh, cm, s, c);
 }
 
 // The 7 th values of the lattice of [y0, y1] split at t: y0 + l hc
@@ -949,8 +949,8 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
     // integer lattice's is the particle's own th unless clamped)
     ff stn, ctn, sth, cth;
     if (same_bits(tn_c, t)) {
-        stn = ff_from(s);
-        ctn = ff_from(c);
+        stn = ff_cut(s);
+        ctn = ff_cut(c);
     } else {
         sincos_from_node(sn[jn], cn[jn], tn_c - G.tn[jn], stn, ctn);
     }
@@ -964,7 +964,7 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
     const double Ur = fma(g.gurr, ur, g.gurp * up), Ut = g.gutt * ut, Up = fma(g.gurp, ur, g.gupp * up);
     const double Qd = k.w[p] * k.qm[p];
     const double QiG = Qd * rsqrt_nr(fma(ur, Ur, fma(ut, Ut, fma(up, Up, 1.0))));
-    const ff Q = ff_from(Qd), Qr = ff_from(QiG * Ur), Qt = ff_from(QiG * Ut), Qp = ff_from(QiG * Up);
+    const ff Q = ff_cut(Qd), Qr = ff_cut(QiG * Ur), Qt = ff_cut(QiG * Ut), Qp = ff_cut(QiG * Up);
     const long long n = k.n_alive;
     // the split column / row are shared between the sub-grids unless clamped
     const bool share = same_bits(rn_c, rh_c) && same_bits(tn_c, th_c);
@@ -981,17 +981,17 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
             const double* sY = hth ? sh : sn;
             const double* cY = hth ? ch : cn;
             const double tc = hth ? th_c : tn_c;
-            hc = ff_mul(ff_from(tc - Y[jj]), bh.third);
-            hd = ff_mul(ff_from(Y[jj + 1] - tc), bh.third);
-            theta_lattice_ff(hc, hd, ff_from(sY[jj]), ff_from(cY[jj]), hth ? sth : stn, hth ? cth : ctn,
-                             ff_from(sY[jj + 1]), ff_from(cY[jj + 1]), sy, cy);
+            hc = ff_mul(ff_cut(tc - Y[jj]), bh.third);
+            hd = ff_mul(ff_cut(Y[jj + 1] - tc), bh.third);
+            theta_lattice_ff(hc, hd, ff_cut(sY[jj]), ff_cut(cY[jj]), hth ? sth : stn, hth ? cth : ctn,
+                             ff_cut(sY[jj + 1]), ff_cut(cY[jj + 1]), sy, cy);
         }
         const bool hr = sg == 1;
         const double x0 = hr ? G.rh[i1] : G.rn[i0], x1 = hr ? G.rh[i1 + 1] : G.rn[i0 + 1];
         const double rc = hr ? rh_c : rn_c;
-        const ff ha = ff_mul(ff_from(rc - x0), bh.third), hb = ff_mul(ff_from(x1 - rc), bh.third);
+        const ff ha = ff_mul(ff_cut(rc - x0), bh.third), hb = ff_mul(ff_cut(x1 - rc), bh.third);
         ff V[4];
-        subvolumes_ff(bh, ff_from(x0), ff_from(rc), ha, hb, hc, hd, sy, cy, V, col, row, share && sg == 1,
+        subvolumes_ff(bh, ff_cut(x0), ff_cut(rc), ha, hb, hc, hd, sy, cy, V, col, row, share && sg == 1,
                       share && sg == 2, sg == 0);
         const ff iV = ff_rcp(ff_add(ff_add(V[0], V[1]), ff_add(V[2], V[3])));
         // share of node (i+a, j+b) = V(opposite corner) / V
@@ -1008,17 +1008,19 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
     k.code[p] = (uint32_t)(i1 - i0 + 1) | ((uint32_t)(j1 - j0 + 1) << 2);
 }
 
-// Builds the cells' polynomials (sub-grid blockIdx.z, row blockIdx.y), the
-// 1-D tables and the largest bound over the cells (as the bits of a
-// non-negative double; a NaN exceeds every tolerance).  Once per grid, about
-// 250 FP64 operations a cell: less than the first deposit saves.
+// Builds the cells' polynomials (sub-grid blockIdx.z; a thread walks `rows`
+// cells down one th column, whose trigonometry it takes once), the 1-D
+// tables and the largest bound over the cells (as the bits of a non-negative
+// float; a NaN exceeds every tolerance).  Once per grid, about 60 FP64
+// operations a cell.
 struct PolyBuild {
     BH bh;
     GridDev G;
     float4* c[3];
     float2* ir[2];
     float4* t[2];
-    unsigned long long* bound;
+    unsigned* bound;
+    int rows;
 };
 
 __device__ __forceinline__ float2 pair_of(double d)
@@ -1029,31 +1031,39 @@ __device__ __forceinline__ float2 pair_of(double d)
 
 __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ PolyBuild k)
 {
-    const int sg = blockIdx.z, i = blockIdx.y, j = blockIdx.x * 128 + threadIdx.x;
+    const int sg = blockIdx.z, j = blockIdx.x * 128 + threadIdx.x;
     const GridDev& G = k.G;
     const bool hr = sg == 1, hth = sg == 2;
-    double e = 0.0;
-    if (i < G.Nr - hr && j < G.Nth - hth) {
+    const int i0 = blockIdx.y * k.rows, i1 = min(i0 + k.rows, G.Nr - hr);
+    float e = 0.f;
+    if (j < G.Nth - hth) {
         const double* X = hr ? G.rh : G.rn;
         const double* Y = hth ? G.th : G.tn;
-        const double dx = X[i + 1] - X[i], dy = Y[j + 1] - Y[j], y = 0.5 * (Y[j] + Y[j + 1]);
-        double f[7][7];
-        poly_series(k.bh.M, k.bh.a, 0.5 * (X[i] + X[i + 1]), y, dx, dy, f);
-        e = poly_bound(f);
-        float4* c = k.c[sg] + ((size_t)i * G.Nth + j) * (POLY_STRIDE / 4);
-        const float2 f10 = pair_of(f[1][0]), f01 = pair_of(f[0][1]), f20 = pair_of(f[2][0]), f11 = pair_of(f[1][1]),
-                     f02 = pair_of(f[0][2]);
-        c[0] = make_float4(f10.x, f10.y, f01.x, f01.y);
-        c[1] = make_float4(f20.x, f20.y, f11.x, f11.y);
-        c[2] = make_float4(f02.x, f02.y, (float)f[3][0], (float)f[2][1]);
-        c[3] = make_float4((float)f[1][2], (float)f[0][3], (float)f[4][0], (float)f[3][1]);
-        c[4] = make_float4((float)f[2][2], (float)f[1][3], (float)f[0][4], (float)f[5][0]);
-        c[5] = make_float4((float)f[4][1], (float)f[3][2], (float)f[2][3], (float)f[1][4]);
-        c[6] = make_float4((float)f[0][5], 0.f, 0.f, 0.f);
-        if (j == 0 && sg < 2) k.ir[sg][i] = pair_of(1.0 / dx);
-        if (i == 0 && sg != 1) {
-            double s, co;
-            sincos(y, &s, &co);
+        const double dy = Y[j + 1] - Y[j], y = 0.5 * (Y[j] + Y[j + 1]);
+        double s, co;
+        sincos(y, &s, &co);
+        PolyTheta th;
+        poly_theta(k.bh.a, s, co, dy, th);
+        for (int i = i0; i < i1; ++i) {
+            const double dx = X[i + 1] - X[i];
+            double f[4][4];
+            float q[7][7];
+            poly_series(k.bh.M, 0.5 * (X[i] + X[i + 1]), dx, th, f, q);
+            e = fmaxf(e, poly_bound(q));
+            if (!(e == e)) e = INFINITY;
+            float4* c = k.c[sg] + ((size_t)i * G.Nth + j) * (POLY_STRIDE / 4);
+            const float2 f10 = pair_of(f[1][0]), f01 = pair_of(f[0][1]), f20 = pair_of(f[2][0]),
+                         f11 = pair_of(f[1][1]), f02 = pair_of(f[0][2]);
+            c[0] = make_float4(f10.x, f10.y, f01.x, f01.y);
+            c[1] = make_float4(f20.x, f20.y, f11.x, f11.y);
+            c[2] = make_float4(f02.x, f02.y, q[3][0], q[2][1]);
+            c[3] = make_float4(q[1][2], q[0][3], q[4][0], q[3][1]);
+            c[4] = make_float4(q[2][2], q[1][3], q[0][4], q[5][0]);
+            c[5] = make_float4(q[4][1], q[3][2], q[2][3], q[1][4]);
+            c[6] = make_float4(q[0][5], 0.f, 0.f, 0.f);
+            if (j == 0 && sg < 2) k.ir[sg][i] = pair_of(1.0 / dx);
+        }
+        if (i0 == 0 && sg != 1) {
             const double tau = dy * co / s;
             const float2 it = pair_of(1.0 / dy), tp = pair_of(tau), d2 = pair_of(0.5 * dy * dy), d6 = pair_of(dy * dy / 6.0);
             float4* t = k.t[hth] + 2 * j;
@@ -1062,14 +1072,8 @@ __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ Poly
             if (!(s > 0.0 && dy <= POLY_MAX_DTH && fabs(tau) <= POLY_MAX_TAU)) e = INFINITY;
         }
     }
-    // NaN bits sort above every number's
-    for (int o = 16; o > 0; o >>= 1) {
-        const double y = __shfl_xor_sync(0xffffffffu, e, o);
-        const unsigned long long be = (unsigned long long)__double_as_longlong(e) & ~(1ull << 63),
-                                 by = (unsigned long long)__double_as_longlong(y) & ~(1ull << 63);
-        e = __longlong_as_double((long long)(be > by ? be : by));
-    }
-    if ((threadIdx.x & 31) == 0) atomicMax(k.bound, (unsigned long long)__double_as_longlong(e) & ~(1ull << 63));
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(e));
+    if ((threadIdx.x & 31) == 0) atomicMax(k.bound, m);
 }
 
 // The polynomials of the context's grid (built on first use, with one wait
@@ -1097,6 +1101,17 @@ static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
         for (int i = 0; i < c->Nr; ++i) dr = fmax(dr, (X[i + 1] - X[i]) / X[i]);
         for (int j = 0; j < c->Nth; ++j) dt = fmax(dt, Y[j + 1] - Y[j]);
         if (bytes > POLY_MAX_BYTES || dr > 0.05 || dt > POLY_MAX_DTH) return 0;
+        // a few cells of the first row, where the bound is largest on a log grid
+        for (int q = 0; q < 16; ++q) {
+            const int j = (int)((long long)q * (c->Nth - 1) / 15);
+            const double y = 0.5 * (Y[j] + Y[j + 1]);
+            PolyTheta th;
+            double f[4][4];
+            float g[7][7];
+            poly_theta(c->a, sin(y), cos(y), Y[j + 1] - Y[j], th);
+            poly_series(c->M, 0.5 * (X[0] + X[1]), X[1] - X[0], th, f, g);
+            if (!(poly_bound(g) <= POLY_TOL)) return 0;
+        }
         if (cudaMalloc(&c->d_poly, bytes) != cudaSuccess) {
             cudaGetLastError();
             c->d_poly = nullptr;
@@ -1105,21 +1120,21 @@ static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
     }
     if (!c->d_poly) return 0;
     char* b = (char*)c->d_poly;
-    PolyBuild k{c->bh, c->G, {}, {}, {}, nullptr};
+    PolyBuild k{c->bh, c->G, {}, {}, {}, nullptr, 8};
     for (int q = 0; q < 3; ++q) k.c[q] = (float4*)(b + q * cells * POLY_STRIDE * 4);
     b += 3 * cells * POLY_STRIDE * 4;
     for (int q = 0; q < 2; ++q) k.t[q] = (float4*)b + q * 2 * (size_t)c->Nth;
     b += 4 * (size_t)c->Nth * 16;
     for (int q = 0; q < 2; ++q) k.ir[q] = (float2*)b + q * row;
-    k.bound = (unsigned long long*)(b + 2 * row * 8);
+    k.bound = (unsigned*)(b + 2 * row * 8);
     if (fresh) {
-        FPIC_CUDA(cudaMemsetAsync(k.bound, 0, 8, s));
-        k_poly_build<<<dim3((unsigned)((c->Nth + 127) / 128), c->Nr, 3), 128, 0, s>>>(k);
-        unsigned long long bits = 0;
-        FPIC_CUDA(cudaMemcpyAsync(&bits, k.bound, 8, cudaMemcpyDeviceToHost, s));
+        const long long cols = (c->Nth + 127) / 128;
+        while (k.rows > 1 && 3 * cols * (c->Nr / k.rows) < 8LL * c->sm_count) k.rows >>= 1;
+        FPIC_CUDA(cudaMemsetAsync(k.bound, 0, 4, s));
+        k_poly_build<<<dim3((unsigned)cols, (unsigned)((c->Nr + k.rows - 1) / k.rows), 3), 128, 0, s>>>(k);
+        float e = 0.f;
+        FPIC_CUDA(cudaMemcpyAsync(&e, k.bound, 4, cudaMemcpyDeviceToHost, s));
         FPIC_CUDA(cudaStreamSynchronize(s));
-        double e;
-        memcpy(&e, &bits, 8);
         c->poly_ok = e <= POLY_TOL;
         if (!c->poly_ok) {
             FPIC_CUDA(cudaFree(c->d_poly));
