@@ -904,6 +904,26 @@ __device__ __forceinline__ bool same_bits(double a, double b)
     return __double_as_longlong(a) == __double_as_longlong(b);
 }
 
+// The charge times the FIDO three-velocity gamma^ij u_j / Gamma, the terms
+// shared as in eval_rhs_sc_t (24 FP64 instructions besides the reciprocal's
+// and the two roots' six;
+// through the metric's components 5 more, k_dep_particle_poly 552 -> 532 us at
+// 4.0e6 particles with the sin/cos series in paired FP32).  FP64: the 1/sin^2 th of g^phph and the cancellation
+// between the two terms of U^r and U^ph want more than paired FP32's 46 bits.
+__device__ __forceinline__ void charge_flux(const BH& bh, double r, double s, double c, double ur, double ut, double up,
+                                            double Q, double& Qr, double& Qt, double& Qp)
+{
+    const double s2 = s * s, rho2 = fma(bh.a2, c * c, r * r);
+    const double gpp = rcp_nr(rho2 * s2), irho2 = gpp * s2;
+    const double alpha = rsqrt_nr(fma(bh.twoM * irho2, r, 1.0));
+    const double gurp = bh.a * irho2, g1 = fma(bh.a * s2, ur, up), iu = (alpha * alpha) * ur, tu = gpp * up;
+    const double W = fma(bh.a * ur, g1 + up, ut * ut);
+    const double QiG = Q * rsqrt_nr(fma(iu, ur, 1.0 + fma(W, irho2, tu * up)));
+    Qr = QiG * fma(gurp, g1, iu);
+    Qt = QiG * (irho2 * ut);
+    Qp = QiG * fma(gurp, ur, tu);
+}
+
 // The deposit's per-particle pass: the sin/cos of the lattices' split
 // points (angle addition from the node tables by the in-cell offset), the
 // three sub-grid lattices, their subvolumes, weights and the charge products
@@ -939,12 +959,7 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
     // sin / cos - 1 by the series (libm beyond a cell: a clamped th).
     const int jn = j0 + (__double2hiint(cn[j0]) < 0 ? 1 : 0);
     double s, c;
-    {
-        double sd, cm;
-        sincos_step(t - G.tn[jn], sd, cm);
-        s = fma(sn[jn], cm, fma(cn[jn], sd, sn[jn]));
-        c = fma(cn[jn], cm, fma(-sn[jn], sd, cn[jn]));
-    }
+    sincos_near(G.tn[jn], sn[jn], cn[jn], t, s, c);
     // ... and at the split points of the two th lattices in paired FP32 (the
     // integer lattice's is the particle's own th unless clamped)
     ff stn, ctn, sth, cth;
@@ -955,16 +970,10 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
         sincos_from_node(sn[jn], cn[jn], tn_c - G.tn[jn], stn, ctn);
     }
     sincos_from_node(sh[j1], ch[j1], th_c - G.th[j1], sth, cth);
-    // FIDO three-velocity v^i = gamma^ij u_j / Gamma, in FP64 (the 1/sin^2 th
-    // of g^pp and the cancellation between the two terms of U^r and U^ph
-    // want more than paired FP32's 46 bits)
-    Geo g;
-    geo_eval(k.bh, r, s, c, g);
-    const double ur = k.ur[p], ut = k.uth[p], up = k.uph[p];
-    const double Ur = fma(g.gurr, ur, g.gurp * up), Ut = g.gutt * ut, Up = fma(g.gurp, ur, g.gupp * up);
     const double Qd = k.w[p] * k.qm[p];
-    const double QiG = Qd * rsqrt_nr(fma(ur, Ur, fma(ut, Ut, fma(up, Up, 1.0))));
-    const ff Q = ff_cut(Qd), Qr = ff_cut(QiG * Ur), Qt = ff_cut(QiG * Ut), Qp = ff_cut(QiG * Up);
+    double Fr, Ft, Fp;
+    charge_flux(k.bh, r, s, c, k.ur[p], k.uth[p], k.uph[p], Qd, Fr, Ft, Fp);
+    const ff Q = ff_cut(Qd), Qr = ff_cut(Fr), Qt = ff_cut(Ft), Qp = ff_cut(Fp);
     const long long n = k.n_alive;
     // the split column / row are shared between the sub-grids unless clamped
     const bool share = same_bits(rn_c, rh_c) && same_bits(tn_c, th_c);
@@ -1190,9 +1199,9 @@ __device__ __forceinline__ int cell_split(const double* __restrict__ X, int m, d
 // positions' offsets in their cells.  The shares are stored as pairs of
 // floats: turning them into doubles is integer work that k_dep_cell, bound
 // by its FP64 additions, has the issue slots for.  FP64-pipe
-// bound (78 % busy, 68 instructions a particle) at 92 instead of 370
-// instructions per charge share: 1511 -> 552 us at 4.0e6 particles on
-// 512 x 512, 23.7 -> 9.4 ms at 6.4e7 on 1024 x 1024 (64 or 80 registers alike).
+// bound (61 % busy, some 57 instructions a particle) at 92 instead of 370
+// instructions per charge share: 1511 -> 532 us at 4.0e6 particles on
+// 512 x 512, 23.7 -> 9 ms at 6.4e7 on 1024 x 1024 (64 or 80 registers alike).
 __global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_constant__ DepK k,
                                                               const __grid_constant__ PolyTab T)
 {
@@ -1218,19 +1227,15 @@ __global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_const
         const double* sn = k.trig;
         const double* cn = k.trig + (G.Nth + 1);
         const int jn = j0 + (__double2hiint(cn[j0]) < 0 ? 1 : 0);
-        double sd, cm;
-        sincos_step(t - G.tn[jn], sd, cm);
-        const double s = fma(sn[jn], cm, fma(cn[jn], sd, sn[jn])), c = fma(cn[jn], cm, fma(-sn[jn], sd, cn[jn]));
-        const double ur = k.ur[p], ut = k.uth[p], up = k.uph[p];
-        Geo g;
-        geo_eval(k.bh, r, s, c, g);
-        const double Ur = fma(g.gurr, ur, g.gurp * up), Ut = g.gutt * ut, Up = fma(g.gurp, ur, g.gupp * up);
+        double s, c;
+        sincos_near(G.tn[jn], sn[jn], cn[jn], t, s, c);
         const double Qd = k.w[p] * k.qm[p];
-        const double QiG = Qd * rsqrt_nr(fma(ur, Ur, fma(ut, Ut, fma(up, Up, 1.0))));
+        double Fr, Ft, Fp;
+        charge_flux(k.bh, r, s, c, k.ur[p], k.uth[p], k.uph[p], Qd, Fr, Ft, Fp);
         Q = ff_from(Qd);
-        Qr = ff_from(QiG * Ur);
-        Qt = ff_from(QiG * Ut);
-        Qp = ff_from(QiG * Up);
+        Qr = ff_from(Fr);
+        Qt = ff_from(Ft);
+        Qp = ff_from(Fp);
     }
     const long long n = k.n_alive;
     float2* rec = (float2*)k.rec + p;
