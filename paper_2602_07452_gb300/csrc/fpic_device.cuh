@@ -2,19 +2,22 @@
 // metric and derivatives (Appendix A), the equations of motion (Eqs. p1, p2,
 // O1, O2), the Hamiltonian (Eq. Ham) and the staggered-grid field gather.
 //
-// GB300 note: FP64 issues at 1/64 of the FP32 rate, so these helpers are
-// written to minimise FP64-pipe instructions: one sincos, one reciprocal and
-// two reciprocal square roots per evaluation, fused multiply-adds throughout,
-// corrections and differences that need 46 bits or fewer in paired FP32
-// (ff.cuh), and cell location by integer comparison of the IEEE bit patterns
-// (order-preserving) instead of FP64 compares.  Against an extended-precision
-// RK4 step the pushed states' relative errors are those of the all-FP64 forms
-// (4.8e-17 to 5.1e-17 on either side, at 48 to 900 cells a side).
+// GB300 note: FP64 issues at 1/64 of the FP32 rate, so the right-hand side
+// runs on integer mantissas of 60 bits (rhs_x, xf.cuh; the FP64 form remains
+// for the Newton iteration and for arguments that have none), differences
+// that need 46 bits or fewer in paired FP32 (ff.cuh), and cell location by
+// integer comparison of the IEEE bit patterns (order-preserving) instead of
+// FP64 compares.  What is left in FP64 is written to minimise its
+// instructions: one reciprocal and two reciprocal square roots per
+// evaluation, fused multiply-adds throughout.  Against an extended-precision
+// RK4 step the pushed states' relative errors are 4.8e-17 to 5.1e-17 at 48 to
+// 900 cells a side, H's 7e-17 to 9e-17 (all in FP64 16e-17).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "ff.cuh"
+#include "xf.cuh"
 
 namespace fpic {
 
@@ -179,6 +182,13 @@ __device__ __forceinline__ void sincos_step_ff(double hd, ff& sh, ff& cm)
     sincos_step_ff(ff_from(hd), sh, cm);
 }
 
+static __device__ __noinline__ double2 sincos_far(double t)
+{
+    double2 v;
+    sincos(t, &v.x, &v.y);
+    return v;
+}
+
 // sin and cos of t from those of a nearby t0 by the angle-addition formula,
 // with sin d and cos d - 1 of d = t - t0 by their Taylor series (the first
 // omitted terms are below 1e-23 for |d| < 2^-7); farther away, sincos.  The
@@ -201,7 +211,9 @@ __device__ __forceinline__ void sincos_near(double t0, double s0, double c0, dou
         s = fma(s0, cm, fma(c0, sd, s0));
         c = fma(c0, cm, fma(-s0, sd, c0));
     } else {
-        sincos(t, &s, &c);
+        const double2 v = sincos_far(t);
+        s = v.x;
+        c = v.y;
     }
 }
 
@@ -384,19 +396,23 @@ __device__ __forceinline__ void locate(const double* __restrict__ X, const doubl
     w = ww;
 }
 
-// The same with the weight in paired FP32: the FP64 difference x - X[i]
-// (exact but for its own rounding) times the inverse spacing, to 2^-47.
+// The same with the weight in paired FP32 -- the FP64 difference x - X[i]
+// (exact but for its own rounding) times the inverse spacing, to 2^-47 -- and
+// without walking: the weight is a NaN where the estimated cell is not x's,
+// once in some ten thousand on grids even in ln r and th.  (Walks in the push's
+// main path took a twentieth of its time, and a flag as much.)
 __device__ __forceinline__ void locate_ff(const double* __restrict__ X, const float2* __restrict__ pX, int m, double x,
                                           float est, int& i, ff& w)
 {
     const long long kx = okey(x);
-    const int k = locate_walk(X, m, kx, est);
-    i = k;
-    const double x0 = __ldg(X + k);
+    const int k = max(0, min(__float2int_rd(est), m - 2));
+    const double x0 = __ldg(X + k), x1 = __ldg(X + k + 1);
     const float2 ix = __ldg(pX + k);
+    const float wrong = __int_as_float(0x7fffffff);
+    i = k;
     w = ff_mul(ff_from(x - x0), {ix.x, ix.y});
-    if (kx < okey(x0)) w = {0.f, 0.f};
-    if (kx >= okey(__ldg(X + k + 1))) w = {1.f, 0.f};
+    if (kx < okey(x0)) w = {k > 0 ? wrong : 0.f, 0.f};
+    if (kx >= okey(x1)) w = {k < m - 2 ? wrong : 1.f, 0.f};
 }
 
 struct Fields {
@@ -465,24 +481,64 @@ __device__ __forceinline__ ff ff_bits(double x)      // a pair of floats stored 
     return {__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x))};
 }
 
+// A component's value from its cell's coefficients; odd if the cell is marked
+// or a weight is not of the cell (NaNs either way).
+__device__ __forceinline__ double cell_value(double2 ab, double2 cd, ff wr, ff wt, bool& odd)
+{
+    const ff d = ff_add(ff_mul(ff_bits(ab.y), wr), ff_mul(wt, ff_add(ff_bits(cd.x), ff_mul(ff_bits(cd.y), wr))));
+    odd = odd || d.hi != d.hi;
+    return ab.x + ff_to_bits(d);
+}
+
+// gather_c where a cell is marked or an estimated cell not the right one.
+static __device__ __noinline__ void gather_far(const GridDev& G, const FieldsC& F, const Fields& raw, double r, double th,
+                                               double v[6])
+{
+    const float lr = __logf(f32_cut(r));
+    double x[4] = {r, r, 0.0, 0.0};
+    int mh;
+    theta_views(G, th, x[2], x[3], mh);
+    const double* const X[4] = {G.rn, G.rh, G.tn, G.th};
+    const float2* const pX[4] = {G.prn, G.prh, G.ptn, G.pth};
+    const int m[4] = {G.Nr + 1, G.Nr, G.Nth + 1, mh};
+    const float est[4] = {(lr - G.lr0) * G.ilr, (lr - G.lrh0) * G.ilr, (f32_cut(x[2]) - G.t0) * G.it,
+                          (f32_cut(x[3]) - G.th0) * G.it};
+    int at[4];
+    ff w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        at[q] = locate_walk(X[q], m[q], okey(x[q]), est[q]);
+        locate_ff(X[q], pX[q], m[q], x[q], (float)at[q], at[q], w[q]);
+    }
+    bool odd = false;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const bool ro = (k == 0 || k == 4 || k == 5);
+        const bool to = (k == 1 || k == 3 || k == 5);
+        const double2* q = reinterpret_cast<const double2*>(F.c[k] + 4 * ((size_t)at[ro] * G.ld + at[2 + to]));
+        v[k] = cell_value(__ldg(q), __ldg(q + 1), w[ro], w[2 + to], odd);
+    }
+    if (odd) gather(G, raw, r, th, v);
+}
+
 template <bool STAGED = false>
 __device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, const Fields& raw, double r, double th,
                                          double D[3], double B[3], const StageTile* T = nullptr)
 {
-    const float lr = __logf(f32_est(r));
-    int i0, i1, j0, j1;
-    ff wr0, wr1, wt0, wt1;
-    locate_ff(G.rn, G.prn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
-    locate_ff(G.rh, G.prh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
+    const float lr = __logf(f32_cut(r));
     double tnv, thv;
     int mh;
     theta_views(G, th, tnv, thv, mh);
-    const float tfn = f32_est(tnv), tfh = G.full ? f32_est(thv) : tfn;
+    const float tfn = f32_cut(tnv), tfh = G.full ? f32_cut(thv) : tfn;
+    int i0, i1, j0, j1;
+    ff wr0, wr1, wt0, wt1;
+    bool odd = false;
+    locate_ff(G.rn, G.prn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
+    locate_ff(G.rh, G.prh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
     locate_ff(G.tn, G.ptn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
     locate_ff(G.th, G.pth, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
     const int ld = G.ld;
     double v[6];
-    bool odd = false;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         const bool ro = (k == 0 || k == 4 || k == 5);
@@ -500,13 +556,11 @@ __device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, con
             ab = __ldg(q);
             cd = __ldg(q + 1);
         }
-        const ff b = ff_bits(ab.y);
-        odd = odd || b.hi != b.hi;
-        v[k] = ab.x + ff_to_bits(ff_add(ff_mul(b, wr), ff_mul(wt, ff_add(ff_bits(cd.x), ff_mul(ff_bits(cd.y), wr)))));
+        v[k] = cell_value(ab, cd, wr, wt, odd);
     }
     if (odd) {
         double u[6];
-        gather(G, raw, r, th, u);
+        gather_far(G, F, raw, r, th, u);
 #pragma unroll
         for (int k = 0; k < 6; ++k) v[k] = u[k];
     }
@@ -614,6 +668,89 @@ __device__ __forceinline__ void eval_rhs_sc_t(const BH& bh, const double y[6], d
         // A_0 = B0 a r (1 + cos^2 th) / rho^2   (Sec. 3.1.3)
         H = fma(-qm * B0pot * bh.a * r, fma(c, c, 1.0) * irho2, H);
     }
+}
+
+// eval_rhs_sc_t<false> out of line, for the arguments rhs_x does not take.
+static __device__ __noinline__ void eval_rhs_call(const BH& bh, const double* y, double s, double c, double qm, bool em,
+                                                  const double* D, const double* B, double B0pot, double* f, double& H)
+{
+    eval_rhs_sc_t<false>(bh, y, s, c, qm, em, D, B, B0pot, f, H, nullptr);
+}
+
+// The same right-hand side and H on integer mantissas of 63 bits (xf.cuh):
+// results rounded once.  False, with nothing set, for what those do not
+// carry: r, s not positive normal, an infinity or a NaN among the arguments, a Gamma^2
+// that is not positive.
+FPIC_HD bool rhs_x(double bh_a, double bh_a2, double bh_twoM, const double y[6], double s, double c, double qm, bool em,
+                   const double D[3], const double B[3], double B0pot, double f[6], double& H, bool want_F = true, bool want_H = true)
+{
+    // exponent fields: r and s in 1 .. 2046 and positive, the others below 2047
+    unsigned big = 0;
+    {
+        const double z[9] = {c, y[3], y[4], y[5], bh_a, bh_a2, bh_twoM, qm, B0pot};
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const unsigned h = (unsigned)(x_bits(z[i]) >> 32) & 0x7fffffffu;
+            big = big > h ? big : h;
+        }
+        if (em) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                const unsigned h = (unsigned)(x_bits(i < 3 ? D[i] : B[i - 3]) >> 32) & 0x7fffffffu;
+                big = big > h ? big : h;
+            }
+        }
+        const unsigned hr = (unsigned)(x_bits(y[0]) >> 32), hs = (unsigned)(x_bits(s) >> 32);
+        if (big >= 0x7ff00000u || hr - 0x00100000u >= 0x7fe00000u || hs - 0x00100000u >= 0x7fe00000u) return false;
+    }
+    const xf r = x_from_pos(y[0]), sx = x_from_pos(s), cx = x_from(c), ur = x_from(y[3]), ut = x_from(y[4]),
+             up = x_from(y[5]);
+    const xf a = x_from(bh_a), a2 = x_from(bh_a2), one = x_pow2(0);
+    const xf s2 = x_sqr(sx), rho2 = x_norm(x_add(x_sqr(r), x_mul(a2, x_sqr(cx))));
+    const xf t = x_rcp(x_mul(rho2, s2)), irho2 = x_norm(x_mul(t, s2));
+    const xf mi = x_mul(x_from(bh_twoM), irho2), e = x_mul(mi, r), xi = x_norm(x_add(one, e));
+    const xf alpha = x_rsqrt(xi), ixi = x_sqr(alpha), beta = x_mul(e, ixi);
+    const xf gurp = x_mul(a, irho2), as2 = x_mul(a, s2);
+    const xf g1 = x_norm(x_add(x_mul(as2, ur), up)), iu = x_mul(ixi, ur), tu = x_norm(x_mul(t, up));
+    const xf Ur = x_add(x_mul(gurp, g1), iu), Ut = x_mul(irho2, ut), Up = x_add(x_mul(gurp, ur), tu);
+    const xf W = x_norm(x_add(x_mul(x_mul(a, ur), x_add(g1, up)), x_sqr(ut))), Wi = x_mul(W, irho2);
+    const xf Q = x_add(Wi, x_mul(tu, up)), G2 = x_norm(x_add(x_mul(iu, ur), x_add(one, Q)));
+    if (G2.m <= 0) return false;
+    const xf iG = x_rsqrt(G2), aiG = x_norm(x_mul(alpha, iG));
+    const xf GA = x_mul(aiG, G2);
+    if (want_F) {
+        f[0] = x_to(x_add(x_mul(aiG, Ur), x_neg(beta)));
+        f[1] = x_to(x_mul(aiG, Ut));
+        f[2] = x_to(x_mul(aiG, Up));
+        const xf k2 = x_norm(x_mul(ixi, x_add(x_mul(iu, x_add(x_mul(aiG, ur), x_pow2(1))), GA)));
+        const xf rr = x_mul(r, irho2), xk = x_mul(mi, x_add(x_pow2(-1), x_neg(x_mul(rr, r))));
+        const xf P = x_add(Wi, x_sqr(ur)), br = x_add(x_mul(e, k2), x_neg(x_mul(aiG, P)));
+        const xf X2 = x_add(rho2, x_neg(x_mul(a, as2)));
+        xf f4 = x_mul(x_mul(sx, cx), x_add(x_mul(aiG, x_norm(x_mul(x_sqr(tu), X2))), x_mul(x_mul(a, gurp), br)));
+        xf f3 = x_add(x_mul(x_mul(aiG, rr), Q), x_mul(xk, k2));
+        f[5] = 0.0;
+        if (em) {
+            const xf q = x_from(qm), B0 = x_from(B[0]), B1 = x_from(B[1]), B2 = x_from(B[2]), D2 = x_from(D[2]);
+            const xf k = x_mul(q, alpha), kr = x_mul(k, rho2), ks = x_norm(x_mul(x_mul(q, rho2), x_mul(sx, iG)));
+            const xf cr = x_add(x_mul(Ut, B2), x_neg(x_mul(Up, B1))), ct = x_add(x_mul(Up, B0), x_neg(x_mul(Ur, B2))),
+                     cp = x_add(x_mul(Ur, B1), x_neg(x_mul(Ut, B0)));
+            const xf kx = x_mul(x_mul(k, xi), x_add(x_from(D[0]), x_neg(x_mul(as2, D2))));
+            f3 = x_add3(f3, x_mul(ks, cr), kx);
+            f4 = x_add3(f4, x_mul(kr, x_from(D[1])), x_mul(ks, ct));
+            f[5] = x_to(x_add(x_mul(s2, x_add(x_mul(kr, D2), x_neg(x_mul(a, kx)))), x_mul(ks, cp)));
+        }
+        f[3] = x_to(f3);
+        f[4] = x_to(f4);
+    }
+    if (want_H) {
+        xf h = x_add(GA, x_neg(x_mul(beta, ur)));             // alpha Gamma - beta^r u_r
+        if (x_bits(B0pot) << 1 && x_bits(qm) << 1)
+            // A_0 = B0 a r (1 + cos^2 th) / rho^2   (Sec. 3.1.3)
+            h = x_add(h, x_neg(x_mul(x_mul(x_mul(x_from(qm), x_from(B0pot)), x_mul(a, r)),
+                                     x_mul(x_add(one, x_sqr(cx)), irho2))));
+        H = x_to(h);
+    }
+    return true;
 }
 
 // Hamiltonian only (no derivatives, no force), given sin/cos of y[1].

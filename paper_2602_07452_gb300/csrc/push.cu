@@ -183,10 +183,11 @@ __device__ __forceinline__ uint32_t cell_of(const GridDev& G, double r, double t
 // looks in the block's staged field tile T first.
 template <bool JAC = false, bool STAGED = false>
 __device__ __forceinline__ void F_at_sc(const RunK& R, const double y[6], double s, double c, double qm, bool em,
-                                        double f[6], double& H, RhsJ* J = nullptr, const StageTile* T = nullptr)
+                                        double f[6], double& H, RhsJ* J = nullptr, const StageTile* T = nullptr,
+                                        bool want_F = true, bool want_H = true)
 {
     double D[3] = {0, 0, 0}, B[3] = {0, 0, 0};
-    if (em) {
+    if (em && want_F) {
         if (not_zero(R.B0field)) wald_point_sc(R.bh, R.B0field, y[0], s, c, D, B);
         else if (R.has_coef) gather_c<STAGED>(R.G, R.FC, R.F, y[0], y[1], D, B, T);
         else {
@@ -199,7 +200,23 @@ __device__ __forceinline__ void F_at_sc(const RunK& R, const double y[6], double
             }
         }
     }
-    eval_rhs_sc_t<JAC>(R.bh, y, s, c, qm, em, D, B, R.B0pot, f, H, J);
+    if (JAC) {
+        eval_rhs_sc_t<JAC>(R.bh, y, s, c, qm, em, D, B, R.B0pot, f, H, J);
+    } else if (!rhs_x(R.bh.a, R.bh.a2, R.bh.twoM, y, s, c, qm, em && want_F, D, B, R.B0pot, f, H, want_F, want_H)) {
+        const double yc[6] = {y[0], y[1], y[2], y[3], y[4], y[5]}, Dc[3] = {D[0], D[1], D[2]}, Bc[3] = {B[0], B[1], B[2]};
+        double fc[6], Hc;
+        eval_rhs_call(R.bh, yc, s, c, qm, em && want_F, Dc, Bc, R.B0pot, fc, Hc);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) f[i] = fc[i];
+        H = Hc;
+    }
+}
+
+// The same out of line, for the rarer places (one copy of the code).
+static __device__ __noinline__ void F_call(const RunK& R, const double* y, double s, double c, double qm, bool em,
+                                           double* f, double& H)
+{
+    F_at_sc<false>(R, y, s, c, qm, em, f, H);
 }
 
 // Bounded waits of the field-tile staging (polls of the mbarrier).
@@ -379,42 +396,47 @@ __device__ __forceinline__ void warp_add(long long* c, long long v, unsigned mas
 enum { STG_K1 = 0, STG_K2 = 6, STG_ACC = 12, STG_K4 = 18, STG_Z0 = 24, STG_TRIAL = 30, STG_GUESS = 36,
        STG_ROWS = 42 };
 
-// Corrector form, rejected particle in queue slot idx: its slopes k1, k2
-// (kept in shared memory, column threadIdx.x), acc, k4, z^n and the trial go
+// Corrector form, rejected particle in queue slot idx: its slopes k1, k2, k4
+// (kept in shared memory, column threadIdx.x), acc, z^n and the trial go
 // to stg at column idx (a warp's rejected lanes hold consecutive slots, so
 // the stores coalesce).  Plain copies: the arithmetic on them runs where
 // every lane of a warp has a queue entry, and every later read is
 // slot-ordered.
 __device__ __forceinline__ void trial_store(const PushK& k, unsigned long long idx, const double (*sk)[128],
-                                            const double acc[6], const double k4[6], const double z0[6],
-                                            const double zt[6])
+                                            const double (*sa)[128], const double z0[6], const double zt[6])
 {
     const int t = threadIdx.x;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
         k.stg[(size_t)(STG_K1 + i) * k.n + idx] = sk[i][t];
         k.stg[(size_t)(STG_K2 + i) * k.n + idx] = sk[6 + i][t];
-        k.stg[(size_t)(STG_ACC + i) * k.n + idx] = acc[i];
-        k.stg[(size_t)(STG_K4 + i) * k.n + idx] = k4[i];
+        k.stg[(size_t)(STG_ACC + i) * k.n + idx] = sa[i][t];
+        k.stg[(size_t)(STG_K4 + i) * k.n + idx] = sk[12 + i][t];
         k.stg[(size_t)(STG_Z0 + i) * k.n + idx] = z0[i];
         k.stg[(size_t)(STG_TRIAL + i) * k.n + idx] = zt[i];
     }
 }
 
-// Bound by the FP64 pipe (82 % busy; 64 issue slots per FP64 instruction), so
-// its cost is the count of those: 470 a particle with the reused slope, 610
-// before the reciprocals, the sin/cos series and the gather's differences
-// went to paired FP32 and integer instructions (fpic_device.cuh) and the
-// force's common factors were shared: 1.164 -> 0.951 ms per 2^20 particles
-// (ncu), 76.2 -> 61 ms for the RK4 push of 6.4e7 on 1024 x 1024.
+// Bound by its issue slots (54 % used by four warps a scheduler, the rest lost
+// to fixed latencies and instruction fetches; FP64 pipe 38 % busy): some 2600
+// instructions an evaluation, two thirds of them the right-hand side on
+// integer mantissas (rhs_x).  With that in FP64, 470 FP64 instructions a
+// particle of 64 slots each were the bound, 610 before the reciprocals, the
+// sin/cos series and the gather's differences left that pipe: per 2^20
+// charged particles 1.164 -> 0.951 -> 0.70 ms, RK4 push of 6.4e7 sorted ones on
+// 1024 x 1024 76 -> 61 -> 35 ms.  One copy of the evaluation serves all stages
+// (five would be 200 KB of code); z^n and the slopes' sum wait in shared memory
+// meanwhile.  3, 4 or 5 resident blocks, 256 threads, or warps held together by
+// barriers: within 3 %.
 // MODE 0: RK4 only.  MODE 1: hybrid (RK4 trial + test + enqueue).  MODE 2:
 // hybrid that also parks the RK4 slopes of each rejected particle
-// (corrector form of the learned guess); k1, k2 wait in shared memory
-// (12 KB per block) rather than in registers across the later stages.
+// (corrector form of the learned guess); k1, k2, k4 wait in shared memory
+// (18 KB per block) rather than in registers across the later stages.
 template <int MODE, bool BATCHED = false, bool STAGED = false>
-__global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK k)
+__global__ void __launch_bounds__(128, 4) k_explicit(const __grid_constant__ PushK k)
 {
-    __shared__ double sk[MODE == 2 ? 12 : 1][128];
+    __shared__ double sk[MODE == 2 ? 18 : 1][128];
+    __shared__ double sz[8][128], sa[6][128];      // z^n and its sin, cos th; the sum of the slopes
     __shared__ __align__(128) double s_coef[STAGED ? 6 * STAGE_TI * STAGE_TJ * 4 : 2];
     __shared__ __align__(8) uint64_t s_mbar;
     __shared__ int s_red[4 * 4 + 4];
@@ -442,7 +464,8 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
         return;
     }
     const RunK& R = BATCHED ? k.runs[run_of(k.runs, k.nruns, p)] : k.run;
-    double z0[6], kk[6], acc[6], y[6];
+    const int tx = threadIdx.x;
+    double z0[6], kk[6], y[6];
     load_state(k.P, p, z0);
     if (k.before.r) {
         k.before.r[p] = z0[0];
@@ -454,7 +477,7 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
     const double qm = k.P.qm[p];
     const bool em = (R.has_fields || not_zero(R.B0field)) && not_zero(qm);
     const double dt = k.dt, hdt = 0.5 * k.dt;
-    double Hd, s0, c0, sn, cn;
+    double s0, c0, H1;
     // k1 = F(z^n): from the slope cache when this particle's state is the
     // one stored there, else evaluated
     const bool reuse = !BATCHED && k.slope && !k.slope_cold && slope_valid(k, p, z0, qm);
@@ -470,39 +493,44 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
         s0 = __ldcs(k.slope + (size_t)SLOPE_S * k.n + p);
         c0 = __ldcs(k.slope + (size_t)SLOPE_C * k.n + p);
     } else {
-        sincos(z0[1], &s0, &c0);
-        F_at_sc<false, STAGED>(R, z0, s0, c0, qm, em, kk, Hd, nullptr, &tile);
+        const double2 v = sincos_far(z0[1]);
+        s0 = v.x;
+        c0 = v.y;
     }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        acc[i] = kk[i];
-        y[i] = fma(hdt, kk[i], z0[i]);
-        if (MODE == 2) sk[i][threadIdx.x] = kk[i];
-    }
-    sincos_near(z0[1], s0, c0, y[1], sn, cn);
-    F_at_sc<false, STAGED>(R, y, sn, cn, qm, em, kk, Hd, nullptr, &tile);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        acc[i] = fma(2.0, kk[i], acc[i]);
-        y[i] = fma(hdt, kk[i], z0[i]);
-        if (MODE == 2) sk[6 + i][threadIdx.x] = kk[i];
-    }
-    sincos_near(z0[1], s0, c0, y[1], sn, cn);
-    F_at_sc<false, STAGED>(R, y, sn, cn, qm, em, kk, Hd, nullptr, &tile);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) { acc[i] = fma(2.0, kk[i], acc[i]); y[i] = fma(dt, kk[i], z0[i]); }
-    sincos_near(z0[1], s0, c0, y[1], sn, cn);
-    F_at_sc<false, STAGED>(R, y, sn, cn, qm, em, kk, Hd, nullptr, &tile);
-    const double d6 = k.d6;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) y[i] = fma(d6, acc[i] + kk[i], z0[i]);
-    sincos_near(z0[1], s0, c0, y[1], sn, cn);
-    // H of the trial; with the slope cache the whole right-hand side at the
-    // trial point, kept for the next step if the trial is accepted
-    double H1, fy[6];
+    // Evaluations 0 to 3 are the RK4 stages; the last one, at the trial,
+    // gives its H and, with the slope cache, the right-hand side kept for the
+    // next step if the trial is accepted.  One copy of the code serves all.
     const bool keep = !BATCHED && k.slope && !k.record;
-    if (keep) F_at_sc<false, STAGED>(R, y, sn, cn, qm, em, fy, H1, nullptr, &tile);
-    else H1 = eval_H_sc(R.bh, y, sn, cn, qm, R.B0pot);
+    double sn = s0, cn = c0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) sz[i][tx] = y[i] = z0[i];
+    sz[6][tx] = s0;
+    sz[7][tx] = c0;
+    const volatile double(*vz)[128] = sz;
+#pragma unroll 1
+    for (int ev = 0; ; ++ev) {
+        if (ev > 0 || !reuse)
+            F_at_sc<false, STAGED>(R, y, sn, cn, qm, em, kk, H1, nullptr, &tile, ev < 4 || keep, ev == 4);
+        if (ev == 4) break;
+        if (MODE == 2 && ev != 2) {
+            double (*row)[128] = sk + (ev == 3 ? 12 : 6 * ev);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) row[i][tx] = kk[i];
+        }
+        if (ev == 3) {
+            const double d6 = k.d6;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) y[i] = fma(d6, sa[i][tx] + kk[i], vz[i][tx]);
+        } else {
+            const double h = ev == 2 ? dt : hdt;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                sa[i][tx] = ev == 0 ? kk[i] : fma(2.0, kk[i], sa[i][tx]);
+                if (i != 2) y[i] = fma(h, kk[i], vz[i][tx]);      // F does not depend on ph
+            }
+        }
+        sincos_near(vz[1][tx], vz[6][tx], vz[7][tx], y[1], sn, cn);
+    }
     bool accept = true;
     double Hn0 = 0.0, D00 = 1.0;     // H^n and D_0, kept for the stash of a rejected particle
     if (MODE >= 1) {
@@ -537,9 +565,14 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
         if (keep && alive) {
             if (y[1] != th_trial && !R.G.full) {   // reflected at a pole: the slope of the stored state
                 sn = -sn;                              // (a full-theta wrap changes neither F nor sin/cos)
-                F_at_sc<false, STAGED>(R, y, sn, cn, qm, em, fy, Hd, nullptr, &tile);
+                double yr[6], fr[6], Hr;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) yr[i] = y[i];
+                F_call(R, yr, sn, cn, qm, em, fr, Hr);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) kk[i] = fr[i];
             }
-            slope_store(k, p, y, qm, fy, sn, cn);
+            slope_store(k, p, y, qm, kk, sn, cn);
         }
     } else if (keep) {
         slope_drop(k, p);                 // the implicit partner sets its own entry, if any
@@ -551,6 +584,8 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
             base = atomicAdd((unsigned long long*)&k.cnt[CNT_QUEUE], (unsigned long long)__popc(rej));
         base = __shfl_sync(act, base, leader);
         if (!accept) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) z0[i] = vz[i][tx];
             const unsigned long long idx = base + __popc(rej & lanemask_lt());
             k.queue[idx] = (uint32_t)p;
             if (k.dt_imp == dt) {
@@ -564,8 +599,8 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
                 for (int i = 0; i < 6; ++i)
                     k.guess[(size_t)i * k.n + p] = __dadd_rn(z0[i], __dmul_rn(__dsub_rn(y[i], z0[i]), ratio));
             }
-            k.sc0[p] = s0;
-            k.sc0[k.n + p] = c0;
+            k.sc0[p] = vz[6][tx];
+            k.sc0[k.n + p] = vz[7][tx];
             if (k.z0s) {
 #pragma unroll
                 for (int i = 0; i < 6; ++i) k.z0s[(size_t)i * k.n + idx] = z0[i];
@@ -574,7 +609,7 @@ __global__ void __launch_bounds__(128) k_explicit(const __grid_constant__ PushK 
                 k.z0s[(size_t)8 * k.n + idx] = D00;
             }
             if (MODE == 2) {
-                trial_store(k, idx, sk, acc, kk, z0, y);
+                trial_store(k, idx, sk, sa, z0, y);
                 if (k.record) k.recS[idx] = label;
             }
         }
@@ -726,7 +761,7 @@ __global__ void __launch_bounds__(128, NEWTON ? 3 : 4) k_imr(const __grid_consta
             double sy, cy;
             sincos_near(z0[1], s0, c0, y[1], sy, cy);
             RhsJ J;
-            F_at_sc<NEWTON>(*R, y, sy, cy, qm, em, f, H, &J);
+            F_at_sc<NEWTON>(*R, y, sy, cy, qm, em, f, H, &J, nullptr, true, false);
             ++n_ev;
             double zn[6];
 #pragma unroll
@@ -853,7 +888,7 @@ __device__ bool imr_solve_serial(const PushK& k, const RunK& R, const double zs[
         for (int i = 0; i < 6; ++i) y[i] = 0.5 * (zs[i] + zk[i]);
         sincos_near(zs[1], ss, cs, y[1], sy, cy);
         RhsJ J;
-        F_at_sc<NEWTON>(R, y, sy, cy, qm, em, f, H, &J);
+        F_at_sc<NEWTON>(R, y, sy, cy, qm, em, f, H, &J, nullptr, true, false);
         ++evals;
 #pragma unroll
         for (int i = 0; i < 6; ++i) zn[i] = fma(h, f[i], zs[i]);
@@ -910,7 +945,7 @@ __device__ __forceinline__ bool implicit_end(const PushK& k, const RunK& R, long
         if (z[1] != th_new && !R.G.full) {     // reflected at a pole (a full-theta wrap changes nothing)
             double Hd;
             sn = -sn;
-            F_at_sc(R, z, sn, cn, qm, em, f, Hd);
+            F_call(R, z, sn, cn, qm, em, f, Hd);
         }
         slope_store(k, p, z, qm, f, sn, cn);
     }
@@ -943,7 +978,7 @@ __global__ void __launch_bounds__(256) k_imr_finish(const __grid_constant__ Push
         const bool keep = !BATCHED && k.slope && !all_mode && !k.record;
         double H, f[6];
         const bool em = (R.has_fields || not_zero(R.B0field)) && not_zero(qm);
-        if (keep) F_at_sc(R, z, sn, cn, qm, em, f, H);
+        if (keep) F_call(R, z, sn, cn, qm, em, f, H);
         else H = eval_H_sc(R.bh, z, sn, cn, qm, R.B0pot);
         if (k.substeps > 0 && !k.record) {
             const bool flagged = k.strag_flag[idx] != 0;
@@ -1031,7 +1066,7 @@ __global__ void __launch_bounds__(128) k_imr_substep(const __grid_constant__ Pus
         double sn, cn, H, f[6];
         sincos(z[1], &sn, &cn);
         const bool keep = !BATCHED && k.slope && !all_mode;
-        if (keep) F_at_sc(R, z, sn, cn, qm, em, f, H);
+        if (keep) F_call(R, z, sn, cn, qm, em, f, H);
         else H = eval_H_sc(R.bh, z, sn, cn, qm, R.B0pot);
         if (!implicit_end(k, R, p, z, sn, cn, qm, em, H, f, keep, its_out)) ++n_rm;
     }
