@@ -670,19 +670,22 @@ __device__ __forceinline__ void eval_rhs_sc_t(const BH& bh, const double y[6], d
     }
 }
 
-// eval_rhs_sc_t<false> out of line, for the arguments rhs_x does not take.
+// eval_rhs_sc_t out of line, for the arguments rhs_x does not take.
+template <bool JAC>
 static __device__ __noinline__ void eval_rhs_call(const BH& bh, const double* y, double s, double c, double qm, bool em,
-                                                  const double* D, const double* B, double B0pot, double* f, double& H)
+                                                  const double* D, const double* B, double B0pot, double* f, double& H,
+                                                  RhsJ* J)
 {
-    eval_rhs_sc_t<false>(bh, y, s, c, qm, em, D, B, B0pot, f, H, nullptr);
+    eval_rhs_sc_t<JAC>(bh, y, s, c, qm, em, D, B, B0pot, f, H, J);
 }
 
 // The same right-hand side and H on integer mantissas of 63 bits (xf.cuh):
 // results rounded once.  False, with nothing set, for what those do not
 // carry: r, s not positive normal, an infinity or a NaN among the arguments, a Gamma^2
 // that is not positive.
+template <bool JAC = false>
 FPIC_HD bool rhs_x(double bh_a, double bh_a2, double bh_twoM, const double y[6], double s, double c, double qm, bool em,
-                   const double D[3], const double B[3], double B0pot, double f[6], double& H, bool want_F = true, bool want_H = true)
+                   const double D[3], const double B[3], double B0pot, double f[6], double& H, bool want_F = true, bool want_H = true, RhsJ* J = nullptr)
 {
     // exponent fields: r and s in 1 .. 2046 and positive, the others below 2047
     unsigned big = 0;
@@ -717,6 +720,16 @@ FPIC_HD bool rhs_x(double bh_a, double bh_a2, double bh_twoM, const double y[6],
     const xf Q = x_add(Wi, x_mul(tu, up)), G2 = x_norm(x_add(x_mul(iu, ur), x_add(one, Q)));
     if (G2.m <= 0) return false;
     const xf iG = x_rsqrt(G2), aiG = x_norm(x_mul(alpha, iG));
+    if (JAC) {
+        J->U[0] = x_to(Ur); J->U[1] = x_to(Ut); J->U[2] = x_to(Up);
+        J->iG = x_to(iG); J->aiG = x_to(aiG);
+        J->gurr = x_to(x_add(x_mul(x_mul(a, as2), irho2), ixi)); J->gurp = x_to(gurp);
+        J->gutt = x_to(irho2); J->gupp = x_to(t);
+        // no field: the force terms of the Newton matrix vanish (set, not left undefined)
+        J->ks = 0.0;
+        J->B[0] = J->B[1] = J->B[2] = 0.0;
+        J->cx[0] = J->cx[1] = J->cx[2] = 0.0;
+    }
     const xf GA = x_mul(aiG, G2);
     if (want_F) {
         f[0] = x_to(x_add(x_mul(aiG, Ur), x_neg(beta)));
@@ -734,6 +747,11 @@ FPIC_HD bool rhs_x(double bh_a, double bh_a2, double bh_twoM, const double y[6],
             const xf k = x_mul(q, alpha), kr = x_mul(k, rho2), ks = x_norm(x_mul(x_mul(q, rho2), x_mul(sx, iG)));
             const xf cr = x_add(x_mul(Ut, B2), x_neg(x_mul(Up, B1))), ct = x_add(x_mul(Up, B0), x_neg(x_mul(Ur, B2))),
                      cp = x_add(x_mul(Ur, B1), x_neg(x_mul(Ut, B0)));
+            if (JAC) {
+                J->ks = x_to(ks);
+                J->B[0] = B[0]; J->B[1] = B[1]; J->B[2] = B[2];
+                J->cx[0] = x_to(cr); J->cx[1] = x_to(ct); J->cx[2] = x_to(cp);
+            }
             const xf kx = x_mul(x_mul(k, xi), x_add(x_from(D[0]), x_neg(x_mul(as2, D2))));
             f3 = x_add3(f3, x_mul(ks, cr), kx);
             f4 = x_add3(f4, x_mul(kr, x_from(D[1])), x_mul(ks, ct));

@@ -200,12 +200,12 @@ __device__ __forceinline__ void F_at_sc(const RunK& R, const double y[6], double
             }
         }
     }
-    if (JAC) {
-        eval_rhs_sc_t<JAC>(R.bh, y, s, c, qm, em, D, B, R.B0pot, f, H, J);
-    } else if (!rhs_x(R.bh.a, R.bh.a2, R.bh.twoM, y, s, c, qm, em && want_F, D, B, R.B0pot, f, H, want_F, want_H)) {
+    if (!rhs_x<JAC>(R.bh.a, R.bh.a2, R.bh.twoM, y, s, c, qm, em && want_F, D, B, R.B0pot, f, H, want_F, want_H, J)) {
         const double yc[6] = {y[0], y[1], y[2], y[3], y[4], y[5]}, Dc[3] = {D[0], D[1], D[2]}, Bc[3] = {B[0], B[1], B[2]};
         double fc[6], Hc;
-        eval_rhs_call(R.bh, yc, s, c, qm, em && want_F, Dc, Bc, R.B0pot, fc, Hc);
+        RhsJ Jc;
+        eval_rhs_call<JAC>(R.bh, yc, s, c, qm, em && want_F, Dc, Bc, R.B0pot, fc, Hc, &Jc);
+        if (JAC) *J = Jc;
 #pragma unroll
         for (int i = 0; i < 6; ++i) f[i] = fc[i];
         H = Hc;
