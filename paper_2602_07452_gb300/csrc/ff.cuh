@@ -33,6 +33,13 @@ __device__ __forceinline__ ff ff_fast2(float a, float b)
     return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
+// a + b of any two floats: exact.
+__device__ __forceinline__ ff ff_sum2(float a, float b)
+{
+    const float s = __fadd_rn(a, b), v = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v))};
+}
+
 __device__ __forceinline__ ff ff_of(float a)
 {
     return {a, 0.f};

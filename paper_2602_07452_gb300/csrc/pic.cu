@@ -1303,9 +1303,10 @@ __device__ __forceinline__ double sel_bits(bool p, double a, double b)
 
 // PAIRS: the shares are pairs of floats (k_dep_particle_poly).  The high
 // floats are summed in FP64, the low ones (2^-24 of them) in FP32: 2^-48 of the
-// sum of |share|, under the shares' own rounding, at one FP64 addition a
-// share (198 -> 235 us at 4.0e6 particles in 262144 cells, for 16 conversions a
-// particle less in the FP64-bound kernel before it).
+// sum of |share|, under the shares' own rounding, at one FP64 addition to
+// four shares, after a tree of exact FP32 two-sums whose errors join the low
+// floats (one addition a share: deposit of 4.0e6 particles on 512^2 1136 -> 1108
+// us); the 16 conversions a particle are not in the FP64-bound kernel before it.
 template <bool PAIRS>
 __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* __restrict__ rec,
                                                                    const uint32_t* __restrict__ code,
@@ -1339,18 +1340,40 @@ __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* 
         cw[lane] = cd;
         __syncwarp();
         const int kend = (int)(cnt + 1) >> 1;
+        if (PAIRS) {
+            // four particles to an addition: their high floats by a tree of
+            // exact two-sums, whose errors join the low floats
+            for (int k = 0; k < kend; k += 4) {
+                float h[2][4], l[2] = {0.f, 0.f};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int pp = 2 * (k + u) + par;      // particles past the group's end hold zeros
+                    const double y = v[row * DEP_CELL_LD + pp];
+                    const float2 f = make_float2(__uint_as_float((unsigned)__double2loint(y)),
+                                                 __uint_as_float((unsigned)__double2hiint(y)));
+                    const bool bit = ((cw[pp] >> bsh) & bmask) != 0u;
+                    h[0][u] = bit ? 0.f : f.x;
+                    h[1][u] = bit ? f.x : 0.f;
+                    l[0] += bit ? 0.f : f.y;
+                    l[1] += bit ? f.y : 0.f;
+                }
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    const ff a = ff_sum2(h[m][0], h[m][1]), c = ff_sum2(h[m][2], h[m][3]), t = ff_sum2(a.hi, c.hi);
+                    l[m] += (a.lo + c.lo) + t.lo;
+                    h[m][0] = t.hi;
+                }
+                acc0 += f2d_bits(h[0][0]);
+                acc1 += f2d_bits(h[1][0]);
+                lo0 += l[0];
+                lo1 += l[1];
+            }
+            continue;
+        }
         for (int k = 0; k < kend; ++k) {
             const int pp = 2 * k + par;     // a particle past the group's end holds zeros
-            double y = v[row * DEP_CELL_LD + pp];
+            const double y = v[row * DEP_CELL_LD + pp];
             const bool bit = ((cw[pp] >> bsh) & bmask) != 0u;
-            if (PAIRS) {
-                const float2 f = make_float2(__uint_as_float((unsigned)__double2loint(y)),
-                                             __uint_as_float((unsigned)__double2hiint(y)));
-                y = f2d_bits(f.x);
-                const float s = (bit ? lo1 : lo0) + f.y;
-                lo1 = bit ? s : lo1;
-                lo0 = bit ? lo0 : s;
-            }
             const double s = sel_bits(bit, acc1, acc0) + y;
             acc1 = sel_bits(bit, s, acc1);
             acc0 = sel_bits(bit, acc0, s);
