@@ -1189,11 +1189,11 @@ def run_div_clean(device, grid_n=1024, n_iter=500, reps=3):
             "sweep_achieved_gbs": bytes_sweep * n_iter / t / 1e9 if n_iter else None}
 
 
-# Per full FDTD step (stages 1 and 2, no particles), the grid arrays each
-# kernel reads or writes once, counted per component: the level averages
-# (9), E twice (2 x 24 with the metric tables), B^{n+3/2} and B^{n+2} (15,
-# 12), H twice (2 x 24), D^{n+2} and D^{n+5/2} with the sources (26, 19).
-FDTD_ARRAY_PASSES = 9 + 24 + 15 + 24 + 12 + 24 + 26 + 24 + 19
+# Per full FDTD step (stages 1 and 2, no particles), the grid arrays each of
+# the four launches reads or writes once, counted per component, metric
+# coefficients included: B^{n+3/2} (30), B^{n+2} with E (29), D^{n+2} (40) and
+# D^{n+5/2} with H (39).
+FDTD_ARRAY_PASSES = 30 + 29 + 40 + 39
 
 
 def run_vacuum_wald(device, Nr=4196, Nth=1024, steps=20, warmup=3):
