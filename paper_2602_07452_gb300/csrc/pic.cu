@@ -1840,8 +1840,8 @@ namespace fpic {
 // thread per particle, and k_cdep_cell adds the records up.  FP64-pipe
 // bound: with one warp per cell, its 30 partials by every lane and a
 // reduction tree, a cell of 16 particles left half the lanes idle:
-// 4.0e6 particles on 512 x 512 3604 us, now 842 (particles, 86 % of the pipe,
-// 113 FP64 operations each) + 188 (cells).
+// 4.0e6 particles on 512 x 512 3604 us, then 842 (particles, 86 % of the pipe,
+// 113 FP64 operations each; some 435 with 43, see phdot_x) + 188 (cells).
 enum { CD_Q = 0, CD_P = 9, CD_R = 18, CD_T = 24, CD_SLOTS = 30 };
 // rows of a move inside its cell: Q and P at node (x, y) in row x + 2 y, the r
 // face's charge at th node y, the th face's at r node x
