@@ -232,49 +232,65 @@ FPIC_HD unsigned x_float_bits(float f)
 #endif
 }
 
+// The FP32 estimate's 24 significant bits, for a value of at least 1/2 and below
+// 1.  The hardware's may fall an ulp or two outside (its documented error is an
+// ulp for the reciprocal and 2^-22.9 for the root): held to the ends, which are
+// as good an estimate there.
+FPIC_HD unsigned x_est24(float y)
+{
+    unsigned u = x_float_bits(y);
+    u = u < 0x3f7fffffu ? u : 0x3f7fffffu;
+    u = u > 0x3f000000u ? u : 0x3f000000u;
+    return (u & 0x7fffffu) | 0x800000u;
+}
+
 // 1/a for a > 0: with X = m / 2^61 in [1, 2), the FP32 estimate Y of 1/X in 31
 // fraction bits, e = 1 - X Y exact to 2^-61 and Y (1 + e + e^2): e is below
-// 2^-21, the next term below 2^-63.
+// 2^-21, the next term below 2^-63.  a normalised, y the estimate of 1 / x_rcp_arg(a).
+FPIC_HD float x_rcp_arg(xf a)
+{
+    return x_float(0x3f800000u | (((unsigned)x_hi((long long)((unsigned long long)a.m << 1)) >> 7) & 0x7fffffu));
+}
+
+FPIC_HD xf x_rcp_est(xf a, float y)
+{
+    const unsigned long long m = (unsigned long long)a.m << 1;
+    const int h = x_hi((long long)m);
+    const unsigned Y = x_est24(y) << 7;
+    const long long p = (long long)h * (int)Y + (long long)x_umulhi((unsigned)m, Y);
+    const long long E = 0x2000000000000000ll - p;                       // e 2^61
+    const int e12 = (int)(E >> 12), t = x_mulhi(e12, e12);              // e 2^49, e^2 2^66
+    const int t2 = x_mulhi(t << 6, (int)Y) >> 11;                       // Y e^2 2^60
+    const long long r = ((long long)Y << 29) + (x_scale32(E, Y) + t2);  // 2^60 / X
+    return {r << 1, -122 - a.e};
+}
+
 FPIC_HD xf x_rcp(xf a)
 {
     a = x_norm(a);
-    const unsigned long long m = (unsigned long long)a.m << 1;
-    const int h = x_hi((long long)m);
-    const float x = x_float(0x3f800000u | (((unsigned)h >> 7) & 0x7fffffu));
+    const float x = x_rcp_arg(a);
     float y;
 #ifdef __CUDA_ARCH__
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
 #else
     y = 1.f / x;
 #endif
-    unsigned u = x_float_bits(y);
-    u = u < 0x3f7fffffu ? u : 0x3f7fffffu;                              // below 1
-    const unsigned Y = ((u & 0x7fffffu) | 0x800000u) << 7;
-    const long long p = (long long)h * (int)Y + (long long)x_umulhi((unsigned)m, Y);
-    const long long E = 0x2000000000000000ll - p;                       // e 2^61
-    const int e12 = (int)(E >> 12), t = x_mulhi(e12, e12);              // e 2^49, e^2 2^66
-    const int t2 = x_mulhi(t << 8, (int)Y) >> 13;                       // Y e^2 2^60
-    const long long r = ((long long)Y << 29) + (x_scale32(E, Y) + t2);  // 2^60 / X
-    return {r << 1, -122 - a.e};
+    return x_rcp_est(a, y);
 }
 
 // 1/sqrt(a) for a > 0 in the same way: X in [1, 4) (an even exponent), e = 1 -
 // X Y^2 with Y of 24 bits (Y^2 exact), Y (1 + e/2 + 3 e^2/8).
-FPIC_HD xf x_rsqrt(xf a)
+FPIC_HD float x_rsqrt_arg(xf a)
 {
-    a = x_norm(a);
+    const unsigned odd = (unsigned)(a.e + 61) & 1u;
+    return x_float(x_float_bits(x_rcp_arg(a)) + (odd << 23));
+}
+
+FPIC_HD xf x_rsqrt_est(xf a, float y)
+{
     const unsigned long long m = (unsigned long long)a.m << 1;
     const int h = x_hi((long long)m), E0 = a.e + 61, odd = E0 & 1;
-    const float x = x_float((0x3f800000u | (((unsigned)h >> 7) & 0x7fffffu)) + ((unsigned)odd << 23));
-    float y;
-#ifdef __CUDA_ARCH__
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-#else
-    y = (float)(1.0 / __builtin_sqrt((double)x));
-#endif
-    unsigned u = x_float_bits(y);
-    u = u < 0x3f7fffffu ? u : 0x3f7fffffu;
-    const unsigned y24 = (u & 0x7fffffu) | 0x800000u, Y = y24 << 7;
+    const unsigned y24 = x_est24(y), Y = y24 << 7;
     const long long y2 = (long long)((unsigned long long)y24 * y24 << 14);   // Y^2 2^62
     const int hy = x_hi(y2), ly = (int)((unsigned)y2 >> 1), la = (int)((unsigned)m >> 1);
     const long long c = x_mulhi(h, ly) + x_mulhi(hy, la);
@@ -284,6 +300,19 @@ FPIC_HD xf x_rsqrt(xf a)
     const int t2 = x_mulhi((3 * t) << 4, (int)Y) >> 12;                      // 3/8 Y e^2 2^60
     const long long r = ((long long)Y << 29) + (x_scale32(E, Y) + t2);
     return {r << 1, -61 - (E0 >> 1)};
+}
+
+FPIC_HD xf x_rsqrt(xf a)
+{
+    a = x_norm(a);
+    const float x = x_rsqrt_arg(a);
+    float y;
+#ifdef __CUDA_ARCH__
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+#else
+    y = (float)(1.0 / __builtin_sqrt((double)x));
+#endif
+    return x_rsqrt_est(a, y);
 }
 
 }  // namespace fpic
