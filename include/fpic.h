@@ -394,7 +394,7 @@ int fpic_probe_fp64(double *gflops_out, int reps);
  *     the hardware estimate and one Goldschmidt step (2^-39.6 measured).
  *     Lattice points, weights and node shares are the same; results differ
  *     by rounding only (1e-13 relative and below on the deposited sources).
- *     With 1, grids fine enough (about 200 cells a side over two decades in
+ *     With 1, grids fine enough (120 to 240 cells a side over two decades in
  *     r) take the same trapezoid sums from a degree-5 polynomial of
  *     sqrt(gamma) per cell, tabulated by the first fpic_deposit on a grid
  *     (336 bytes a cell; that call waits for the stream once, and uses the

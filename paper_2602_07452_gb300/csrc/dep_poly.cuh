@@ -22,13 +22,14 @@
 namespace fpic {
 
 constexpr int POLY_STRIDE = 28;      // floats of a cell (25 used): seven 16-byte loads
-// The polynomial is used where poly_bound, the largest error of a node share
-// over every cell of the grid, stays below POLY_TOL = 2^-45.5: the lattice
-// form's own square root is good to 2^-44.5.  Grids uniform in ln r and th from
-// 0.9 r_+ to 50 M meet it from about 200 cells a side (there the shares
-// differ from an extended-precision quadrature by at most 7e-16 in 200 random
-// cells, 2e-17 at 512); coarser ones keep the lattices.
-constexpr double POLY_TOL = 2e-14;
+// The polynomial is used where poly_bound, the largest relative error of a node
+// share over every cell of the grid (those inside the horizon too), stays below
+// POLY_TOL.  Grids uniform in ln r and th from 0.9 r_+ to 50 M meet it from 122 (a =
+// 0.5), 182 (0.9) or 222 (0.99) cells a side.  There a share down to 1e-6 is off by
+// 5e-15 to 7e-15 of itself (rms over a million; at most 1.1e-13), from the lattices
+// by 1.1e-14 (1.0e-13); at five times the bound the polynomial's tail is the longer
+// one (0.1 % of the shares beyond 7e-14, of the lattices' 5.4e-14).
+constexpr double POLY_TOL = 1.3e-13;
 constexpr double POLY_MAX_DTH = 0.03, POLY_MAX_TAU = 4.0;     // limits of the sin th series
 
 // What a th cell of centre yc (sin, cos given) and size dy brings to its cells'
@@ -118,19 +119,17 @@ __host__ __device__ inline void poly_series(double M, double x, double dx, const
         }
 }
 
-// Bound on the error of a node share (a fraction of the cell): the terms of
-// degree 6 that are left out and the FP32 rounding of those of degree 3 to 5,
-// an interval's share of a cell's moment of xi^m being at most 2^-m / (2 m + 1).
+// Bound on the relative error of a node share: the terms of degree 6 that are
+// left out and the FP32 rounding of those of degree 3 to 5, at the cell's
+// corners (where the interval of a small share lies).
 __host__ __device__ inline float poly_bound(const float f[7][7])
 {
     float e = 0.f;
 #pragma unroll
     for (int d = 3; d <= 6; ++d)
 #pragma unroll
-        for (int m = 0; m <= d; ++m) {
-            const int n = d - m;
-            e += fabsf(f[m][n]) * (d == 6 ? 1.f : 5.9604644775390625e-8f) / (float)((1 << d) * (2 * m + 1) * (2 * n + 1));
-        }
+        for (int m = 0; m <= d; ++m)
+            e += fabsf(f[m][d - m]) * (d == 6 ? 1.f : 5.9604644775390625e-8f) / (float)(1 << d);
     return e;
 }
 
@@ -184,6 +183,17 @@ __device__ __forceinline__ ff ff_addf(ff a, float b)      // a + b, |b| far belo
     return {a.hi, __fadd_rn(a.lo, b)};
 }
 
+// a b of pairs whose low floats carry FP32 terms of their own, far above 2^-24 of
+// the high ones: their product counts (R_1 E_1 and R_2 E_2: up to 10^-12 of the sum
+// on grids of 150 cells a side).
+__device__ __forceinline__ ff ff_mul_lo(ff a, ff b)
+{
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.lo, b.lo, __fmaf_rn(a.hi, b.hi, -p));
+    e = __fmaf_rn(a.hi, b.lo, e);
+    return {p, __fmaf_rn(a.lo, b.hi, e)};
+}
+
 // d2_2, d2_6: dth^2 / 2 and dth^2 / 6.  The cubic term of sin th, up to 10^-6
 // of the sum in the cells at the poles, is paired too.
 __device__ __forceinline__ void moments_th(const Mom M[2], ff tau, ff d2_2, ff d2_6, MomT E[2])
@@ -231,8 +241,8 @@ __device__ __forceinline__ void poly_shares(const float4* __restrict__ c, const 
         for (int g = 0; g < 2; ++g) {
             const MomT& e = Y[g];
             // sum - 1 = e0 + R0 + R0 e0 + R1 e1 + R2 e2 + ...
-            ff S = ff_add(ff_add(e.e0, R0), ff_add(ff_mul(R0, e.e0), ff_mul(R1, e.e1)));
-            S = ff_add(S, ff_addf(ff_mul(R2, e.e2), fmaf(R3, e.e3, fmaf(R4, e.e4, f05 * e.e5))));
+            ff S = ff_add(ff_add(e.e0, R0), ff_add(ff_mul(R0, e.e0), ff_mul_lo(R1, e.e1)));
+            S = ff_add(S, ff_addf(ff_mul_lo(R2, e.e2), fmaf(R3, e.e3, fmaf(R4, e.e4, f05 * e.e5))));
             const ff area = ff_mul(m.len, e.len);
             const ff v = ff_add(area, ff_mul(area, S));
             V[h + 2 * g] = ff_fast2(v.hi, v.lo);         // normalized: S carries FP32 terms in its lo
