@@ -1560,19 +1560,28 @@ __global__ void k_field_coef(const __grid_constant__ CoefJobs jobs)
     }
 }
 
-static int launch_coefs(const std::vector<CoefJob>& v, cudaStream_t s)
+struct CoefTodo {
+    fpic_ctx* c;
+    CoefJob job;
+};
+
+// A context counts its coefficients as built from these fields (fcoef_src) only
+// once their launch is in: a batch that fails before drops the work.
+static int launch_coefs(const std::vector<CoefTodo>& v, cudaStream_t s)
 {
     for (size_t b = 0; b < v.size(); b += COEF_JOBS) {
         CoefJobs J{};
         const int m = (int)(v.size() - b < COEF_JOBS ? v.size() - b : COEF_JOBS);
         int Nr = 0, Nth = 0;
         for (int q = 0; q < m; ++q) {
-            J.job[q] = v[b + q];
+            J.job[q] = v[b + q].job;
             Nr = J.job[q].Nr > Nr ? J.job[q].Nr : Nr;
             Nth = J.job[q].Nth > Nth ? J.job[q].Nth : Nth;
         }
         k_field_coef<<<dim3((unsigned)((Nth + 1 + 127) / 128), Nr + 1, m), 128, 0, s>>>(J);
         FPIC_CUDA(cudaGetLastError());
+        for (int q = 0; q < m; ++q)
+            for (int i = 0; i < 6; ++i) v[b + q].c->fcoef_src[i] = v[b + q].job.f[i];
     }
     return 0;
 }
@@ -1582,7 +1591,7 @@ static int launch_coefs(const std::vector<CoefJob>& v, cudaStream_t s)
 // adds the work to it instead, for the caller's launch_coefs) and points
 // R at it.
 static int field_coefs(fpic_ctx* c, const double* const fields[6], RunK& R, cudaStream_t s,
-                       std::vector<CoefJob>* batch = nullptr)
+                       std::vector<CoefTodo>* batch = nullptr)
 {
     const size_t sz = (size_t)(c->Nr + 1) * c->ld;
     const size_t bytes = 6 * 4 * sz * sizeof(double);
@@ -1598,11 +1607,11 @@ static int field_coefs(fpic_ctx* c, const double* const fields[6], RunK& R, cuda
     for (int i = 0; i < 6; ++i) same = same && c->fcoef_src[i] == fields[i];
     if (!same) {
         CoefJob job{c->Nr, c->Nth, c->ld, c->G.full, {}, out, sz};
-        for (int i = 0; i < 6; ++i) c->fcoef_src[i] = job.f[i] = fields[i];
+        for (int i = 0; i < 6; ++i) job.f[i] = fields[i];
         if (batch) {
-            batch->push_back(job);
+            batch->push_back({c, job});
         } else {
-            const int rc = launch_coefs({job}, s);
+            const int rc = launch_coefs({{c, job}}, s);
             if (rc) return rc;
         }
     }
@@ -2845,7 +2854,7 @@ static int push_batched(const fpic_run* runs, int nruns, fpic_mlp* m, fpic_parti
                : ensure_scratch(c, (size_t)nn * (8 * sizeof(double) + 3 * sizeof(uint32_t) + 1) + 256);
     if (rc) return rc;
     std::vector<RunK> tab(nruns);
-    std::vector<CoefJob> jobs;
+    std::vector<CoefTodo> jobs;
     for (int i = 0; i < nruns; ++i) {
         const fpic_run& r = runs[i];
         RunK R{};
