@@ -17,6 +17,8 @@
 // paired FP32, the others (below 2^-22 of the sum where the table is used)
 // in FP32.
 #pragma once
+#include <math.h>
+
 #include "ff.cuh"
 
 namespace fpic {
@@ -131,6 +133,14 @@ __host__ __device__ inline float poly_bound(const float f[7][7])
         for (int m = 0; m <= d; ++m)
             e += fabsf(f[m][d - m]) * (d == 6 ? 1.f : 5.9604644775390625e-8f) / (float)(1 << d);
     return e;
+}
+
+// The larger of two bounds, b possibly a NaN (a series past the range of its
+// numbers): infinite then, above every tolerance.
+__host__ __device__ inline float poly_worst(float e, float b)
+{
+    if (!(b <= 3.402823466e38f)) return HUGE_VALF;
+    return b > e ? b : e;
 }
 
 struct PolyTab {

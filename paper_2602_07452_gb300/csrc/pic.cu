@@ -1019,9 +1019,8 @@ __global__ void __launch_bounds__(256) k_dep_particle_ff(DepK k)
 
 // Builds the cells' polynomials (sub-grid blockIdx.z; a thread walks `rows`
 // cells down one th column, whose trigonometry it takes once), the 1-D
-// tables and the largest bound over the cells (as the bits of a non-negative
-// float; a NaN exceeds every tolerance).  Once per grid, about 60 FP64
-// operations a cell.
+// tables and the largest bound over the cells (poly_worst, as the bits of a
+// non-negative float).  Once per grid, about 60 FP64 operations a cell.
 struct PolyBuild {
     BH bh;
     GridDev G;
@@ -1058,8 +1057,7 @@ __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ Poly
             double f[4][4];
             float q[7][7];
             poly_series(k.bh.M, 0.5 * (X[i] + X[i + 1]), dx, th, f, q);
-            e = fmaxf(e, poly_bound(q));
-            if (!(e == e)) e = INFINITY;
+            e = poly_worst(e, poly_bound(q));
             float4* c = k.c[sg] + ((size_t)i * G.Nth + j) * (POLY_STRIDE / 4);
             const float2 f10 = pair_of(f[1][0]), f01 = pair_of(f[0][1]), f20 = pair_of(f[2][0]),
                          f11 = pair_of(f[1][1]), f02 = pair_of(f[0][2]);
