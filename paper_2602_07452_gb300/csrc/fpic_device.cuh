@@ -679,15 +679,16 @@ static __device__ __noinline__ void eval_rhs_call(const BH& bh, const double* y,
     eval_rhs_sc_t<JAC>(bh, y, s, c, qm, em, D, B, B0pot, f, H, J);
 }
 
-// The same right-hand side and H on integer mantissas of 63 bits (xf.cuh):
+// The same right-hand side and H on integer mantissas of 60 bits (xf.cuh):
 // results rounded once.  False, with nothing set, for what those do not
-// carry: r, s not positive normal, an infinity or a NaN among the arguments, a Gamma^2
-// that is not positive.
+// carry: r not positive normal, s not normal (of either sign: half of the
+// full-theta domain has sin th < 0), an infinity or a NaN among the arguments, a
+// Gamma^2 that is not positive.
 template <bool JAC = false>
 FPIC_HD bool rhs_x(double bh_a, double bh_a2, double bh_twoM, const double y[6], double s, double c, double qm, bool em,
                    const double D[3], const double B[3], double B0pot, double f[6], double& H, bool want_F = true, bool want_H = true, RhsJ* J = nullptr)
 {
-    // exponent fields: r and s in 1 .. 2046 and positive, the others below 2047
+    // exponent fields: r and s in 1 .. 2046, r positive, the others below 2047
     unsigned big = 0;
     {
         const double z[9] = {c, y[3], y[4], y[5], bh_a, bh_a2, bh_twoM, qm, B0pot};
@@ -703,10 +704,10 @@ FPIC_HD bool rhs_x(double bh_a, double bh_a2, double bh_twoM, const double y[6],
                 big = big > h ? big : h;
             }
         }
-        const unsigned hr = (unsigned)(x_bits(y[0]) >> 32), hs = (unsigned)(x_bits(s) >> 32);
+        const unsigned hr = (unsigned)(x_bits(y[0]) >> 32), hs = (unsigned)(x_bits(s) >> 32) & 0x7fffffffu;
         if (big >= 0x7ff00000u || hr - 0x00100000u >= 0x7fe00000u || hs - 0x00100000u >= 0x7fe00000u) return false;
     }
-    const xf r = x_from_pos(y[0]), sx = x_from_pos(s), cx = x_from(c), ur = x_from(y[3]), ut = x_from(y[4]),
+    const xf r = x_from_pos(y[0]), sx = x_from(s), cx = x_from(c), ur = x_from(y[3]), ut = x_from(y[4]),
              up = x_from(y[5]);
     const xf a = x_from(bh_a), a2 = x_from(bh_a2), one = x_pow2(0);
     const xf s2 = x_sqr(sx), rho2 = x_norm(x_add(x_sqr(r), x_mul(a2, x_sqr(cx))));
