@@ -330,12 +330,11 @@ extern "C" int fpic_set_grid(fpic_ctx* c, int Nr, int Nth, const double* rn, con
     FPIC_CUDA(cudaSetDevice(c->device));
     // the half-th list carries one more node, th[Nth] = th[0] + (tn[Nth] - tn[0]):
     // the upper end of the full-theta wrap cell (unused in the half-theta domain)
-    const size_t tot = 3 * ((size_t)(Nr + 1) + Nr + (Nth + 1) + (Nth + 1));    // nodes, 1/spacing, the same as pairs of floats
+    const size_t tot = 2 * ((size_t)(Nr + 1) + Nr + (Nth + 1) + (Nth + 1));    // nodes, 1/spacing
     std::vector<double> h(tot);
     double* p = h.data();
     size_t o_rn = 0, o_rh = o_rn + Nr + 1, o_tn = o_rh + Nr, o_th = o_tn + Nth + 1;
     size_t o_irn = o_th + Nth + 1, o_irh = o_irn + Nr + 1, o_itn = o_irh + Nr, o_ith = o_itn + Nth + 1;
-    size_t o_prn = o_ith + Nth + 1, o_prh = o_prn + Nr + 1, o_ptn = o_prh + Nr, o_pth = o_ptn + Nth + 1;
     memcpy(p + o_rn, rn, (Nr + 1) * sizeof(double));
     memcpy(p + o_rh, rh, Nr * sizeof(double));
     memcpy(p + o_tn, tn, (Nth + 1) * sizeof(double));
@@ -349,16 +348,6 @@ extern "C" int fpic_set_grid(fpic_ctx* c, int Nr, int Nth, const double* rn, con
     inv(rh, Nr, p + o_irh);
     inv(tn, Nth + 1, p + o_itn);
     inv(p + o_th, Nth + 1, p + o_ith);
-    auto pairs = [](const double* iX, int m, double* out) {
-        for (int i = 0; i < m; ++i) {
-            const float f[2] = {(float)iX[i], (float)(iX[i] - (double)(float)iX[i])};
-            memcpy(out + i, f, sizeof f);
-        }
-    };
-    pairs(p + o_irn, Nr + 1, p + o_prn);
-    pairs(p + o_irh, Nr, p + o_prh);
-    pairs(p + o_itn, Nth + 1, p + o_ptn);
-    pairs(p + o_ith, Nth + 1, p + o_pth);
     retire(c, (void**)&c->d_nodes);
     FPIC_CUDA(cudaMalloc(&c->d_nodes, tot * sizeof(double)));
     FPIC_CUDA(cudaMemcpy(c->d_nodes, p, tot * sizeof(double), cudaMemcpyHostToDevice));
@@ -370,8 +359,6 @@ extern "C" int fpic_set_grid(fpic_ctx* c, int Nr, int Nth, const double* rn, con
     G.ld = Nth + 1;
     G.rn = d + o_rn; G.rh = d + o_rh; G.tn = d + o_tn; G.th = d + o_th;
     G.irn = d + o_irn; G.irh = d + o_irh; G.itn = d + o_itn; G.ith = d + o_ith;
-    G.prn = (const float2*)(d + o_prn); G.prh = (const float2*)(d + o_prh);
-    G.ptn = (const float2*)(d + o_ptn); G.pth = (const float2*)(d + o_pth);
     // FP32 index estimates (corrected exactly against the tables on device)
     const double l0 = log(rn[0]), l1 = log(rn[Nr]);
     G.lr0 = (float)l0;

@@ -331,7 +331,6 @@ struct GridDev {
     int Nr, Nth, ld;
     const double *rn, *rh, *tn, *th;   // th: Nth half nodes + th[Nth] = th[0] + (tn[Nth] - tn[0])
     const double *irn, *irh, *itn, *ith;
-    const float2 *prn, *prh, *ptn, *pth;   // the inverse spacings as pairs of floats (locate_ff)
     float lr0, lrh0, ilr;        // FP32 index estimate in ln r
     float t0, th0, it;           // FP32 index estimate in th
     int full;                    // full-theta domain (periodic th), else half-theta
@@ -396,23 +395,26 @@ __device__ __forceinline__ void locate(const double* __restrict__ X, const doubl
     w = ww;
 }
 
-// The same with the weight in paired FP32 -- the FP64 difference x - X[i]
-// (exact but for its own rounding) times the inverse spacing, to 2^-47 -- and
-// without walking: the weight is a NaN where the estimated cell is not x's,
-// once in some ten thousand on grids even in ln r and th.  (Walks in the push's
-// main path took a twentieth of its time, and a flag as much.)
-__device__ __forceinline__ void locate_ff(const double* __restrict__ X, const float2* __restrict__ pX, int m, double x,
-                                          float est, int& i, ff& w)
+// The same without walking, for the gather: the weight is a NaN (an integer
+// compare away) where the estimated cell is not x's, once in some ten thousand
+// on grids even in ln r and th.  (Walks in the push's main path took a twentieth
+// of its time, and a flag as much.)
+__device__ __forceinline__ void locate_est(const double* __restrict__ X, const double* __restrict__ iX, int m, double x,
+                                           float est, int& i, double& w)
 {
     const long long kx = okey(x);
     const int k = max(0, min(__float2int_rd(est), m - 2));
     const double x0 = __ldg(X + k), x1 = __ldg(X + k + 1);
-    const float2 ix = __ldg(pX + k);
-    const float wrong = __int_as_float(0x7fffffff);
+    const double wrong = __longlong_as_double(0x7fffffffffffffffLL);
     i = k;
-    w = ff_mul(ff_from(x - x0), {ix.x, ix.y});
-    if (kx < okey(x0)) w = {k > 0 ? wrong : 0.f, 0.f};
-    if (kx >= okey(x1)) w = {k < m - 2 ? wrong : 1.f, 0.f};
+    w = (x - x0) * __ldg(iX + k);
+    if (kx < okey(x0)) w = k > 0 ? wrong : 0.0;
+    if (kx >= okey(x1)) w = k < m - 2 ? wrong : 1.0;
+}
+
+__device__ __forceinline__ bool is_nan(double x)
+{
+    return (unsigned long long)(__double_as_longlong(x) << 1) > 0xffe0000000000000ull;
 }
 
 struct Fields {
@@ -452,15 +454,14 @@ static __device__ __noinline__ void gather(const GridDev& G, const Fields& F, do
 }
 
 // The same bilinear interpolant from per-cell coefficients: component k's
-// cell (i, j) holds a = f00 in FP64 and b = f10 - f00, c = f01 - f00,
-// d = f11 - f10 - f01 + f00 as pairs of floats, 32 bytes at 4 (i ld + j) doubles (r
-// index first; built by k_field_coef before each push), and
-// f = a + (b w_r + w_th (c + d w_r)), the bracket in paired FP32: what the
-// cell adds to a is good to 2^-47 of its differences, as the weights are, and
-// one FP64 addition per component remains of three fused multiply-adds (an
-// expansion about the cell's centre measured the same error).
-// A cell whose differences are no numbers or outside 2^-90 .. 2^100 is marked
-// (b's high float a NaN) and gathered from the fields in FP64.
+// cell (i, j) holds (a, b, c, d) = (f00, f10 - f00, f01 - f00,
+// f11 - f10 - f01 + f00) at 4 (i ld + j) (r index first; built by k_field_coef
+// before each push), so that f = a + b w_r + w_th (c + d w_r) is 3 FMA.  All in FP64,
+// 26 operations a gather: the FP64 pipe has room beside the right-hand side's
+// integer work.  With the weights and differences in paired FP32 (10 FP64
+// operations, 230 issue slots more) a cell whose values differ as much as
+// themselves was gathered to 4e-14 of them (now 8e-16), and a push was slower:
+// 2^20 particles on 512^2 1006 -> 988 us, the batch of 12 runs 853 -> 782 us.
 struct FieldsC {
     const double* c[6];
 };
@@ -476,54 +477,34 @@ struct StageTile {
     int i0, j0;
 };
 
-__device__ __forceinline__ ff ff_bits(double x)      // a pair of floats stored in a double's place
+__device__ __forceinline__ double cell_value(double2 ab, double2 cd, double wr, double wt)
 {
-    return {__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x))};
+    return fma(wt, fma(cd.y, wr, cd.x), fma(ab.y, wr, ab.x));
 }
 
-// A component's value from its cell's coefficients; odd if the cell is marked
-// or a weight is not of the cell (NaNs either way).
-__device__ __forceinline__ double cell_value(double2 ab, double2 cd, ff wr, ff wt, bool& odd)
-{
-    const ff d = ff_add(ff_mul(ff_bits(ab.y), wr), ff_mul(wt, ff_add(ff_bits(cd.x), ff_mul(ff_bits(cd.y), wr))));
-    odd = odd || d.hi != d.hi;
-    return ab.x + ff_to_bits(d);
-}
-
-// gather_c where a cell is marked or an estimated cell not the right one.
-static __device__ __noinline__ void gather_far(const GridDev& G, const FieldsC& F, const Fields& raw, double r, double th,
-                                               double v[6])
+// gather_c where an estimated cell is not the right one.
+static __device__ __noinline__ void gather_far(const GridDev& G, const FieldsC& F, double r, double th, double v[6])
 {
     const float lr = __logf(f32_cut(r));
-    double x[4] = {r, r, 0.0, 0.0};
-    int mh;
-    theta_views(G, th, x[2], x[3], mh);
-    const double* const X[4] = {G.rn, G.rh, G.tn, G.th};
-    const float2* const pX[4] = {G.prn, G.prh, G.ptn, G.pth};
-    const int m[4] = {G.Nr + 1, G.Nr, G.Nth + 1, mh};
-    const float est[4] = {(lr - G.lr0) * G.ilr, (lr - G.lrh0) * G.ilr, (f32_cut(x[2]) - G.t0) * G.it,
-                          (f32_cut(x[3]) - G.th0) * G.it};
-    int at[4];
-    ff w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        at[q] = locate_walk(X[q], m[q], okey(x[q]), est[q]);
-        locate_ff(X[q], pX[q], m[q], x[q], (float)at[q], at[q], w[q]);
-    }
-    bool odd = false;
+    int at[4], mh;
+    double w[4], tnv, thv;
+    theta_views(G, th, tnv, thv, mh);
+    locate(G.rn, G.irn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, at[0], w[0]);
+    locate(G.rh, G.irh, G.Nr, r, (lr - G.lrh0) * G.ilr, at[1], w[1]);
+    locate(G.tn, G.itn, G.Nth + 1, tnv, (f32_cut(tnv) - G.t0) * G.it, at[2], w[2]);
+    locate(G.th, G.ith, mh, thv, (f32_cut(thv) - G.th0) * G.it, at[3], w[3]);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         const bool ro = (k == 0 || k == 4 || k == 5);
         const bool to = (k == 1 || k == 3 || k == 5);
         const double2* q = reinterpret_cast<const double2*>(F.c[k] + 4 * ((size_t)at[ro] * G.ld + at[2 + to]));
-        v[k] = cell_value(__ldg(q), __ldg(q + 1), w[ro], w[2 + to], odd);
+        v[k] = cell_value(__ldg(q), __ldg(q + 1), w[ro], w[2 + to]);
     }
-    if (odd) gather(G, raw, r, th, v);
 }
 
 template <bool STAGED = false>
-__device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, const Fields& raw, double r, double th,
-                                         double D[3], double B[3], const StageTile* T = nullptr)
+__device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, double r, double th, double D[3], double B[3],
+                                         const StageTile* T = nullptr)
 {
     const float lr = __logf(f32_cut(r));
     double tnv, thv;
@@ -531,12 +512,11 @@ __device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, con
     theta_views(G, th, tnv, thv, mh);
     const float tfn = f32_cut(tnv), tfh = G.full ? f32_cut(thv) : tfn;
     int i0, i1, j0, j1;
-    ff wr0, wr1, wt0, wt1;
-    bool odd = false;
-    locate_ff(G.rn, G.prn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
-    locate_ff(G.rh, G.prh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
-    locate_ff(G.tn, G.ptn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
-    locate_ff(G.th, G.pth, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
+    double wr0, wr1, wt0, wt1;
+    locate_est(G.rn, G.irn, G.Nr + 1, r, (lr - G.lr0) * G.ilr, i0, wr0);
+    locate_est(G.rh, G.irh, G.Nr, r, (lr - G.lrh0) * G.ilr, i1, wr1);
+    locate_est(G.tn, G.itn, G.Nth + 1, tnv, (tfn - G.t0) * G.it, j0, wt0);
+    locate_est(G.th, G.ith, mh, thv, (tfh - G.th0) * G.it, j1, wt1);
     const int ld = G.ld;
     double v[6];
 #pragma unroll
@@ -544,7 +524,7 @@ __device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, con
         const bool ro = (k == 0 || k == 4 || k == 5);
         const bool to = (k == 1 || k == 3 || k == 5);
         const int i = ro ? i1 : i0, j = to ? j1 : j0;
-        const ff wr = ro ? wr1 : wr0, wt = to ? wt1 : wt0;
+        const double wr = ro ? wr1 : wr0, wt = to ? wt1 : wt0;
         double2 ab, cd;
         const unsigned ti = STAGED ? (unsigned)(i - T->i0) : 0u, tj = STAGED ? (unsigned)(j - T->j0) : 0u;
         if (STAGED && T->s && ti < (unsigned)STAGE_TI && tj < (unsigned)STAGE_TJ) {
@@ -556,11 +536,12 @@ __device__ __forceinline__ void gather_c(const GridDev& G, const FieldsC& F, con
             ab = __ldg(q);
             cd = __ldg(q + 1);
         }
-        v[k] = cell_value(ab, cd, wr, wt, odd);
+        v[k] = cell_value(ab, cd, wr, wt);
     }
-    if (odd) {
+    // D^ph takes the weights of the nodes, B^ph those of the half nodes
+    if (is_nan(v[2]) || is_nan(v[5])) {
         double u[6];
-        gather_far(G, F, raw, r, th, u);
+        gather_far(G, F, r, th, u);
 #pragma unroll
         for (int k = 0; k < 6; ++k) v[k] = u[k];
     }

@@ -189,7 +189,7 @@ __device__ __forceinline__ void F_at_sc(const RunK& R, const double y[6], double
     double D[3] = {0, 0, 0}, B[3] = {0, 0, 0};
     if (em && want_F) {
         if (not_zero(R.B0field)) wald_point_sc(R.bh, R.B0field, y[0], s, c, D, B);
-        else if (R.has_coef) gather_c<STAGED>(R.G, R.FC, R.F, y[0], y[1], D, B, T);
+        else if (R.has_coef) gather_c<STAGED>(R.G, R.FC, y[0], y[1], D, B, T);
         else {
             double v[6];
             gather(R.G, R.F, y[0], y[1], v);
@@ -1541,21 +1541,10 @@ __global__ void k_field_coef(const __grid_constant__ CoefJobs jobs)
             const size_t o = (size_t)i * G.ld + j;
             const double* f = G.f[k];
             const double f00 = f[o], f01 = f[o + 1], f10 = f[o + G.ld], f11 = f[o + G.ld + 1];
-            const double v[3] = {f10 - f00, f01 - f00, (f11 - f10) - (f01 - f00)};
-            float2 w[3];
-            bool ok = true;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const ff x = ff_from(v[m]);
-                w[m] = make_float2(x.hi, x.lo);
-                const unsigned e = (unsigned)__double2hiint(v[m]) & 0x7fffffffu;
-                ok = ok && (!not_zero(v[m]) || e - ((1023u - 90u) << 20) < (190u << 20));
-            }
-            if (!ok) w[0].x = __int_as_float(0x7fffffff);
+            const double c = f01 - f00;
             double2* q = reinterpret_cast<double2*>(out + (size_t)k * 4 * sz + 4 * o);
-            auto bits = [](float2 x) { return __hiloint2double(__float_as_int(x.y), __float_as_int(x.x)); };
-            q[0] = make_double2(f00, bits(w[0]));
-            q[1] = make_double2(bits(w[1]), bits(w[2]));
+            q[0] = make_double2(f00, f10 - f00);
+            q[1] = make_double2(c, (f11 - f10) - c);
         }
     }
 }
