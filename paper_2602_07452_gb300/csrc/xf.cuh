@@ -232,16 +232,15 @@ FPIC_HD unsigned x_float_bits(float f)
 #endif
 }
 
-// The FP32 estimate's 24 significant bits, for a value of at least 1/2 and below
-// 1.  The hardware's may fall an ulp or two outside (its documented error is an
-// ulp for the reciprocal and 2^-22.9 for the root): held to the ends, which are
-// as good an estimate there.
+// The FP32 estimate in units of 2^-24, for a value of at least 1/2 and below 1.  The
+// hardware's may fall an ulp or two outside (its documented error is an ulp for
+// the reciprocal and 2^-22.9 for the root): below 1/2, where an ulp is half a
+// unit, counting down in whole ones is as good an estimate; at 1 it is held
+// below.
 FPIC_HD unsigned x_est24(float y)
 {
-    unsigned u = x_float_bits(y);
-    u = u < 0x3f7fffffu ? u : 0x3f7fffffu;
-    u = u > 0x3f000000u ? u : 0x3f000000u;
-    return (u & 0x7fffffu) | 0x800000u;
+    const unsigned u = x_float_bits(y);
+    return (u < 0x3f7fffffu ? u : 0x3f7fffffu) - 0x3e800000u;
 }
 
 // 1/a for a > 0: with X = m / 2^61 in [1, 2), the FP32 estimate Y of 1/X in 31
