@@ -28,6 +28,7 @@ int set_error(int code, const char* fmt, ...)
 int check_cuda(cudaError_t e, const char* what)
 {
     if (e == cudaSuccess) return 0;
+    cudaGetLastError();      // reported here: not the next call's launch error too
     if (e == cudaErrorMemoryAllocation) return set_error(FPIC_ENOMEM, "%s: %s", what, cudaGetErrorString(e));
     return set_error(FPIC_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }

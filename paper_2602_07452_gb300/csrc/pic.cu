@@ -1947,15 +1947,23 @@ __device__ __forceinline__ double cd_phdots(const CDepK& k, uint32_t p, const do
     return ok ? x : x + (d[0] + d[1]);
 }
 
-// One thread per sorted entry: entries below off[C] are moves inside their
-// cell (CI_ROWS records), the rest up to off[2 C] the general ones (CD_SLOTS).
+// The records' buffer holds CDEP_CHUNK sorted entries (4 GB of 30 rows) at most:
+// more particles take it in turns, each chunk's cell sums added to the ones
+// before: 240 bytes a particle are 15 GB at 6.4e7, and sets of a few 1e8 would not
+// fit.  As many entries as leave a large run a few chunks, each of which looks at
+// every cell's range once.
+constexpr long long CDEP_CHUNK = 1LL << 24, CDEP_CHUNK_MIN = 1LL << 20;
+
+// One thread per sorted entry a0 .. a0 + m - 1: entries below off[C] are moves
+// inside their cell (CI_ROWS records), the rest up to off[2 C] the general ones
+// (CD_SLOTS).
 __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ CDepK k,
                                                        const uint32_t* __restrict__ off,
                                                        const uint32_t* __restrict__ perm, double* __restrict__ rec,
-                                                       uint32_t C)
+                                                       long long a0, long long m, uint32_t C)
 {
-    const long long a = blockIdx.x * 128LL + threadIdx.x;
-    if (a >= (long long)off[2 * (size_t)C]) return;
+    const long long t = blockIdx.x * 128LL + threadIdx.x, a = a0 + t;
+    if (t >= m || a >= (long long)off[2 * (size_t)C]) return;
     const uint32_t p = perm[a];
     const bool inside = a < (long long)off[C];
     int ia, ja, ib, jb;
@@ -1967,8 +1975,8 @@ __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ C
     const double rr[2] = {r0, r1}, tt[2] = {t0, t1};
     const int jj[2] = {ja, jb};
     const double Qh = 0.25 * Q * cd_phdots(k, p, rr, tt, jj);         // Q (dph/dt)_mid / 2
-    rec += a;
-    auto put = [&](int row, double v) { rec[row * k.n] = v; };
+    rec += t;
+    auto put = [&](int row, double v) { rec[row * m] = v; };
     if (inside) {
         const double qx = Q * frb, qc = Q - qx, q11 = qx * ftb, q01 = qc * ftb;
         put(CI_Q + 0, qc - q01);
@@ -2033,49 +2041,61 @@ __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ C
 // One warp per cell: the 12 rows of its inside moves (32 particles at a time
 // through shared memory, lane 2 row + parity sums its row over the particles
 // of its parity, as in k_dep_cell), then lane q < 30 slot q of its general
-// moves; both in a fixed order.
+// moves; both in a fixed order.  Of the entries a0 .. a0 + m - 1; LATER: a chunk
+// after the first, which adds to the cells' sums and over which the grid strides.
 constexpr int CDEP_WARPS = 8;
+template <bool LATER>
 __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __restrict__ rec,
-                                                               const uint32_t* __restrict__ off, long long n,
-                                                               double* __restrict__ part, uint32_t C)
+                                                               const uint32_t* __restrict__ off, uint32_t a0,
+                                                               uint32_t m, double* __restrict__ part, uint32_t C)
 {
     __shared__ double sv[CDEP_WARPS][CI_ROWS * DEP_CELL_LD];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long cell = blockIdx.x * (long long)CDEP_WARPS + wid;
-    if (cell >= C) return;                  // whole warps
     double* v = sv[wid];
-    const uint32_t b0 = off[cell], b1 = off[cell + 1], c0 = off[(size_t)C + cell], c1 = off[(size_t)C + cell + 1];
     const int row = min(lane >> 1, CI_ROWS - 1), par = lane & 1;
-    double acc = 0.0;
-    for (uint32_t base = b0; base < b1; base += 32) {
-        const uint32_t cnt = min(32u, b1 - base);
-        const bool live = (uint32_t)lane < cnt;
-        double x[CI_ROWS];
+    // entry a's place in the chunk
+    const auto at = [&](uint32_t a) { return min(LATER ? (a > a0 ? a - a0 : 0u) : a, m); };
+    long long cell = blockIdx.x * (long long)CDEP_WARPS + wid;
+    if (cell >= C) return;                  // whole warps
+    do {
+        const uint32_t b0 = at(off[cell]), b1 = at(off[cell + 1]), c0 = at(off[(size_t)C + cell]),
+                       c1 = at(off[(size_t)C + cell + 1]);
+        if (LATER && b0 == b1 && c0 == c1) continue;
+        double acc = 0.0;
+        for (uint32_t base = b0; base < b1; base += 32) {
+            const uint32_t cnt = min(32u, b1 - base);
+            const bool live = (uint32_t)lane < cnt;
+            double x[CI_ROWS];
 #pragma unroll
-        for (int q = 0; q < CI_ROWS; ++q) x[q] = live ? __ldg(rec + (size_t)q * n + base + lane) : 0.0;
-        __syncwarp();                       // the previous group's reads are done
+            for (int q = 0; q < CI_ROWS; ++q) x[q] = live ? __ldg(rec + (size_t)q * m + base + lane) : 0.0;
+            __syncwarp();                       // the previous group's reads are done
 #pragma unroll
-        for (int q = 0; q < CI_ROWS; ++q) v[q * DEP_CELL_LD + lane] = x[q];
-        __syncwarp();
-        const int kend = (int)(cnt + 1) >> 1;
-        for (int k = 0; k < kend; ++k) acc += v[row * DEP_CELL_LD + 2 * k + par];
-    }
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    double g = 0.0;
-    const int slot = min(lane, CD_SLOTS - 1);
-    for (uint32_t a = c0; a < c1; ++a) g += __ldg(rec + (size_t)slot * n + a);
-    // the inside row that belongs to this lane's slot, if any
-    int src = -1;
-    if (slot < CD_R) {
-        const int q = slot % 9, x = q / 3, y = q % 3;
-        if (x < 2 && y < 2) src = (slot < CD_P ? CI_Q : CI_P) + x + 2 * y;
-    } else if (slot < CD_T) {
-        if (slot - CD_R < 2) src = CI_R + (slot - CD_R);
-    } else if (slot == CD_T || slot == CD_T + 2) {
-        src = CI_T + ((slot - CD_T) >> 1);
-    }
-    const double in = __shfl_sync(0xffffffffu, acc, 2 * max(src, 0));
-    if (lane < CD_SLOTS) part[(size_t)lane * C + cell] = src >= 0 ? in + g : g;
+            for (int q = 0; q < CI_ROWS; ++q) v[q * DEP_CELL_LD + lane] = x[q];
+            __syncwarp();
+            const int kend = (int)(cnt + 1) >> 1;
+            for (int k = 0; k < kend; ++k) acc += v[row * DEP_CELL_LD + 2 * k + par];
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        double g = 0.0;
+        const int slot = min(lane, CD_SLOTS - 1);
+        for (uint32_t a = c0; a < c1; ++a) g += __ldg(rec + (size_t)slot * m + a);
+        // the inside row that belongs to this lane's slot, if any
+        int src = -1;
+        if (slot < CD_R) {
+            const int q = slot % 9, x = q / 3, y = q % 3;
+            if (x < 2 && y < 2) src = (slot < CD_P ? CI_Q : CI_P) + x + 2 * y;
+        } else if (slot < CD_T) {
+            if (slot - CD_R < 2) src = CI_R + (slot - CD_R);
+        } else if (slot == CD_T || slot == CD_T + 2) {
+            src = CI_T + ((slot - CD_T) >> 1);
+        }
+        const double in = __shfl_sync(0xffffffffu, acc, 2 * max(src, 0));
+        if (lane < CD_SLOTS) {
+            double* o = part + (size_t)lane * C + cell;
+            const double sum = src >= 0 ? in + g : g;
+            *o = LATER ? *o + sum : sum;
+        }
+    } while (LATER && (cell += gridDim.x * (long long)CDEP_WARPS) < C);
 }
 
 __device__ __forceinline__ double cd_dual_r(const GridDev& G, int i)
@@ -2138,9 +2158,14 @@ extern "C" int fpic_deposit_conserving(fpic_ctx* c, const fpic_particles* before
     cudaStream_t s = (cudaStream_t)stream;
     const long long C = (long long)c->Nr * c->Nth;
     Work w;
-    void* part_v = nullptr;     // per-cell window partials (CD_SLOTS x C), the particles' records (CD_SLOTS x n)
+    void* part_v = nullptr;     // per-cell window partials (CD_SLOTS x C), a chunk's records (CD_SLOTS x chunk)
     const long long nn = n > 0 ? n : 1;
-    int rc = work_layout(c, nn, false, w, (size_t)CD_SLOTS * (C + nn) * sizeof(double), &part_v, 2);
+    // entries at a time; fewer where the records do not fit the memory left
+    long long chunk = nn < CDEP_CHUNK ? nn : CDEP_CHUNK;
+    int rc;
+    while ((rc = work_layout(c, nn, false, w, (size_t)CD_SLOTS * (C + chunk) * sizeof(double), &part_v, 2)) == FPIC_ENOMEM &&
+           chunk > CDEP_CHUNK_MIN)
+        chunk = chunk / 4 > CDEP_CHUNK_MIN ? chunk / 4 : CDEP_CHUNK_MIN;
     if (rc) return rc;
     double* part = (double*)part_v;
     double* rec = part + (size_t)CD_SLOTS * C;
@@ -2156,9 +2181,16 @@ extern "C" int fpic_deposit_conserving(fpic_ctx* c, const fpic_particles* before
     if (rc) return rc;
     if (n > 0) k_scatter<<<nb, 256, 0, s>>>(w.key, w.off, w.cursor, w.perm, n);
     k_bucket_rank<<<(unsigned)((2 * C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, 2 * (uint32_t)C);
-    if (n > 0) k_cdep_particle<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(k, w.off, w.perm2, rec, (uint32_t)C);
-    k_cdep_cell<<<(unsigned)((C + CDEP_WARPS - 1) / CDEP_WARPS), 32 * CDEP_WARPS, 0, s>>>(rec, w.off, nn, part,
-                                                                                         (uint32_t)C);
+    for (long long a0 = 0; a0 < nn; a0 += chunk) {
+        const long long m = nn - a0 < chunk ? nn - a0 : chunk;
+        if (n > 0) k_cdep_particle<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(k, w.off, w.perm2, rec, a0, m, (uint32_t)C);
+        const long long cb = (C + CDEP_WARPS - 1) / CDEP_WARPS, few = 16LL * c->sm_count;
+        if (a0 == 0)
+            k_cdep_cell<false><<<(unsigned)cb, 32 * CDEP_WARPS, 0, s>>>(rec, w.off, 0, (uint32_t)m, part, (uint32_t)C);
+        else
+            k_cdep_cell<true><<<(unsigned)(cb < few ? cb : few), 32 * CDEP_WARPS, 0, s>>>(rec, w.off, (uint32_t)a0,
+                                                                                        (uint32_t)m, part, (uint32_t)C);
+    }
     k_cdep_node<<<dim3((unsigned)((c->Nth + 1 + 255) / 256), c->Nr + 1), 256, 0, s>>>(k, tabs_of(c), part,
                                                                                      (uint32_t)C, dt, rho, jr,
                                                                                      jth, jph);
