@@ -1978,11 +1978,11 @@ __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ C
     rec += t;
     auto put = [&](int row, double v) { rec[row * m] = v; };
     if (inside) {
-        const double qx = Q * frb, qc = Q - qx, q11 = qx * ftb, q01 = qc * ftb;
-        put(CI_Q + 0, qc - q01);
-        put(CI_Q + 1, qx - q11);
-        put(CI_Q + 2, q01);
-        put(CI_Q + 3, q11);
+        const double qx = Q * frb, qc = fma(-Q, frb, Q);
+        put(CI_Q + 0, fma(-qc, ftb, qc));
+        put(CI_Q + 1, fma(-qx, ftb, qx));
+        put(CI_Q + 2, qc * ftb);
+        put(CI_Q + 3, qx * ftb);
         const double sx = fra + frb, sy = fta + ftb, px = Qh * sx;
         const double p11 = Qh * fma(fra, fta, frb * ftb), p01 = fma(Qh, sy, -p11);
         put(CI_P + 0, fma(2.0, Qh, -px) - p01);
@@ -2040,8 +2040,10 @@ __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ C
 
 // One warp per cell: the 12 rows of its inside moves (32 particles at a time
 // through shared memory, lane 2 row + parity sums its row over the particles
-// of its parity, as in k_dep_cell), then lane q < 30 slot q of its general
-// moves; both in a fixed order.  Of the entries a0 .. a0 + m - 1; LATER: a chunk
+// of its parity), then lane q < 30 slot q of its general moves; both in a fixed
+// order, a group of 32 by itself (the inside moves by fours): as many additions as
+// one after the other in shorter chains (rho of 60 particles a cell 9e-16 -> 5e-16
+// off).  Of the entries a0 .. a0 + m - 1; LATER: a chunk
 // after the first, which adds to the cells' sums and over which the grid strides.
 constexpr int CDEP_WARPS = 8;
 template <bool LATER>
@@ -2072,13 +2074,21 @@ __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __r
 #pragma unroll
             for (int q = 0; q < CI_ROWS; ++q) v[q * DEP_CELL_LD + lane] = x[q];
             __syncwarp();
-            const int kend = (int)(cnt + 1) >> 1;
-            for (int k = 0; k < kend; ++k) acc += v[row * DEP_CELL_LD + 2 * k + par];
+            const double* u = v + row * DEP_CELL_LD + par;
+            const int kend = (int)cnt;          // particles past the group's end hold zeros
+            double t = (u[0] + u[2]) + (u[4] + u[6]);
+            for (int k = 8; k < kend; k += 8) t += (u[k] + u[k + 2]) + (u[k + 4] + u[k + 6]);
+            acc += t;
         }
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         double g = 0.0;
         const int slot = min(lane, CD_SLOTS - 1);
-        for (uint32_t a = c0; a < c1; ++a) g += __ldg(rec + (size_t)slot * m + a);
+        const double* rs = rec + (size_t)slot * m;
+        for (uint32_t a = c0; a < c1;) {
+            double t = 0.0;
+            for (const uint32_t e = min(a + 32u, c1); a < e; ++a) t += __ldg(rs + a);
+            g += t;
+        }
         // the inside row that belongs to this lane's slot, if any
         int src = -1;
         if (slot < CD_R) {
