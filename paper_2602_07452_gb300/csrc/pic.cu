@@ -365,15 +365,11 @@ __global__ void k_scatter(const uint32_t* key, const uint32_t* off, uint32_t* cu
     if (valid) perm[off[k] + base + (uint32_t)__popc(peers & ((1u << lane) - 1u))] = (uint32_t)p;
 }
 
-// Order every bucket by particle index (rank = number of smaller indices in
-// the bucket): one warp per bucket.  Removed particles (last bucket) are
-// handled by k_dead_rank.
-__global__ void k_bucket_rank(const uint32_t* off, const uint32_t* perm, uint32_t* perm2, uint32_t C)
+// Order a bucket (perm[b0] .. perm[b1 - 1]) by particle index (rank = number of
+// smaller indices in the bucket), by a warp.
+__device__ __forceinline__ void rank_bucket(uint32_t b0, uint32_t b1, const uint32_t* perm, uint32_t* perm2)
 {
-    const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (warp >= C) return;
-    const uint32_t b0 = off[warp], b1 = off[warp + 1];
     // a bucket already in index order (the usual case: nearly sorted input,
     // whole warps placed in lane order) is copied as it is
     bool sorted = true;
@@ -388,6 +384,23 @@ __global__ void k_bucket_rank(const uint32_t* off, const uint32_t* perm, uint32_
         for (uint32_t b = b0; b < b1; ++b) rank += perm[b] < x ? 1u : 0u;
         perm2[b0 + rank] = x;
     }
+}
+
+// Every bucket, one warp per cell: its one bucket, or (SETS 2) the two of the
+// cell, C apart.  Removed particles (last bucket) are handled by k_dead_rank.
+template <int SETS>
+__global__ void k_bucket_rank(const uint32_t* off, const uint32_t* perm, uint32_t* perm2, uint32_t C)
+{
+    const long long cell = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    if (cell >= C) return;
+    uint32_t b[SETS][2];
+#pragma unroll
+    for (int q = 0; q < SETS; ++q) {
+        b[q][0] = off[(size_t)q * C + cell];
+        b[q][1] = off[(size_t)q * C + cell + 1];
+    }
+#pragma unroll
+    for (int q = 0; q < SETS; ++q) rank_bucket(b[q][0], b[q][1], perm, perm2);
 }
 
 // Removed particles keep their relative order: position = off[C] + number of
@@ -567,7 +580,7 @@ static int sort_impl(fpic_ctx* c, fpic_particles* p, Work& w, cudaStream_t s, do
     int rc = scan_u32(w.count, w.off, w.bsum, (long long)C + 1, s);
     if (rc) return rc;
     k_scatter<<<nb, 256, 0, s>>>(w.key, w.off, w.cursor, w.perm, n);
-    k_bucket_rank<<<(unsigned)(((long long)C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, C);
+    k_bucket_rank<1><<<(unsigned)(((long long)C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, C);
     // removed particles: per-block counts in w.pos (nbd + 1 <= n + 1 entries)
     const unsigned nbd = (unsigned)((n + DEAD_PER * DEAD_T - 1) / (DEAD_PER * DEAD_T));
     k_dead_count<<<nbd, DEAD_T, 0, s>>>(p->alive, w.pos, n);
@@ -1319,6 +1332,10 @@ __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* 
     double* v = sv[wid];
     uint32_t* cw = sc[wid];
     const uint32_t b0 = off[cell], b1 = off[cell + 1];
+    if (b0 == b1) {                         // an empty cell
+        if (lane < 20) part[(size_t)lane * C + cell] = 0.0;
+        return;
+    }
     const int row = lane >> 1, par = lane & 1;
     const int bsh = row >= 12 ? 2 : 0;      // the offset bit this row splits on
     const uint32_t bmask = row >= 8 ? 1u : 0u;
@@ -2062,7 +2079,10 @@ __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __r
     do {
         const uint32_t b0 = at(off[cell]), b1 = at(off[cell + 1]), c0 = at(off[(size_t)C + cell]),
                        c1 = at(off[(size_t)C + cell + 1]);
-        if (LATER && b0 == b1 && c0 == c1) continue;
+        if (b0 == b1 && c0 == c1) {             // an empty cell
+            if (!LATER && lane < CD_SLOTS) part[(size_t)lane * C + cell] = 0.0;
+            continue;
+        }
         double acc = 0.0;
         for (uint32_t base = b0; base < b1; base += 32) {
             const uint32_t cnt = min(32u, b1 - base);
@@ -2182,15 +2202,15 @@ extern "C" int fpic_deposit_conserving(fpic_ctx* c, const fpic_particles* before
     CDepK k{c->Nr, c->Nth, c->ld, c->G, c->bh, n, before->r, before->th, before->ur, before->uth, before->uph,
             before->alive, after->r, after->th, after->ur, after->uth, after->uph, after->qm, after->w,
             c->d_metric + (size_t)MT_N * c->metric_stride};
-    FPIC_CUDA(cudaMemsetAsync(w.count, 0, 4 * (2 * (size_t)C + 2), s));
-    FPIC_CUDA(cudaMemsetAsync(w.cursor, 0, 4 * (2 * (size_t)C + 2), s));
+    // count and cursor follow one another
+    FPIC_CUDA(cudaMemsetAsync(w.count, 0, (char*)(w.cursor + 2 * (size_t)C + 2) - (char*)w.count, s));
     FPIC_CUDA(cudaMemsetAsync(c->d_cnt + CNT_ERR, 0, sizeof(long long), s));
     const unsigned nb = (unsigned)((n + 255) / 256);
     if (n > 0) k_cdep_keys<<<nb, 256, 0, s>>>(k, w.key, w.count, (uint32_t)C, c->d_cnt + CNT_ERR);
     rc = scan_u32(w.count, w.off, w.bsum, 2 * C + 1, s);
     if (rc) return rc;
     if (n > 0) k_scatter<<<nb, 256, 0, s>>>(w.key, w.off, w.cursor, w.perm, n);
-    k_bucket_rank<<<(unsigned)((2 * C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, 2 * (uint32_t)C);
+    k_bucket_rank<2><<<(unsigned)((C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, (uint32_t)C);
     for (long long a0 = 0; a0 < nn; a0 += chunk) {
         const long long m = nn - a0 < chunk ? nn - a0 : chunk;
         if (n > 0) k_cdep_particle<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(k, w.off, w.perm2, rec, a0, m, (uint32_t)C);
@@ -2440,7 +2460,7 @@ extern "C" int fpic_inject_pairs(fpic_ctx* c, fpic_particles* p, long long capac
     rc = scan_u32(w.count, w.off, w.bsum, C + 1, s);
     if (rc) return rc;
     if (n > 0) k_scatter<<<nb, 256, 0, s>>>(w.key, w.off, w.cursor, w.perm, n);
-    k_bucket_rank<<<(unsigned)((C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, (uint32_t)C);
+    k_bucket_rank<1><<<(unsigned)((C * 32 + 255) / 256), 256, 0, s>>>(w.off, w.perm, w.perm2, (uint32_t)C);
     const double r_h = c->r_h;
     InjK k{c->Nr, c->Nth, c->ld, c->G, c->bh, c->a / (2.0 * c->M * r_h), prm->r_lo, prm->r_hi, prm->multiplicity,
            prm->n0, prm->qm_e, prm->B0pot, Br, Bth, draws, p->w, p->qm, w.off, w.perm2, w.flag, flags, w.tmp};
