@@ -1314,10 +1314,12 @@ __device__ __forceinline__ double sel_bits(bool p, double a, double b)
 
 // PAIRS: the shares are pairs of floats (k_dep_particle_poly).  The high
 // floats are summed in FP64, the low ones (2^-24 of them) in FP32: 2^-48 of the
-// sum of |share|, under the shares' own rounding, at one FP64 addition to
-// four shares, after a tree of exact FP32 two-sums whose errors join the low
-// floats (one addition a share: deposit of 4.0e6 particles on 512^2 1136 -> 1108
-// us); the 16 conversions a particle are not in the FP64-bound kernel before it.
+// sum of |share|, under the shares' own rounding, at one FP64 addition to four
+// shares, after a tree of exact FP32 two-sums whose errors join the low floats
+// (one addition a share: deposit of 4.0e6 particles on 512^2 1136 -> 1108 us).  The
+// low sums join the FP64 ones after every 128 particles: in a crowded cell they
+// would lose what is small beside them (16384 equal shares 3e-12 off).  The 16
+// conversions a particle are not in the FP64-bound kernel before it.
 template <bool PAIRS>
 __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* __restrict__ rec,
                                                                    const uint32_t* __restrict__ code,
@@ -1382,6 +1384,11 @@ __global__ void __launch_bounds__(32 * DEP_CELL_WARPS) k_dep_cell(const double* 
                 acc1 += f2d_bits(h[1][0]);
                 lo0 += l[0];
                 lo1 += l[1];
+            }
+            if (((base - b0) & 96u) == 96u) {
+                acc0 += f2d_bits(lo0);
+                acc1 += f2d_bits(lo1);
+                lo0 = lo1 = 0.f;
             }
             continue;
         }
