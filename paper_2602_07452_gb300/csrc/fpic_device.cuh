@@ -4,14 +4,13 @@
 //
 // GB300 note: FP64 issues at 1/64 of the FP32 rate, so the right-hand side
 // runs on integer mantissas of 60 bits (rhs_x, xf.cuh; the FP64 form remains
-// for the Newton iteration and for arguments that have none), differences
-// that need 46 bits or fewer in paired FP32 (ff.cuh), and cell location by
-// integer comparison of the IEEE bit patterns (order-preserving) instead of
-// FP64 compares.  What is left in FP64 is written to minimise its
-// instructions: one reciprocal and two reciprocal square roots per
-// evaluation, fused multiply-adds throughout.  Against an extended-precision
-// RK4 step the pushed states' relative errors are 4.8e-17 to 5.1e-17 at 48 to
-// 900 cells a side, H's 7e-17 to 9e-17 (all in FP64 16e-17).
+// for arguments that have none), the sin/cos series of small steps and the
+// corrections of reciprocals and roots in paired FP32 (ff.cuh), and cell
+// location by integer comparison of the IEEE bit patterns (order-preserving)
+// instead of FP64 compares.  The field gather and the stages' sums are FP64,
+// fused multiply-adds throughout.  Against an extended-precision RK4 step the
+// pushed states' relative errors are 4.8e-17 to 5.1e-17 at 48 to 900 cells a
+// side, H's 7e-17 to 9e-17 (all in FP64 16e-17).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -35,8 +34,8 @@ struct BH {
 // FP64 pipe takes 64 issue slots per operation, so the 40 or so FP32 and
 // integer instructions cost less than the two (three) FP64 operations they
 // replace.  Arguments outside 2^-60 .. 2^60 (where the correction's low float
-// keeps its bits), zeros, infinities and NaNs take the FP64 forms: the hardware estimate y and y (1 + e + e^2), or y (1 + e/2 +
-// 3 e^2/8).
+// keeps its bits), zeros, infinities and NaNs take the FP64 forms: the hardware
+// estimate y and y (1 + e + e^2), or y (1 + e/2 + 3 e^2/8).
 __device__ __forceinline__ bool f32_range(unsigned hi)      // 2^-60 <= x < 2^60, hi the high word of |x|
 {
     return hi - ((1023u - 60u) << 20) < (120u << 20);

@@ -918,11 +918,11 @@ __device__ __forceinline__ bool same_bits(double a, double b)
 }
 
 // The charge times the FIDO three-velocity gamma^ij u_j / Gamma, the terms
-// shared as in eval_rhs_sc_t (24 FP64 instructions besides the reciprocal's
-// and the two roots' six;
-// through the metric's components 5 more, k_dep_particle_poly 552 -> 532 us at
-// 4.0e6 particles with the sin/cos series in paired FP32).  FP64: the 1/sin^2 th of g^phph and the cancellation
-// between the two terms of U^r and U^ph want more than paired FP32's 46 bits.
+// shared as in eval_rhs_sc_t (24 FP64 instructions besides the reciprocal's and
+// the two roots' six; through the metric's components 5 more, k_dep_particle_poly
+// 552 -> 532 us at 4.0e6 particles with the sin/cos series in paired FP32).  FP64:
+// the 1/sin^2 th of g^phph and the cancellation between the two terms of U^r and
+// U^ph want more than paired FP32's 46 bits.
 __device__ __forceinline__ void charge_flux(const BH& bh, double r, double s, double c, double ur, double ut, double up,
                                             double Q, double& Qr, double& Qt, double& Qp)
 {

@@ -169,11 +169,6 @@ FPIC_HD xf x_neg(xf a)
     return {~a.m, a.e};
 }
 
-FPIC_HD xf x_scale(xf a, int k)       // a 2^k
-{
-    return {a.m, a.e + k};
-}
-
 // m >> n, the sign for n above 63
 FPIC_HD long long x_shr(long long m, int n)
 {
