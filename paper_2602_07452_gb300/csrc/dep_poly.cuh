@@ -193,17 +193,6 @@ __device__ __forceinline__ ff ff_addf(ff a, float b)      // a + b, |b| far belo
     return {a.hi, __fadd_rn(a.lo, b)};
 }
 
-// a b of pairs whose low floats carry FP32 terms of their own, far above 2^-24 of
-// the high ones: their product counts (R_1 E_1 and R_2 E_2: up to 10^-12 of the sum
-// on grids of 150 cells a side).
-__device__ __forceinline__ ff ff_mul_lo(ff a, ff b)
-{
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.lo, b.lo, __fmaf_rn(a.hi, b.hi, -p));
-    e = __fmaf_rn(a.hi, b.lo, e);
-    return {p, __fmaf_rn(a.lo, b.hi, e)};
-}
-
 // d2_2, d2_6: dth^2 / 2 and dth^2 / 6.  The cubic term of sin th, up to 10^-6
 // of the sum in the cells at the poles, is paired too.
 __device__ __forceinline__ void moments_th(const Mom M[2], ff tau, ff d2_2, ff d2_6, MomT E[2])
@@ -251,8 +240,12 @@ __device__ __forceinline__ void poly_shares(const float4* __restrict__ c, const 
         for (int g = 0; g < 2; ++g) {
             const MomT& e = Y[g];
             // sum - 1 = e0 + R0 + R0 e0 + R1 e1 + R2 e2 + ...
-            ff S = ff_add(ff_add(e.e0, R0), ff_add(ff_mul(R0, e.e0), ff_mul_lo(R1, e.e1)));
-            S = ff_add(S, ff_addf(ff_mul_lo(R2, e.e2), fmaf(R3, e.e3, fmaf(R4, e.e4, f05 * e.e5))));
+            ff S = ff_add(ff_add(e.e0, R0), ff_add(ff_mul(R0, e.e0), ff_mul(R1, e.e1)));
+            // the low floats of R_1, E_1, R_2, E_2 carry FP32 terms of their own, far above
+            // 2^-24 of the high ones: their products, which ff_mul leaves out, count
+            // (up to 10^-12 of the sum on grids of 150 cells a side)
+            const float ll = fmaf(R1.lo, e.e1.lo, fmaf(R2.lo, e.e2.lo, f05 * e.e5));
+            S = ff_add(S, ff_addf(ff_mul(R2, e.e2), fmaf(R3, e.e3, fmaf(R4, e.e4, ll))));
             const ff area = ff_mul(m.len, e.len);
             const ff v = ff_add(area, ff_mul(area, S));
             V[h + 2 * g] = ff_fast2(v.hi, v.lo);         // normalized: S carries FP32 terms in its lo

@@ -393,14 +393,9 @@ __global__ void k_bucket_rank(const uint32_t* off, const uint32_t* perm, uint32_
 {
     const long long cell = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     if (cell >= C) return;
-    uint32_t b[SETS][2];
-#pragma unroll
-    for (int q = 0; q < SETS; ++q) {
-        b[q][0] = off[(size_t)q * C + cell];
-        b[q][1] = off[(size_t)q * C + cell + 1];
-    }
-#pragma unroll
-    for (int q = 0; q < SETS; ++q) rank_bucket(b[q][0], b[q][1], perm, perm2);
+    const uint32_t c0 = SETS > 1 ? off[(size_t)C + cell] : 0u, c1 = SETS > 1 ? off[(size_t)C + cell + 1] : 0u;
+    rank_bucket(off[cell], off[cell + 1], perm, perm2);
+    if (SETS > 1) rank_bucket(c0, c1, perm, perm2);
 }
 
 // Removed particles keep their relative order: position = off[C] + number of
