@@ -394,11 +394,12 @@ int fpic_probe_fp64(double *gflops_out, int reps);
  *     the hardware estimate and one Goldschmidt step (2^-39.6 measured).
  *     Lattice points, weights and node shares are the same; results differ
  *     by rounding only (1e-13 relative and below on the deposited sources).
- *     With 1, grids fine enough (120 to 240 cells a side over two decades in
- *     r) take the same trapezoid sums from a degree-5 polynomial of
- *     sqrt(gamma) per cell, tabulated by the first fpic_deposit on a grid
- *     (336 bytes a cell; that call waits for the stream once, and uses the
- *     lattices if it is being captured).
+ *     With 1, grids fine enough (95 to 180 cells a side over two decades in
+ *     r, by spin) take the same trapezoid sums from a polynomial of degree 6 or
+ *     5 of sqrt(gamma) per cell, tabulated by the first fpic_deposit on a grid
+ *     (up to 384 bytes a cell; that call waits for the stream once or twice,
+ *     and uses the lattices if it is being captured, or if the memory is not
+ *     there, then until the next fpic_set_grid).
  *   FPIC_TUNE_ASYNC: 1 = fpic_push and fpic_push_host never synchronise the
  *     stream: requested stats are assembled on the device and copied into
  *     *stats asynchronously (valid once `stream` has been synchronised; pass

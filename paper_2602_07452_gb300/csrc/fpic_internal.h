@@ -30,7 +30,7 @@ struct fpic_ctx {
     // fpic_deposit on a grid; poly_grid: the grid_gen they belong to
     void* d_poly = nullptr;
     unsigned long long poly_grid = ~0ull;
-    bool poly_ok = false;
+    int poly_deg = 0;                // 0: none
     // metric tables at the Yee points (library-owned), see pic.cu
     double* d_metric = nullptr;
     size_t metric_stride = 0;        // elements per table

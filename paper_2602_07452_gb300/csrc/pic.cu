@@ -1045,6 +1045,7 @@ __device__ __forceinline__ float2 pair_of(double d)
     return make_float2(h, (float)(d - (double)h));
 }
 
+template <int DEG>
 __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ PolyBuild k)
 {
     const int sg = blockIdx.z, j = blockIdx.x * 128 + threadIdx.x;
@@ -1058,15 +1059,15 @@ __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ Poly
         const double dy = Y[j + 1] - Y[j], y = 0.5 * (Y[j] + Y[j + 1]);
         double s, co;
         sincos(y, &s, &co);
-        PolyTheta th;
-        poly_theta(k.bh.a, s, co, dy, th);
+        PolyTheta<DEG> th;
+        poly_theta<DEG>(k.bh.a, s, co, dy, th);
         for (int i = i0; i < i1; ++i) {
             const double dx = X[i + 1] - X[i];
             double f[4][4];
-            float q[7][7];
-            poly_series(k.bh.M, 0.5 * (X[i] + X[i + 1]), dx, th, f, q);
-            e = poly_worst(e, poly_bound(q));
-            float4* c = k.c[sg] + ((size_t)i * G.Nth + j) * (POLY_STRIDE / 4);
+            float q[DEG + 2][DEG + 2];
+            poly_series<DEG>(k.bh.M, 0.5 * (X[i] + X[i + 1]), dx, th, f, q);
+            e = poly_worst(e, poly_bound<DEG>(q));
+            float4* c = k.c[sg] + ((size_t)i * G.Nth + j) * (poly_stride(DEG) / 4);
             const float2 f10 = pair_of(f[1][0]), f01 = pair_of(f[0][1]), f20 = pair_of(f[2][0]),
                          f11 = pair_of(f[1][1]), f02 = pair_of(f[0][2]);
             c[0] = make_float4(f10.x, f10.y, f01.x, f01.y);
@@ -1075,7 +1076,12 @@ __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ Poly
             c[3] = make_float4(q[1][2], q[0][3], q[4][0], q[3][1]);
             c[4] = make_float4(q[2][2], q[1][3], q[0][4], q[5][0]);
             c[5] = make_float4(q[4][1], q[3][2], q[2][3], q[1][4]);
-            c[6] = make_float4(q[0][5], 0.f, 0.f, 0.f);
+            if constexpr (DEG > 5) {
+                c[6] = make_float4(q[0][5], q[6][0], q[5][1], q[4][2]);
+                c[7] = make_float4(q[3][3], q[2][4], q[1][5], q[0][6]);
+            } else {
+                c[6] = make_float4(q[0][5], 0.f, 0.f, 0.f);
+            }
             if (j == 0 && sg < 2) k.ir[sg][i] = pair_of(1.0 / dx);
         }
         if (i0 == 0 && sg != 1) {
@@ -1091,22 +1097,41 @@ __global__ void __launch_bounds__(128) k_poly_build(const __grid_constant__ Poly
     if ((threadIdx.x & 31) == 0) atomicMax(k.bound, m);
 }
 
-// The polynomials of the context's grid (built on first use, with one wait
-// for the bound); T filled and true where they may be used.  Not built while
-// the stream is being captured, nor beyond POLY_MAX_BYTES: the lattices serve.
+// A few cells of the first row, where the bound is largest on a log grid: false
+// where the grid is not worth a look.
+template <int DEG>
+static bool poly_may(const fpic_ctx* c, const double* X, const double* Y)
+{
+    for (int q = 0; q < 16; ++q) {
+        const int j = (int)((long long)q * (c->Nth - 1) / 15);
+        const double y = 0.5 * (Y[j] + Y[j + 1]);
+        PolyTheta<DEG> th;
+        double f[4][4];
+        float g[DEG + 2][DEG + 2];
+        poly_theta<DEG>(c->a, sin(y), cos(y), Y[j + 1] - Y[j], th);
+        poly_series<DEG>(c->M, 0.5 * (X[0] + X[1]), X[1] - X[0], th, f, g);
+        if (!(poly_bound<DEG>(g) <= poly_tol(DEG))) return false;
+    }
+    return true;
+}
+
+// The polynomials of the context's grid (built on first use, with a wait for
+// the bound); T filled and deg their degree where they may be used, else 0.  Not
+// built while the stream is being captured, nor beyond POLY_MAX_BYTES, nor (until
+// the next fpic_set_grid) after an allocation that failed: the lattices serve.
 constexpr size_t POLY_MAX_BYTES = (size_t)16 << 30;
 
-static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
+static int poly_tables(fpic_ctx* c, PolyTab& T, int& deg, cudaStream_t s)
 {
-    use = false;
+    deg = 0;
     const size_t cells = (size_t)c->Nr * c->Nth, row = ((size_t)c->Nr + 31) & ~(size_t)31;
-    const size_t bytes = 3 * cells * POLY_STRIDE * 4 + 2 * row * 8 + 4 * (size_t)c->Nth * 16 + 256;
     const bool fresh = c->poly_grid != c->grid_gen;
+    int want = c->poly_deg;
     if (fresh) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         FPIC_CUDA(cudaStreamIsCapturing(s, &cap));
         if (cap != cudaStreamCaptureStatusNone) return 0;
-        c->poly_ok = false;
+        c->poly_deg = 0;
         c->poly_grid = c->grid_gen;
         retire(c, &c->d_poly);
         // spacings far beyond what the bound admits: not worth a look
@@ -1115,18 +1140,10 @@ static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
         double dr = 0.0, dt = 0.0;
         for (int i = 0; i < c->Nr; ++i) dr = fmax(dr, (X[i + 1] - X[i]) / X[i]);
         for (int j = 0; j < c->Nth; ++j) dt = fmax(dt, Y[j + 1] - Y[j]);
+        const size_t bytes = 3 * cells * poly_stride(6) * 4 + 2 * row * 8 + 4 * (size_t)c->Nth * 16 + 256;
         if (bytes > POLY_MAX_BYTES || dr > 0.05 || dt > POLY_MAX_DTH) return 0;
-        // a few cells of the first row, where the bound is largest on a log grid
-        for (int q = 0; q < 16; ++q) {
-            const int j = (int)((long long)q * (c->Nth - 1) / 15);
-            const double y = 0.5 * (Y[j] + Y[j + 1]);
-            PolyTheta th;
-            double f[4][4];
-            float g[7][7];
-            poly_theta(c->a, sin(y), cos(y), Y[j + 1] - Y[j], th);
-            poly_series(c->M, 0.5 * (X[0] + X[1]), X[1] - X[0], th, f, g);
-            if (!(poly_bound(g) <= POLY_TOL)) return 0;
-        }
+        want = poly_may<5>(c, X, Y) ? 5 : poly_may<6>(c, X, Y) ? 6 : 0;
+        if (!want) return 0;
         if (cudaMalloc(&c->d_poly, bytes) != cudaSuccess) {
             cudaGetLastError();
             c->d_poly = nullptr;
@@ -1134,29 +1151,37 @@ static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
         }
     }
     if (!c->d_poly) return 0;
-    char* b = (char*)c->d_poly;
     PolyBuild k{c->bh, c->G, {}, {}, {}, nullptr, 8};
-    for (int q = 0; q < 3; ++q) k.c[q] = (float4*)(b + q * cells * POLY_STRIDE * 4);
-    b += 3 * cells * POLY_STRIDE * 4;
-    for (int q = 0; q < 2; ++q) k.t[q] = (float4*)b + q * 2 * (size_t)c->Nth;
-    b += 4 * (size_t)c->Nth * 16;
-    for (int q = 0; q < 2; ++q) k.ir[q] = (float2*)b + q * row;
-    k.bound = (unsigned*)(b + 2 * row * 8);
-    if (fresh) {
+    for (;; want = 6) {
+        char* b = (char*)c->d_poly;
+        const size_t per = cells * poly_stride(want) * 4;
+        for (int q = 0; q < 3; ++q) k.c[q] = (float4*)(b + q * per);
+        b += 3 * per;
+        for (int q = 0; q < 2; ++q) k.t[q] = (float4*)b + q * 2 * (size_t)c->Nth;
+        b += 4 * (size_t)c->Nth * 16;
+        for (int q = 0; q < 2; ++q) k.ir[q] = (float2*)b + q * row;
+        k.bound = (unsigned*)(b + 2 * row * 8);
+        if (!fresh) break;
         const long long cols = (c->Nth + 127) / 128;
         while (k.rows > 1 && 3 * cols * (c->Nr / k.rows) < 8LL * c->sm_count) k.rows >>= 1;
+        const dim3 grid((unsigned)cols, (unsigned)((c->Nr + k.rows - 1) / k.rows), 3);
         FPIC_CUDA(cudaMemsetAsync(k.bound, 0, 4, s));
-        k_poly_build<<<dim3((unsigned)cols, (unsigned)((c->Nr + k.rows - 1) / k.rows), 3), 128, 0, s>>>(k);
+        if (want == 5) k_poly_build<5><<<grid, 128, 0, s>>>(k);
+        else k_poly_build<6><<<grid, 128, 0, s>>>(k);
         float e = 0.f;
         FPIC_CUDA(cudaMemcpyAsync(&e, k.bound, 4, cudaMemcpyDeviceToHost, s));
         FPIC_CUDA(cudaStreamSynchronize(s));
-        c->poly_ok = e <= POLY_TOL;
-        if (!c->poly_ok) {
+        if (e <= poly_tol(want)) {
+            c->poly_deg = want;
+            break;
+        }
+        if (want == 6) {
             FPIC_CUDA(cudaFree(c->d_poly));
             c->d_poly = nullptr;
+            break;
         }
     }
-    if (!c->poly_ok) return 0;
+    if (!c->poly_deg) return 0;
     const double* X = (const double*)c->h_nodes.data();      // rn, rh, tn, th (th with one node more)
     const size_t m[4] = {(size_t)c->Nr + 1, (size_t)c->Nr, (size_t)c->Nth + 1, (size_t)c->Nth};
     for (int q = 0; q < 4; ++q) {
@@ -1169,7 +1194,7 @@ static int poly_tables(fpic_ctx* c, PolyTab& T, bool& use, cudaStream_t s)
         T.ir[q] = k.ir[q];
         T.t[q] = k.t[q];
     }
-    use = true;
+    deg = c->poly_deg;
     return 0;
 }
 
@@ -1208,6 +1233,7 @@ __device__ __forceinline__ int cell_split(const double* __restrict__ X, int m, d
 // bound (61 % busy, some 57 instructions a particle) at 92 instead of 370
 // instructions per charge share: 1511 -> 532 us at 4.0e6 particles on
 // 512 x 512, 23.7 -> 9 ms at 6.4e7 on 1024 x 1024 (64 or 80 registers alike).
+template <int DEG>
 __global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_constant__ DepK k,
                                                               const __grid_constant__ PolyTab T)
 {
@@ -1224,7 +1250,7 @@ __global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_const
         const float4 t0 = __ldg(T.t[0] + 2 * j0), t1 = __ldg(T.t[0] + 2 * j0 + 1);
         const ff inv = {t0.x, t0.y};
         moments(ff_mul(ff_from(d0), inv), ff_mul(ff_from(d1), inv), Y);
-        moments_th(Y, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}, E);
+        moments_th<DEG>(Y, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}, E);
     }
     // FIDO three-velocity, as k_dep_particle_ff (sin/cos th by angle addition
     // from the node on the side where the terms share a sign)
@@ -1257,14 +1283,14 @@ __global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_const
     {   // (i+1/2, j): j^r
         const float2 ir = __ldg(T.ir[1] + i1);
         moments(ff_mul(ff_from(d0), {ir.x, ir.y}), ff_mul(ff_from(d1), {ir.x, ir.y}), X);
-        poly_shares(T.c[1] + ((size_t)i1 * G.Nth + j0) * (POLY_STRIDE / 4), X, E, w);
+        poly_shares<DEG>(T.c[1] + ((size_t)i1 * G.Nth + j0) * (poly_stride(DEG) / 4), X, E, w);
         put(8, Qr, w);
     }
     const int i0 = cell_split(G.rn, G.Nr + 1, T.lo[0], T.hi[0], r, (lr - G.lr0) * G.ilr, d0, d1);
     {   // (i, j): rho and j^ph
         const float2 ir = __ldg(T.ir[0] + i0);
         moments(ff_mul(ff_from(d0), {ir.x, ir.y}), ff_mul(ff_from(d1), {ir.x, ir.y}), X);
-        poly_shares(T.c[0] + ((size_t)i0 * G.Nth + j0) * (POLY_STRIDE / 4), X, E, w);
+        poly_shares<DEG>(T.c[0] + ((size_t)i0 * G.Nth + j0) * (poly_stride(DEG) / 4), X, E, w);
         put(0, Q, w);
         put(4, Qp, w);
     }
@@ -1273,8 +1299,8 @@ __global__ void __launch_bounds__(256, 4) k_dep_particle_poly(const __grid_const
         const float4 t0 = __ldg(T.t[1] + 2 * j1), t1 = __ldg(T.t[1] + 2 * j1 + 1);
         const ff inv = {t0.x, t0.y};
         moments(ff_mul(ff_from(d0), inv), ff_mul(ff_from(d1), inv), Y);
-        moments_th(Y, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}, E);
-        poly_shares(T.c[2] + ((size_t)i0 * G.Nth + j1) * (POLY_STRIDE / 4), X, E, w);
+        moments_th<DEG>(Y, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}, E);
+        poly_shares<DEG>(T.c[2] + ((size_t)i0 * G.Nth + j1) * (poly_stride(DEG) / 4), X, E, w);
         put(12, Qt, w);
     }
     k.code[p] = (uint32_t)(i1 - i0 + 1) | ((uint32_t)(j1 - j0 + 1) << 2);
@@ -1810,7 +1836,7 @@ extern "C" int fpic_deposit(fpic_ctx* c, fpic_particles* p, double* rho, double*
         FPIC_CUDA(cudaMemsetAsync(w.off, 0, 4 * ((size_t)C + 2), s));
     }
     PolyTab pt;
-    bool poly = false;
+    int poly = 0;
     if (n > 0 && c->dep_lattice) {
         rc = poly_tables(c, pt, poly, s);
         if (rc) return rc;
@@ -1822,7 +1848,8 @@ extern "C" int fpic_deposit(fpic_ctx* c, fpic_particles* p, double* rho, double*
         const int dt_ = c->dep_threads;
         const unsigned nb = (unsigned)((n + dt_ - 1) / dt_);
         if (!c->dep_lattice) k_dep_particle<<<nb, dt_, 0, s>>>(k);
-        else if (poly) k_dep_particle_poly<<<nb, dt_, 0, s>>>(k, pt);
+        else if (poly == 5) k_dep_particle_poly<5><<<nb, dt_, 0, s>>>(k, pt);
+        else if (poly == 6) k_dep_particle_poly<6><<<nb, dt_, 0, s>>>(k, pt);
         else k_dep_particle_ff<<<nb, dt_, 0, s>>>(k);
     }
     const unsigned cb = (unsigned)(((long long)C + DEP_CELL_WARPS - 1) / DEP_CELL_WARPS);

@@ -1,5 +1,5 @@
 """Single node shares of the deposit, relative to themselves, on grids about the
-line between the lattices and the per-cell polynomials."""
+lines between the lattices and the per-cell polynomials of degree 6 and 5."""
 import numpy as np
 import pytest
 
@@ -21,14 +21,15 @@ def _volume(a, x0, x1, y0, y1):
     return acc * (x1 - x0) * (y1 - y0) / 9
 
 
-@pytest.mark.parametrize("a,side", [(0.5, 122), (0.9, 150), (0.9, 182), (0.99, 200), (0.99, 230), (0.99, 512)])
+@pytest.mark.parametrize("a,side", [(0.5, 90), (0.5, 100), (0.9, 140), (0.9, 170), (0.9, 182), (0.99, 170),
+                                    (0.99, 200), (0.99, 230), (0.99, 512)])
 def test_small_shares_keep_their_relative_accuracy(a, side):
     """One unit charge in every ninth cell, so that a node holds one share:
     rho times the dual volume is that share.  Relative error of the shares down
     to 1e-6, corners and edges of the cells included: the square root's 4e-14 (the
-    polynomial's bound 1.3e-13 is of the cells within the horizon, a fifth of it
-    where these charges are) and eight roundings of the paired arithmetic
-    (2^-46): 1.6e-13."""
+    polynomials' bound, 1.3e-13 at most, is of the cells within the horizon, a
+    fifth of it where these charges are) and eight roundings of the paired
+    arithmetic (2^-46): 1.6e-13."""
     cuda_or_skip()
     F = fpic()
     g = I.log_grid(side, side, 0.9 * I.horizon(1.0, a), 50.0)
