@@ -2085,11 +2085,11 @@ __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ C
 }
 
 // One warp per cell: the 12 rows of its inside moves (32 particles at a time
-// through shared memory, lane 2 row + parity sums its row over the particles
-// of its parity), then lane q < 30 slot q of its general moves; both in a fixed
-// order, a group of 32 by itself (the inside moves by fours): as many additions as
-// one after the other in shorter chains (rho of 60 particles a cell 9e-16 -> 5e-16
-// off).  Of the entries a0 .. a0 + m - 1; LATER: a chunk
+// through shared memory, lane 2 row + parity sums its row over every other pair
+// of particles), then lane q < 30 slot q of its general moves; both in a fixed
+// order, a group of 32 by itself (the inside moves as a tree, neighbours first, as
+// electrons and positrons alternate): as many additions as one after the other
+// in shorter chains (rho of 60 particles a cell 9e-16 -> 2.7e-16 off).  Of the entries a0 .. a0 + m - 1; LATER: a chunk
 // after the first, which adds to the cells' sums and over which the grid strides.
 constexpr int CDEP_WARPS = 8;
 template <bool LATER>
@@ -2123,10 +2123,11 @@ __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __r
 #pragma unroll
             for (int q = 0; q < CI_ROWS; ++q) v[q * DEP_CELL_LD + lane] = x[q];
             __syncwarp();
-            const double* u = v + row * DEP_CELL_LD + par;
-            const int kend = (int)cnt;          // particles past the group's end hold zeros
-            double t = (u[0] + u[2]) + (u[4] + u[6]);
-            for (int k = 8; k < kend; k += 8) t += (u[k] + u[k + 2]) + (u[k + 4] + u[k + 6]);
+            const double* u = v + row * DEP_CELL_LD + 2 * par;   // particles past the group's end hold zeros
+            const auto four = [&](int k) { return (u[k] + u[k + 1]) + (u[k + 4] + u[k + 5]); };
+            double t = four(0);
+            if (cnt > 8) t += four(8);
+            if (cnt > 16) t += cnt > 24 ? four(16) + four(24) : four(16);
             acc += t;
         }
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);

@@ -14,7 +14,7 @@ def test_sums_of_crowded_cells():
     nodes against extended precision.  An addition is off by 0.29 x 1.5 x 2^-53 of
     its sum (uniform in half an ulp, the ulp's mean), a chain of m that grows
     evenly by 0.58 sqrt(m) times that: 128 groups one after the other and a group's
-    five, twice (the parities, each half the sum): 2.3e-16 rms; four roundings
+    five, twice (a row's two lanes, each half the sum): 2.3e-16 rms; four roundings
     of the normalisation 1e-16.  Held to twice that (a chain of 2048 has 9e-16)."""
     cuda_or_skip()
     F = fpic()
