@@ -536,7 +536,7 @@ int fpic_fdtd_step(fpic_ctx *ctx, fpic_fields *f, const fpic_fdtd_params *prm, i
  * are skipped and counted in *n_skipped (nullable; reading it synchronises
  * the stream).  Deterministic (per-cell warp sums in particle-index order).
  * Library scratch: 28 bytes per particle, 264 per cell and records of 240 bytes
- * for up to 2^24 particles, which larger sets take in turns (fewer at a time
+ * for up to 6.7e7 particles, which larger sets take in turns (fewer at a time
  * where they do not fit).
  * Errors: FPIC_EINVAL, FPIC_ENOMEM, FPIC_ECUDA. */
 int fpic_deposit_conserving(fpic_ctx *ctx, const fpic_particles *before, const fpic_particles *after, double dt,

@@ -1993,12 +1993,13 @@ __device__ __forceinline__ double cd_phdots(const CDepK& k, uint32_t p, const do
     return ok ? x : x + (d[0] + d[1]);
 }
 
-// The records' buffer holds CDEP_CHUNK sorted entries (4 GB of 30 rows) at most:
-// more particles take it in turns, each chunk's cell sums added to the ones
-// before: 240 bytes a particle are 15 GB at 6.4e7, and sets of a few 1e8 would not
-// fit.  As many entries as leave a large run a few chunks, each of which looks at
-// every cell's range once.
-constexpr long long CDEP_CHUNK = 1LL << 24, CDEP_CHUNK_MIN = 1LL << 20;
+// The records' buffer holds CDEP_CHUNK sorted entries (16 GB of 30 rows) at most,
+// and fewer where the memory left does not hold that many: the rest take it in
+// turns, each chunk's cell sums added to the ones before.  (240 bytes a particle
+// are 72 GB at 3e8, which would not fit beside them.)  In turns a deposit is some
+// 10 % longer -- 6.4e7 particles on 1024^2 10.8 ms at once, 12.0 in four chunks:
+// the moves across boundaries, last in order, add to every cell once more.
+constexpr long long CDEP_CHUNK = 67000000, CDEP_CHUNK_MIN = 1000000;
 
 // One thread per sorted entry a0 .. a0 + m - 1: entries below off[C] are moves
 // inside their cell (CI_ROWS records), the rest up to off[2 C] the general ones
@@ -2090,8 +2091,9 @@ __global__ void __launch_bounds__(128) k_cdep_particle(const __grid_constant__ C
 // order, a group of 32 by itself (the inside moves as a tree, neighbours first, as
 // electrons and positrons alternate): as many additions as one after the other
 // in shorter chains (rho of 60 particles a cell 9e-16 -> 2.7e-16 off).  Of the entries a0 .. a0 + m - 1; LATER: a chunk
-// after the first, which adds to the cells' sums and over which the grid strides.
-constexpr int CDEP_WARPS = 8;
+// after the first, which adds to the sums of the cells it has entries of (a block
+// looks at CDEP_CELLS neighbours and leaves if they have none).
+constexpr int CDEP_WARPS = 8, CDEP_CELLS = 64;
 template <bool LATER>
 __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __restrict__ rec,
                                                                const uint32_t* __restrict__ off, uint32_t a0,
@@ -2103,8 +2105,11 @@ __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __r
     const int row = min(lane >> 1, CI_ROWS - 1), par = lane & 1;
     // entry a's place in the chunk
     const auto at = [&](uint32_t a) { return min(LATER ? (a > a0 ? a - a0 : 0u) : a, m); };
-    long long cell = blockIdx.x * (long long)CDEP_WARPS + wid;
-    if (cell >= C) return;                  // whole warps
+    const long long first = blockIdx.x * (long long)(LATER ? CDEP_CELLS : CDEP_WARPS);
+    const long long last = LATER ? min(first + CDEP_CELLS, (long long)C) : (long long)C;
+    if (LATER && at(off[first]) == at(off[last]) && at(off[(size_t)C + first]) == at(off[(size_t)C + last])) return;
+    long long cell = first + wid;
+    if (cell >= last) return;               // whole warps
     do {
         const uint32_t b0 = at(off[cell]), b1 = at(off[cell + 1]), c0 = at(off[(size_t)C + cell]),
                        c1 = at(off[(size_t)C + cell + 1]);
@@ -2155,7 +2160,7 @@ __global__ void __launch_bounds__(32 * CDEP_WARPS) k_cdep_cell(const double* __r
             const double sum = src >= 0 ? in + g : g;
             *o = LATER ? *o + sum : sum;
         }
-    } while (LATER && (cell += gridDim.x * (long long)CDEP_WARPS) < C);
+    } while (LATER && (cell += CDEP_WARPS) < last);
 }
 
 __device__ __forceinline__ double cd_dual_r(const GridDev& G, int i)
@@ -2244,12 +2249,12 @@ extern "C" int fpic_deposit_conserving(fpic_ctx* c, const fpic_particles* before
     for (long long a0 = 0; a0 < nn; a0 += chunk) {
         const long long m = nn - a0 < chunk ? nn - a0 : chunk;
         if (n > 0) k_cdep_particle<<<(unsigned)((m + 127) / 128), 128, 0, s>>>(k, w.off, w.perm2, rec, a0, m, (uint32_t)C);
-        const long long cb = (C + CDEP_WARPS - 1) / CDEP_WARPS, few = 16LL * c->sm_count;
         if (a0 == 0)
-            k_cdep_cell<false><<<(unsigned)cb, 32 * CDEP_WARPS, 0, s>>>(rec, w.off, 0, (uint32_t)m, part, (uint32_t)C);
+            k_cdep_cell<false><<<(unsigned)((C + CDEP_WARPS - 1) / CDEP_WARPS), 32 * CDEP_WARPS, 0, s>>>(
+                rec, w.off, 0, (uint32_t)m, part, (uint32_t)C);
         else
-            k_cdep_cell<true><<<(unsigned)(cb < few ? cb : few), 32 * CDEP_WARPS, 0, s>>>(rec, w.off, (uint32_t)a0,
-                                                                                        (uint32_t)m, part, (uint32_t)C);
+            k_cdep_cell<true><<<(unsigned)((C + CDEP_CELLS - 1) / CDEP_CELLS), 32 * CDEP_WARPS, 0, s>>>(
+                rec, w.off, (uint32_t)a0, (uint32_t)m, part, (uint32_t)C);
     }
     k_cdep_node<<<dim3((unsigned)((c->Nth + 1 + 255) / 256), c->Nr + 1), 256, 0, s>>>(k, tabs_of(c), part,
                                                                                      (uint32_t)C, dt, rho, jr,

@@ -86,7 +86,7 @@ for _ in range(2):
 
 @needs
 def test_conserving_deposit_scratch_is_bounded(tmp_path):
-    """3e8 particles: 28 bytes each for the sort, and records of 2^24 of them at
+    """3e8 particles: 28 bytes each for the sort, and records of 6.7e7 of them at
     a time (240 bytes), in as many turns as that takes; a quarter as many at a
     time when those do not fit."""
     out = _run(tmp_path, """
@@ -100,13 +100,13 @@ out = [at(80 + k) for k in range(4)]
 watch("k_cdep_particle")
 before = fake.fake_bytes()
 rc = L.fpic_deposit_conserving(c.handle, C.byref(p), C.byref(p), 1e-3, *out, None, None)
-print(rc, fake.fake_launches(), int(fake.fake_bytes() - before < 1.13 * (28 * n + 240 * (1 << 24)) + 5e7))
+print(rc, fake.fake_launches(), int(fake.fake_bytes() - before < 1.13 * (28 * n + 240 * 67_000_000) + 5e7))
 del c
 c, g = ctx_of(256)
-asked = size(1 << 24)
+asked = size(67_000_000)
 fake.fake_fail_alloc_of(asked + asked // 8)
 watch("k_cdep_particle")
 rc = L.fpic_deposit_conserving(c.handle, C.byref(p), C.byref(p), 1e-3, *out, None, None)
 print(rc, fake.fake_launches())
 """)
-    assert out == ["0", "18", "1", "0", "72"], out
+    assert out == ["0", "5", "1", "0", "18"], out
