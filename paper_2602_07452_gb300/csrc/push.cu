@@ -417,17 +417,16 @@ __device__ __forceinline__ void trial_store(const PushK& k, unsigned long long i
     }
 }
 
-// Bound by its issue slots (54 % used by four warps a scheduler, the rest lost
-// to fixed latencies and instruction fetches; FP64 pipe 38 % busy): some 2600
-// instructions an evaluation, two thirds of them the right-hand side on
-// integer mantissas (rhs_x).  With that in FP64, 470 FP64 instructions a
-// particle of 64 slots each were the bound, 610 before the reciprocals, the
-// sin/cos series and the gather's differences left that pipe: per 2^20
-// charged particles 1.164 -> 0.951 -> 0.70 ms, RK4 push of 6.4e7 sorted ones on
-// 1024 x 1024 76 -> 61 -> 35 ms.  One copy of the evaluation serves all stages
-// (five would be 200 KB of code); z^n and the slopes' sum wait in shared memory
-// meanwhile.  3, 4 or 5 resident blocks, 256 threads, or warps held together by
-// barriers: within 3 %.
+// Bound by latencies between its issue slots (45 % used by four warps a scheduler)
+// and the FP64 pipe (48 % busy): some 2350 instructions an evaluation, two thirds
+// of them the right-hand side on integer mantissas (rhs_x).  With that in FP64,
+// 470 FP64 instructions a particle of 64 slots each were the bound, 610 before the
+// reciprocals and the sin/cos series left that pipe: per 2^20 charged particles
+// 1.164 -> 0.951 -> 0.67 ms, RK4 push of 6.4e7 sorted ones on 1024 x 1024 76 -> 61 ->
+// 35 ms.  The field gather is FP64 (in pairs of floats 0.68 ms and less exact).
+// One copy of the evaluation serves all stages (five would be 200 KB of code);
+// z^n and the slopes' sum wait in shared memory meanwhile.  3, 4 or 5 resident
+// blocks, 256 threads, or warps held together by barriers: within 3 %.
 // MODE 0: RK4 only.  MODE 1: hybrid (RK4 trial + test + enqueue).  MODE 2:
 // hybrid that also parks the RK4 slopes of each rejected particle
 // (corrector form of the learned guess); k1, k2, k4 wait in shared memory
@@ -1509,9 +1508,9 @@ namespace fpic {
 // Per-cell bilinear coefficients of the six field components (see gather_c),
 // one thread per (node row, column) of grid blockIdx.z; cells past a sub-grid's
 // last node pair are never read (the cell search clamps to the last cell).
-// A batch of runs builds its grids' coefficients in one launch (HBM-bound:
-// 240 bytes a node) instead of one of 7 to 18 us each: 12 grids of 128^2 to
-// 512^2, 115 of the 1181 us of a batched push, now 1102.
+// A batch of runs builds its grids' coefficients in one launch (240 bytes a node,
+// 24 FP64 subtractions) instead of one of 7 to 18 us each: 12 grids of 128^2 to
+// 512^2 115 -> 64 us of a batched push.
 struct CoefJob {
     int Nr, Nth, ld, full;
     const double* f[6];
