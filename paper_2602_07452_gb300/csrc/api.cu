@@ -44,10 +44,11 @@ void retire(fpic_ctx* c, void** p, bool host)
 int ensure_scratch(fpic_ctx* c, size_t bytes)
 {
     if (bytes <= c->scratch_bytes) return 0;
+    const size_t b = bytes + bytes / 8;
+    void* q = nullptr;
+    FPIC_CUDA(cudaMalloc(&q, b));        // one that fails leaves the buffer there was
     retire(c, &c->d_scratch);
-    c->scratch_bytes = 0;
-    size_t b = bytes + bytes / 8;
-    FPIC_CUDA(cudaMalloc(&c->d_scratch, b));
+    c->d_scratch = q;
     c->scratch_bytes = b;
     return 0;
 }
@@ -55,10 +56,11 @@ int ensure_scratch(fpic_ctx* c, size_t bytes)
 int ensure_scratch2(fpic_ctx* c, size_t bytes)
 {
     if (bytes <= c->scratch2_bytes) return 0;
+    const size_t b = bytes + bytes / 8;
+    void* q = nullptr;
+    FPIC_CUDA(cudaMalloc(&q, b));        // one that fails leaves the buffer there was
     retire(c, &c->d_scratch2);
-    c->scratch2_bytes = 0;
-    size_t b = bytes + bytes / 8;
-    FPIC_CUDA(cudaMalloc(&c->d_scratch2, b));
+    c->d_scratch2 = q;
     c->scratch2_bytes = b;
     return 0;
 }

@@ -31,6 +31,7 @@ struct fpic_ctx {
     void* d_poly = nullptr;
     unsigned long long poly_grid = ~0ull;
     int poly_deg = 0;                // 0: none
+    long long cdep_chunk = 0;        // entries at a time of the conserving deposit, once fewer had to do (0: not yet)
     // metric tables at the Yee points (library-owned), see pic.cu
     double* d_metric = nullptr;
     size_t metric_stride = 0;        // elements per table

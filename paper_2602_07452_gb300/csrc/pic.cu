@@ -2226,11 +2226,12 @@ extern "C" int fpic_deposit_conserving(fpic_ctx* c, const fpic_particles* before
     void* part_v = nullptr;     // per-cell window partials (CD_SLOTS x C), a chunk's records (CD_SLOTS x chunk)
     const long long nn = n > 0 ? n : 1;
     // entries at a time; fewer where the records do not fit the memory left
-    long long chunk = nn < CDEP_CHUNK ? nn : CDEP_CHUNK;
+    const long long most = c->cdep_chunk ? c->cdep_chunk : CDEP_CHUNK;
+    long long chunk = nn < most ? nn : most;
     int rc;
     while ((rc = work_layout(c, nn, false, w, (size_t)CD_SLOTS * (C + chunk) * sizeof(double), &part_v, 2)) == FPIC_ENOMEM &&
            chunk > CDEP_CHUNK_MIN)
-        chunk = chunk / 4 > CDEP_CHUNK_MIN ? chunk / 4 : CDEP_CHUNK_MIN;
+        c->cdep_chunk = chunk = chunk / 4 > CDEP_CHUNK_MIN ? chunk / 4 : CDEP_CHUNK_MIN;
     if (rc) return rc;
     double* part = (double*)part_v;
     double* rec = part + (size_t)CD_SLOTS * C;

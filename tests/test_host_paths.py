@@ -88,7 +88,7 @@ for _ in range(2):
 def test_conserving_deposit_scratch_is_bounded(tmp_path):
     """3e8 particles: 28 bytes each for the sort, and records of 6.7e7 of them at
     a time (240 bytes), in as many turns as that takes; a quarter as many at a
-    time when those do not fit."""
+    time when those do not fit, also for the next call, which allocates nothing."""
     out = _run(tmp_path, """
 n = 300_000_000
 size = lambda chunk: sum((b + 255) & ~255 for b in (4*n, 4*n, 4*n, 4*(2*C_+2), 4*(2*C_+2), 4*(2*C_+2), 4*(n//4096 + 2), 4*n,
@@ -108,5 +108,8 @@ fake.fake_fail_alloc_of(asked + asked // 8)
 watch("k_cdep_particle")
 rc = L.fpic_deposit_conserving(c.handle, C.byref(p), C.byref(p), 1e-3, *out, None, None)
 print(rc, fake.fake_launches())
+before = fake.fake_bytes()
+rc = L.fpic_deposit_conserving(c.handle, C.byref(p), C.byref(p), 1e-3, *out, None, None)
+print(rc, fake.fake_launches(), fake.fake_bytes() - before)
 """)
-    assert out == ["0", "5", "1", "0", "18"], out
+    assert out == ["0", "5", "1", "0", "18", "0", "36", "0"], out
